@@ -84,12 +84,11 @@ struct pp_plan_s {
   float *d_mtab_f = nullptr, *d_invd_f = nullptr, *d_zc_f = nullptr;
   int* d_low = nullptr;
   TriF32 tri32{};
-  bool use_tri32 = false;
-  // PP_MIXED_Z64: tables of the FP64-recurrence z solve (TriZ64)
-  double *d_z64m = nullptr, *d_z64e = nullptr;
-  float* d_z64d = nullptr;
-  TriZ64 z64{};
-  bool use_z64 = false;
+  // FP64 and PP_MIXED_Z64: tables of the FP64-recurrence z solve (TriZ)
+  double *d_zm = nullptr, *d_ze = nullptr;
+  void* d_zd = nullptr;  // 1 / d_k in the spectrum's precision
+  int z_nyt = 0, z_ysym = 0;
+  bool use_z = false;
   double* d_rho_tilde = nullptr;
   double* d_delta64 = nullptr;
   double* d_thermo = nullptr;  // [4] sums and rate of Eq. 30
@@ -277,8 +276,6 @@ pp_status solve_pass(pp_plan_s* P, double* p, int p_zero, T* delta = nullptr, fl
   // place, so the z solve works on the second spectrum buffer
   const bool ytc = P->ystretch && std::is_same<T, float>::value;
   C2<T>* zs = ytc ? (C2<T>*)P->d_spec2 : spec;
-  // the split solve (mtab present) keeps its intermediate in the spectrum
-  double2* ybuf = (double2*)zs;
   // the dense y step of a stretched y is W-orthonormal: no 1/ny on the way back
   const double scale = 1.0 / ((double)P->nx * (P->ystretch ? 1.0 : (double)P->ny));
   const C2<T>* dct = (const C2<T>*)P->d_dcty;  // null: periodic y
@@ -335,11 +332,11 @@ pp_status solve_pass(pp_plan_s* P, double* p, int p_zero, T* delta = nullptr, fl
     } else {
       return PP_ERR_UNSUPPORTED;
     }
-  } else if (std::is_same<T, float>::value && P->use_z64) {
-    PP_K(P, K_TRI, launch_tridiag_z64(g, P->z64, reinterpret_cast<float2*>(zs), P->d_st, P->stream));
+  } else if (P->use_z) {
+    const TriZ<T> tz{P->d_zm, P->d_ze, (const T*)P->d_zd, P->z_nyt, P->z_ysym};
+    PP_K(P, K_TRI, launch_zsolve<T>(g, tz, zs, P->d_st, P->stream));
   } else {
-    PP_K(P, K_TRI, launch_tridiag<T>(g, P->d_invd, zs, ybuf, P->d_st, P->stream, P->d_mtab,
-                                     P->use_tri32 ? &P->tri32 : nullptr));
+    PP_K(P, K_TRI, launch_tridiag<T>(g, P->d_invd, zs, nullptr, P->d_st, P->stream, P->d_mtab, &P->tri32));
   }
   if (ytc) PP_K(P, K_FFTY_I, launch_dense_tc(ytc_args(zs, spec, P->d_ytc_i), P->d_st, P->stream));
   else if (P->ystretch) {
@@ -449,9 +446,10 @@ void free_plan(pp_plan_s* P) {
   if (P->faces.rhof) cudaFree(P->faces.rhof);
   if (P->d_low) cudaFree(P->d_low);
   float* fptrs[] = {P->faces.diagf, P->d_delta, P->d_sdelta, P->d_mtab_f, P->d_invd_f, P->d_zc_f,
-                    P->d_z64d, P->d_cw_f};
-  if (P->d_z64m) cudaFree(P->d_z64m);
-  if (P->d_z64e) cudaFree(P->d_z64e);
+                    P->d_cw_f};
+  if (P->d_zm) cudaFree(P->d_zm);
+  if (P->d_ze) cudaFree(P->d_ze);
+  if (P->d_zd) cudaFree(P->d_zd);
   for (float* f : fptrs) if (f) cudaFree(f);
   if (P->d_E) cudaFree(P->d_E);
   if (P->d_mu) cudaFree(P->d_mu);
@@ -690,8 +688,9 @@ pp_status pressure_plan_create(const pp_grid* grid, pp_precision prec, void* str
   const size_t rpb_min = 2;
   P->red_len = std::max((size_t)2 * ((size_t)G.ny * nz + rpb_min - 1) / rpb_min + 2,
                         (size_t)reduce_blocks());
-  if ((st = dalloc(&P->d_invd, nsp * sizeof(double))) != PP_OK ||
-      (st = dalloc(&P->d_mtab, nsp * sizeof(double))) != PP_OK ||
+  const bool hybrid = prec == PP_MIXED_FP32;
+  if ((hybrid && (st = dalloc(&P->d_invd, nsp * sizeof(double))) != PP_OK) ||
+      (hybrid && (st = dalloc(&P->d_mtab, nsp * sizeof(double))) != PP_OK) ||
       (st = dalloc(&P->d_spec, nsp * csz)) != PP_OK ||
       (prec != PP_FP64 && (st = dalloc(&P->d_E, nc * sizeof(float))) != PP_OK) ||
       (prec != PP_FP64 && (st = dalloc(&P->d_delta, nc * sizeof(float))) != PP_OK) ||
@@ -768,7 +767,8 @@ pp_status pressure_plan_create(const pp_grid* grid, pp_precision prec, void* str
     P->ze.a1 = P->d_za1;
     P->ze.a2 = P->d_za2;
   }
-  if (launch_setup_pivots(g, P->d_lamx, P->d_lamy, P->d_invd, P->stream, P->d_mtab) != cudaSuccess ||
+  if ((hybrid &&
+       launch_setup_pivots(g, P->d_lamx, P->d_lamy, P->d_invd, P->stream, P->d_mtab) != cudaSuccess) ||
       launch_init_status(P->d_st, P->stream) != cudaSuccess ||
       cudaStreamSynchronize(P->stream) != cudaSuccess) {
     free_plan(P);
@@ -801,28 +801,25 @@ pp_status pressure_plan_create(const pp_grid* grid, pp_precision prec, void* str
     P->tri32.thr = thr;
     P->tri32.low = P->d_low;
     P->tri32.nlow = (int)low.size();
-    P->use_tri32 = true;
   }
-  if (prec == PP_MIXED_Z64) {
+  if (prec == PP_MIXED_Z64 || prec == PP_FP64) {
     // periodic y: lambda_y(ky) = lambda_y(ny - ky), one table column for both
-    const int ysym = ywall ? 0 : 1;
-    const int nyt = ysym ? G.ny / 2 + 1 : G.ny;
-    const size_t ntab = (size_t)nz * nyt * P->nxh;
-    if ((st = dalloc(&P->d_z64m, ntab * sizeof(double))) != PP_OK ||
-        (st = dalloc(&P->d_z64e, ntab * sizeof(double))) != PP_OK ||
-        (st = dalloc(&P->d_z64d, ntab * sizeof(float))) != PP_OK ||
-        launch_setup_z64(g, P->d_lamx, P->d_lamy, nyt, ysym, P->d_z64m, P->d_z64e, P->d_z64d, P->stream) !=
-            cudaSuccess ||
+    P->z_ysym = ywall ? 0 : 1;
+    P->z_nyt = ywall ? G.ny : G.ny / 2 + 1;
+    const size_t ntab = (size_t)nz * P->z_nyt * P->nxh;
+    const size_t tsz = (prec == PP_FP64) ? sizeof(double) : sizeof(float);
+    if ((st = dalloc(&P->d_zm, ntab * sizeof(double))) != PP_OK ||
+        (st = dalloc(&P->d_ze, ntab * sizeof(double))) != PP_OK ||
+        (st = dalloc((unsigned char**)&P->d_zd, ntab * tsz)) != PP_OK ||
+        (prec == PP_FP64 ? launch_setup_z<double>(g, P->d_lamx, P->d_lamy, P->z_nyt, P->d_zm, P->d_ze,
+                                                  (double*)P->d_zd, P->stream)
+                         : launch_setup_z<float>(g, P->d_lamx, P->d_lamy, P->z_nyt, P->d_zm, P->d_ze,
+                                                 (float*)P->d_zd, P->stream)) != cudaSuccess ||
         cudaStreamSynchronize(P->stream) != cudaSuccess) {
       free_plan(P);
       return st != PP_OK ? st : PP_ERR_CUDA;
     }
-    P->z64.m = P->d_z64m;
-    P->z64.e = P->d_z64e;
-    P->z64.d = P->d_z64d;
-    P->z64.nyt = nyt;
-    P->z64.ysym = ysym;
-    P->use_z64 = true;
+    P->use_z = true;
   }
   *out = P;
   return PP_OK;

@@ -20,7 +20,6 @@ using namespace pp;
 namespace {
 
 constexpr int kChunk = 2048;  // cells per block of the elementwise grouped kernels
-constexpr int kTriThreads = 128;
 constexpr int kExactEveryBatch = 40;
 
 struct GridDev {
@@ -173,11 +172,12 @@ __global__ void __launch_bounds__(256) kb_ffty(GridDev* G, const int2* __restric
   else stage_ffty<float, DIR>(d.g, d.fy, d.twy, d.spec, d.tx, bx, bz, smem_raw);
 }
 
-__global__ void __launch_bounds__(kTriThreads, 8) kb_tridiag(GridDev* G, const int2* __restrict__ work) {
+__global__ void __launch_bounds__(kZThreads, 8) kb_tridiag(GridDev* G, const int2* __restrict__ work) {
   const int2 w = work[blockIdx.x];
   const GridDev& d = G[w.x];
   if (d.st->done) return;
-  stage_tridiag_mixed(d.g, d.mtab, d.invd, d.tri, d.spec, w.y);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  stage_tridiag_mixed(d.g, d.mtab, d.invd, d.tri, d.spec, w.y, smem_raw);
 }
 
 __global__ void __launch_bounds__(256) kb_fftx_inv(GridDev* G, const int2* __restrict__ work) {
@@ -330,7 +330,7 @@ cudaError_t launch_pass(pp_batch_s* B, cudaStream_t s) {
   kb_resid<<<B->n_x, kThreads, B->smem_x, s>>>(B->d_dev, B->w_x);
   kb_check<<<B->n, 1024, 0, s>>>(B->d_dev, B->d_ctl, kExactEveryBatch);
   kb_ffty<-1><<<B->n_y, kThreads, B->smem_y, s>>>(B->d_dev, B->w_y);
-  kb_tridiag<<<B->n_z, kTriThreads, 0, s>>>(B->d_dev, B->w_z);
+  kb_tridiag<<<B->n_z, kZThreads, zsweep_smem<ZForm32, 1>(), s>>>(B->d_dev, B->w_z);
   kb_ffty<1><<<B->n_y, kThreads, B->smem_y, s>>>(B->d_dev, B->w_y);
   kb_fftx_inv<<<B->n_x, kThreads, B->smem_x, s>>>(B->d_dev, B->w_x);
   return cudaGetLastError();

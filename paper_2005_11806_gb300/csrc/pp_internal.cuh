@@ -96,14 +96,11 @@ struct Faces {
 // part is the scarce resource).  Subnormal inputs become signed zeros.
 __device__ __forceinline__ double widen_f32(float f) {
   const unsigned b = __float_as_uint(f);
-  const unsigned sign = b & 0x80000000u;
-  const unsigned e = (b >> 23) & 0xFFu;
-  const unsigned m = b & 0x7FFFFFu;
-  unsigned hi = sign | ((e + 896u) << 20) | (m >> 3);
-  unsigned lo = m << 29;
-  if (e == 0u) { hi = sign; lo = 0u; }
-  if (e == 0xFFu) hi = sign | 0x7FF00000u | (m >> 3);
-  return __hiloint2double((int)hi, (int)lo);
+  const unsigned t = b & 0x7FFFFFFFu;
+  unsigned hi = (t >> 3) + 0x38000000u, lo = b << 29;
+  if (t >= 0x7F800000u) hi += 0x38000000u;  // Inf, NaN
+  if (t < 0x00800000u) hi = lo = 0u;
+  return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)lo);
 }
 
 // 1 / rho_f of a face from its two cells' FP32 densities (arithmetic face
@@ -136,12 +133,12 @@ inline std::vector<float> layer_factors_f32(int nz, const std::vector<double>& d
 // the first dropped bit; underflow flushes to zero, overflow/NaN give Inf.
 __device__ __forceinline__ float narrow_f64(double d) {
   const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
-  const unsigned sign = hi & 0x80000000u;
-  const int e = (int)((hi >> 20) & 0x7FFu) - 896;
-  unsigned bits = ((unsigned)e << 23) + (((hi & 0xFFFFFu) << 3) | (lo >> 29)) + ((lo >> 28) & 1u);
-  if (e <= 0) bits = 0u;
-  if (e >= 255) bits = 0x7F800000u;
-  return __uint_as_float(sign | bits);
+  const unsigned t = hi & 0x7FFFFFFFu;
+  const unsigned long long r = (((unsigned long long)(t - 0x38000000u) << 32) | lo) + 0x10000000ull;
+  unsigned bits = (unsigned)(r >> 29);
+  if (t < 0x38100000u) bits = 0u;
+  if (t >= 0x47F00000u) bits = 0x7F800000u;
+  return __uint_as_float(bits | (hi & 0x80000000u));
 }
 
 // ---- launchers (pp_kernels_*.cu) -------------------------------------
@@ -200,38 +197,44 @@ struct TriF32 {
 // Columns (index ky * nxh + kx) that keep FP64: |lambda| < thr, and column 0.
 std::vector<int> tri_low_columns(const std::vector<double>& lamx, const std::vector<double>& lamy,
                                  double thr);
-// Blocks of 128 threads of the mixed z solve.
-inline int tri_mixed_blocks(size_t ncol, int nlow) { return (nlow + 3) / 4 + (int)((ncol + 127) / 128); }
+// Blocks of the mixed z solve (kZThreads threads: a warp per ill-conditioned
+// column, then a thread per column).
+int tri_mixed_blocks(size_t ncol, int nlow);
 
-// With mtab (multipliers m_k = a_k / d_{k-1}) the real and imaginary parts
-// run in separate threads; without it one thread solves a whole column.
-// With f32 (mixed plans) the well-conditioned columns run in FP32.
+// With f32 (PP_MIXED_FP32 plans) the well-conditioned columns run in FP32 and
+// the others in FP64 with the multipliers mtab; without it one thread solves
+// a whole column in FP64 from the inverse pivots alone (ybuf: its forward
+// values; may alias spec).
 template <typename T>
 cudaError_t launch_tridiag(const Geo& g, const double* invd, C2<T>* spec, double2* ybuf,
                            const DevStatus* st, cudaStream_t s, const double* mtab = nullptr,
                            const TriF32* f32 = nullptr);
-// FP64 z solve of PP_MIXED_Z64 plans: FP64 recurrences in every (kx, ky)
-// column, values stored in FP32.  Thomas elimination in the form
+// z solve of FP64 and PP_MIXED_Z64 plans: FP64 recurrences in every (kx, ky)
+// column, values stored in the spectrum's precision T.  Thomas elimination
+// in the form
 //   forward   y_k = f_k - m_k y_{k-1},            m_k = a_k / d_{k-1}
-//             s_k = (1/d_k) y_k                   (stored, FP32)
+//             s_k = (1/d_k) y_k                   (stored)
 //   backward  x_k = s_k - e_k x_{k+1},            e_k = c_k / d_k,
-// so each sweep costs one FP64 FMA per scalar.  The tables depend on the
-// column only through lambda = lambda_x(kx) + lambda_y(ky); with periodic y
+// so each sweep's recurrence is one FP64 FMA per scalar (on FP32 storage the
+// scaling by 1/d_k is an FP32 multiply: the same 2^-24 relative perturbation
+// per value as storing y_k itself).  The tables depend on the column only
+// through lambda = lambda_x(kx) + lambda_y(ky); with periodic y
 // lambda_y(ky) = lambda_y(ny - ky), so ky and ny - ky share one table column
 // (ysym: nyt = ny/2 + 1 table rows of nxh columns per layer, ky' = min(ky,
 // ny - ky)); with walls in y nyt = ny.  Table column 0 is the singular
 // (0, 0) system: its last inverse pivot is 0 (pinned unknown).
-struct TriZ64 {
+template <typename T> struct TriZ {
   const double* m;  // [nz][nyt][nxh]
   const double* e;  // [nz][nyt][nxh]
-  const float* d;   // [nz][nyt][nxh] 1 / d_k
+  const T* d;       // [nz][nyt][nxh] 1 / d_k
   int nyt;
   int ysym;
 };
-cudaError_t launch_setup_z64(const Geo& g, const double* lamx, const double* lamy, int nyt, int ysym,
-                             double* m, double* e, float* d, cudaStream_t s);
-cudaError_t launch_tridiag_z64(const Geo& g, const TriZ64& t, float2* spec, const DevStatus* st,
-                               cudaStream_t s);
+template <typename T>
+cudaError_t launch_setup_z(const Geo& g, const double* lamx, const double* lamy, int nyt, double* m, double* e,
+                           T* d, cudaStream_t s);
+template <typename T>
+cudaError_t launch_zsolve(const Geo& g, const TriZ<T>& t, C2<T>* spec, const DevStatus* st, cudaStream_t s);
 // dst[i] = (float) src[i], i < n.
 cudaError_t launch_narrow(const double* src, float* dst, size_t n, cudaStream_t s);
 // Inverse x-transform; p = scale * z (p_zero) or p += scale * z; when delta

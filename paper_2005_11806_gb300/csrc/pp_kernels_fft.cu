@@ -62,59 +62,52 @@ __global__ void __launch_bounds__(128) k_tridiag(Geo g, const double* __restrict
   else thomas_column<T, false>(g, invd, spec, ybuf, col, ncol);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(128, 16) k_tridiag_split(Geo g, const double* __restrict__ mtab,
-                                                           const double* __restrict__ invd, T* spec,
-                                                           const DevStatus* __restrict__ st) {
+// z solve of FP64 and PP_MIXED_Z64 plans: one thread per column of `spec`
+// (ZForm64: complex entries; ZFormD: scalars, the components apart, which
+// gives small grids twice the chains).  P = 2 (periodic y): a thread takes
+// the columns ky and ny - ky, which share their table column; the columns
+// that are their own mirror are done twice by the same thread.  The warp that
+// holds column 0 first takes its dzf-weighted mean and subtracts it on the
+// way (all its lanes run the ZERO variant, the others with mean 0), so no
+// warp runs two variants.
+template <class F, int P>
+__global__ void __launch_bounds__(kZThreads) k_zsolve(Geo g, F tab, int nyt, int ysym, typename F::Val* spec,
+                                                      const DevStatus* __restrict__ st) {
   if (stopped(st)) return;
-  __shared__ double shm[34];
-  double m0 = 0.0;
-  if (blockIdx.x == 0) {  // holds column 0 (scalars 0 and 1)
-    zero_column_means<T>(g, spec, 2 * (size_t)g.ny * g.nxh, shm);
-    if (threadIdx.x < 2) m0 = shm[32 + threadIdx.x];
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int C = std::is_same<F, ZFormD>::value ? 2 : 1;  // entries per complex column
+  const unsigned n = (unsigned)C * (unsigned)g.ny * (unsigned)g.nxh;  // entries of a row
+  const unsigned work = P == 2 ? (unsigned)C * (unsigned)nyt * (unsigned)g.nxh : n;
+  const unsigned id = blockIdx.x * kZThreads + threadIdx.x;
+  const unsigned col = id / C;
+  const bool first = id < 32u;  // warp-uniform
+  double mx = 0.0, my = 0.0;
+  if (first) {
+    zero_column_mean(g, spec, n, mx, my);
+    if (C == 2 && id == 1u) mx = my;  // the scalars' second entry is the imaginary part
+    if (col != 0u) mx = my = 0.0;
   }
-  stage_tridiag_split<T>(g, mtab, invd, spec, (size_t)blockIdx.x * blockDim.x + threadIdx.x, m0);
+  if (id >= work) return;
+  const unsigned ny = (unsigned)g.ny, nxh = (unsigned)g.nxh;
+  const unsigned ky = col / nxh, kx = col - ky * nxh;
+  const unsigned kyt = (ysym && 2u * ky > ny) ? ny - ky : ky;
+  const size_t t = (size_t)kyt * nxh + kx, tstride = (size_t)nyt * nxh;
+  typename F::Val* vals[P];
+  vals[0] = spec + id;
+  if constexpr (P == 2) {
+    const unsigned ky2 = (ky == 0u || 2u * ky == ny) ? ky : ny - ky;
+    vals[1] = spec + (size_t)(ky2 * nxh + kx) * C + (id - col * C);
+  }
+  if (first) zsweep<F, P, true>(tab, vals, n, t, tstride, g.nz, nullptr, smem_raw, mx, my);
+  else zsweep<F, P, false>(tab, vals, n, t, tstride, g.nz, nullptr, smem_raw, 0.0, 0.0);
 }
 
-// PP_MIXED_Z64 z solve: one thread per (kx, ky) column, all FP64
-// recurrences (stage_tridiag_z64).  The grid is persistent-sized (every
-// block resident at once) and the columns are dealt out a warp at a time,
-// round robin over the blocks (work warp = warp-in-block x gridDim +
-// block), so every SM gets the same number of FP64 chains whatever the
-// block scheduler's placement; a warp still takes 32 consecutive columns.
-// Work warp 0 (warp 0 of block 0) holds the singular column 0 alone, so no
-// warp runs both variants of the sweep one after the other; work warp w > 0
-// holds columns 1 + 32 (w - 1) + lane.  Block 0 first reduces column 0's
-// dzf-weighted z means.
-__global__ void __launch_bounds__(128, 8) k_tridiag_z64(Geo g, TriZ64 t, float2* spec,
-                                                        const DevStatus* __restrict__ st) {
-  if (stopped(st)) return;
-  __shared__ double shm[34];
-  const unsigned ncol = (unsigned)g.ny * g.nxh;
-  const unsigned ntc = (unsigned)t.nyt * g.nxh;
-  if (blockIdx.x == 0) zero_column_means<float>(g, reinterpret_cast<const float*>(spec), 2 * (size_t)ncol, shm);
-  const unsigned wstride = (blockDim.x >> 5) * gridDim.x;
-  const unsigned lane = threadIdx.x & 31u;
-  for (unsigned wq = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; wq == 0 || (wq - 1) * 32u + 1u < ncol;
-       wq += wstride) {
-    if (wq == 0) {  // warp 0 of block 0: column 0 on lane 0
-      if (lane == 0) stage_tridiag_z64<true>(g, t, spec, 0, ncol, 0, ntc, shm[32], shm[33]);
-      continue;
-    }
-    const unsigned col = 1u + (wq - 1) * 32u + lane;
-    if (col >= ncol) continue;
-    const int ky = (int)(col / (unsigned)g.nxh);
-    const int kx = (int)(col - (unsigned)ky * g.nxh);
-    const int kyt = (t.ysym && 2 * ky > g.ny) ? g.ny - ky : ky;
-    stage_tridiag_z64<false>(g, t, spec, col, ncol, (unsigned)kyt * g.nxh + kx, ntc, 0.0, 0.0);
-  }
-}
-
-__global__ void __launch_bounds__(128, 8) k_tridiag_mixed(Geo g, const double* __restrict__ mtab,
+__global__ void __launch_bounds__(kZThreads, 8) k_tridiag_mixed(Geo g, const double* __restrict__ mtab,
                                                          const double* __restrict__ invd, TriF32 f,
                                                          float2* spec, const DevStatus* __restrict__ st) {
   if (stopped(st)) return;
-  stage_tridiag_mixed(g, mtab, invd, f, spec, blockIdx.x);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  stage_tridiag_mixed(g, mtab, invd, f, spec, blockIdx.x, smem_raw);
 }
 
 // p += sdelta when the last residual of the loop was an updated one (the
@@ -227,16 +220,18 @@ cudaError_t launch_zdct(const Geo& g, const FftDesc& fz, const C2<T>* twz, C2<T>
 template cudaError_t launch_zdct<double>(const Geo&, const FftDesc&, const double2*, double2*, int,
                                          const DevStatus*, cudaStream_t, const double2*, const ZDivide&);
 
+int tri_mixed_blocks(size_t ncol, int nlow) {
+  constexpr int kWarps = kZThreads / 32;
+  return (nlow + kWarps - 1) / kWarps + (int)((ncol + kZThreads - 1) / kZThreads);
+}
+
 template <typename T>
 cudaError_t launch_tridiag(const Geo& g, const double* invd, C2<T>* spec, double2* ybuf,
                            const DevStatus* st, cudaStream_t s, const double* mtab, const TriF32* f32) {
   const size_t ncol = (size_t)g.ny * g.nxh;
-  if (mtab != nullptr && f32 != nullptr && sizeof(T) == sizeof(float)) {
-    k_tridiag_mixed<<<tri_mixed_blocks(ncol, f32->nlow), 128, 0, s>>>(g, mtab, invd, *f32,
-                                                                     reinterpret_cast<float2*>(spec), st);
-  } else if (mtab != nullptr) {
-    const int nblk = (int)((2 * ncol + 127) / 128);
-    k_tridiag_split<T><<<nblk, 128, 0, s>>>(g, mtab, invd, reinterpret_cast<T*>(spec), st);
+  if (f32 != nullptr && sizeof(T) == sizeof(float)) {
+    k_tridiag_mixed<<<tri_mixed_blocks(ncol, f32->nlow), kZThreads, zsweep_smem<ZForm32, 1>(), s>>>(
+        g, mtab, invd, *f32, reinterpret_cast<float2*>(spec), st);
   } else {
     const int nblk = (int)((ncol + 127) / 128);
     k_tridiag<T><<<nblk, 128, 0, s>>>(g, invd, spec, ybuf, st);
@@ -244,24 +239,35 @@ cudaError_t launch_tridiag(const Geo& g, const double* invd, C2<T>* spec, double
   return cudaGetLastError();
 }
 
-cudaError_t launch_tridiag_z64(const Geo& g, const TriZ64& t, float2* spec, const DevStatus* st,
-                               cudaStream_t s) {
-  const size_t ncol = (size_t)g.ny * g.nxh;
-  const long long nwarps = 1 + (long long)((ncol - 1 + 31) / 32);  // column 0 alone, then 32 per warp
-  int per_sm = 0, dev = 0, nsm = 0;
-  cudaError_t e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tridiag_z64, 128, 0)) != cudaSuccess) return e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if (per_sm < 1) per_sm = 1;
-  // all blocks resident at once; no more blocks than warps of work (each
-  // block then still holds at least one column in its first warp)
-  long long nblk = (long long)nsm * per_sm;
-  if (nblk > nwarps) nblk = nwarps;
-  if (nblk < 1) nblk = 1;
-  k_tridiag_z64<<<(int)nblk, 128, 0, s>>>(g, t, spec, st);
+template <class F, int P>
+static cudaError_t launch_zsolve_p(const Geo& g, const F& form, int nyt, int ysym, size_t work, typename F::Val* spec,
+                                   const DevStatus* st, cudaStream_t s) {
+  static_assert(zsweep_smem<F, P>() <= 48 * 1024, "fits without the opt-in attribute");
+  k_zsolve<F, P><<<(unsigned)((work + kZThreads - 1) / kZThreads), kZThreads, zsweep_smem<F, P>(), s>>>(
+      g, form, nyt, ysym, spec, st);
   return cudaGetLastError();
 }
+
+// Two columns a thread halve the table traffic and leave half the warps: it
+// pays from about 1.5 such warps an SM partition (measured, one column / two:
+// 512^3, 3.4 warps, 0.533 / 0.512 ms; 384^3, 1.9 warps, 0.235 / 0.214 ms;
+// 256^3, 0.85 warps, 0.088 / 0.115 ms).
+template <typename T>
+cudaError_t launch_zsolve(const Geo& g, const TriZ<T>& t, C2<T>* spec, const DevStatus* st, cudaStream_t s) {
+  const size_t ncol = (size_t)g.ny * g.nxh;
+  if constexpr (std::is_same<T, float>::value) {
+    const ZForm64 form{t.m, t.d, t.e};
+    const size_t pairs = (size_t)t.nyt * g.nxh;
+    if (t.ysym && pairs >= (size_t)152 * 4 * 32 * 3 / 2)
+      return launch_zsolve_p<ZForm64, 2>(g, form, t.nyt, t.ysym, pairs, spec, st, s);
+    return launch_zsolve_p<ZForm64, 1>(g, form, t.nyt, t.ysym, ncol, spec, st, s);
+  } else {
+    const ZFormD form{t.m, t.d, t.e};
+    return launch_zsolve_p<ZFormD, 1>(g, form, t.nyt, t.ysym, 2 * ncol, reinterpret_cast<double*>(spec), st, s);
+  }
+}
+template cudaError_t launch_zsolve<float>(const Geo&, const TriZ<float>&, float2*, const DevStatus*, cudaStream_t);
+template cudaError_t launch_zsolve<double>(const Geo&, const TriZ<double>&, double2*, const DevStatus*, cudaStream_t);
 
 std::vector<int> tri_low_columns(const std::vector<double>& lamx, const std::vector<double>& lamy,
                                  double thr) {

@@ -138,13 +138,14 @@ __global__ void k_setup_pivots(Geo g, const double* __restrict__ lamx, const dou
   }
 }
 
-// Tables of the PP_MIXED_Z64 z solve (TriZ64), one thread per table column
+// Tables of the FP64-recurrence z solve (TriZ), one thread per table column
 // tc = ky' nxh + kx with lambda = lambda_x(kx) + lambda_y(ky'): the same
 // pivot recurrence as k_setup_pivots, stored as m_k = a_k / d_{k-1},
-// e_k = c_k / d_k (FP64) and 1 / d_k (FP32).  Column 0 is the singular
-// (0, 0) system: its last inverse pivot is 0.
-__global__ void k_setup_z64(Geo g, const double* __restrict__ lamx, const double* __restrict__ lamy, int nyt,
-                            double* __restrict__ m, double* __restrict__ e, float* __restrict__ dinv) {
+// e_k = c_k / d_k (FP64) and 1 / d_k (the spectrum's precision).  Column 0 is
+// the singular (0, 0) system: its last inverse pivot is 0.
+template <typename T>
+__global__ void k_setup_z(Geo g, const double* __restrict__ lamx, const double* __restrict__ lamy, int nyt,
+                            double* __restrict__ m, double* __restrict__ e, T* __restrict__ dinv) {
   const size_t ntc = (size_t)nyt * g.nxh;
   const size_t tc = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (tc >= ntc) return;
@@ -159,7 +160,7 @@ __global__ void k_setup_z64(Geo g, const double* __restrict__ lamx, const double
     const size_t o = (size_t)k * ntc + tc;
     m[o] = (k == 0) ? 0.0 : g.za[k] * inv_prev;
     e[o] = (k + 1 < g.nz) ? g.zc[k] * inv : 0.0;
-    dinv[o] = (float)inv;
+    dinv[o] = (T)inv;
     inv_prev = inv;
   }
 }
@@ -669,13 +670,17 @@ cudaError_t launch_setup_pivots(const Geo& g, const double* lamx, const double* 
   return cudaGetLastError();
 }
 
-cudaError_t launch_setup_z64(const Geo& g, const double* lamx, const double* lamy, int nyt, int ysym,
-                             double* m, double* e, float* d, cudaStream_t s) {
-  (void)ysym;  // the table rows are ky' = 0 .. nyt - 1 either way
+template <typename T>
+cudaError_t launch_setup_z(const Geo& g, const double* lamx, const double* lamy, int nyt, double* m, double* e,
+                           T* d, cudaStream_t s) {
   const size_t ntc = (size_t)nyt * g.nxh;
-  k_setup_z64<<<(int)((ntc + 127) / 128), 128, 0, s>>>(g, lamx, lamy, nyt, m, e, d);
+  k_setup_z<T><<<(int)((ntc + 127) / 128), 128, 0, s>>>(g, lamx, lamy, nyt, m, e, d);
   return cudaGetLastError();
 }
+template cudaError_t launch_setup_z<float>(const Geo&, const double*, const double*, int, double*, double*, float*,
+                                           cudaStream_t);
+template cudaError_t launch_setup_z<double>(const Geo&, const double*, const double*, int, double*, double*, double*,
+                                            cudaStream_t);
 
 cudaError_t launch_adj_rhs(const Geo& g, const double* rho, const double* gu, const double* gv,
                            const double* gw, double dt, double* yu, double* yv, double* yw,

@@ -9,6 +9,7 @@
 #include <type_traits>
 
 #include "pp_fft.cuh"
+#include "pp_zsweep.cuh"
 
 namespace pp {
 
@@ -890,178 +891,6 @@ __device__ __forceinline__ void thomas_column(const Geo& g, const double* __rest
   }
 }
 
-// dzf-weighted z means of the real and imaginary parts of column 0 (scalar
-// view T[nz][2 ncol]), reduced by the whole block; returned in sh[0], sh[1]
-// (sh: at least 34 entries) after a barrier.  Every thread must call it.
-template <typename T>
-__device__ __forceinline__ void zero_column_means(const Geo& g, const T* spec, size_t stride, double* sh) {
-  double sx = 0.0, sy = 0.0;
-  for (int k = threadIdx.x; k < g.nz; k += blockDim.x) {
-    sx += g.dzf[k] * (double)spec[(size_t)k * stride];
-    sy += g.dzf[k] * (double)spec[(size_t)k * stride + 1];
-  }
-  sx = block_sum<double>(sx, sh);
-  __syncthreads();
-  sy = block_sum<double>(sy, sh);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    sh[32] = sx / g.lz;
-    sh[33] = sy / g.lz;
-  }
-  __syncthreads();
-}
-
-// The same solve with the real and imaginary parts of a column in two
-// threads (twice the parallelism) and the elimination multipliers
-// m_k = a_k / d_{k-1} read from a table: per scalar one FP64 FMA forward and
-// one FMA + one multiply backward.  The recurrences run in FP64 registers;
-// the forward-sweep values are stored in place in the spectrum's own
-// precision (FP32 on mixed plans, like the spectrum the solve reads and
-// writes).  Scalar view: spec as T[nz][2 ncol].  m0 is subtracted from every
-// right-hand-side value: the dzf-weighted z mean of the singular (0, 0)
-// column, 0 for every other column.
-template <typename T>
-__device__ __forceinline__ void stage_tridiag_split(const Geo& g, const double* __restrict__ mtab,
-                                                    const double* __restrict__ invd, T* spec,
-                                                    size_t sid, double m0 = 0.0) {
-  constexpr int PF = 4;
-  const size_t ncol = (size_t)g.ny * g.nxh;
-  if (sid >= 2 * ncol) return;
-  const size_t col = sid >> 1;
-  const size_t stride = 2 * ncol;
-  const int nz = g.nz;
-  auto ld = [&](size_t o) -> double {
-    if (sizeof(T) == sizeof(float)) return widen_f32((float)spec[o]);
-    return (double)spec[o];
-  };
-  auto stv = [&](size_t o, double v) {
-    if (sizeof(T) == sizeof(float)) spec[o] = (T)narrow_f64(v);
-    else spec[o] = (T)v;
-  };
-  double fq[PF], mq[PF];
-#pragma unroll
-  for (int u = 0; u < PF; ++u) {
-    const int k = u < nz ? u : nz - 1;
-    fq[u] = ld((size_t)k * stride + sid);
-    mq[u] = mtab[(size_t)k * ncol + col];
-  }
-  double y = 0.0;
-  for (int k0 = 0; k0 < nz; k0 += PF) {
-#pragma unroll
-    for (int u = 0; u < PF; ++u) {
-      const int k = k0 + u;
-      if (k < nz) {
-        const double f = fq[u], m = mq[u];
-        const int kn = k + PF < nz ? k + PF : nz - 1;
-        fq[u] = ld((size_t)kn * stride + sid);
-        mq[u] = mtab[(size_t)kn * ncol + col];
-        y = fma(-m, y, f - m0);
-        if (k < nz - 1) stv((size_t)k * stride + sid, y);
-      }
-    }
-  }
-  double x = y * invd[(size_t)(nz - 1) * ncol + col];
-  stv((size_t)(nz - 1) * stride + sid, x);
-  double yq[PF], dq[PF];
-#pragma unroll
-  for (int u = 0; u < PF; ++u) {
-    const int k = nz - 2 - u >= 0 ? nz - 2 - u : 0;
-    yq[u] = ld((size_t)k * stride + sid);
-    dq[u] = invd[(size_t)k * ncol + col];
-  }
-  for (int k0 = nz - 2; k0 >= 0; k0 -= PF) {
-#pragma unroll
-    for (int u = 0; u < PF; ++u) {
-      const int k = k0 - u;
-      if (k >= 0) {
-        const double yy = yq[u], d = dq[u];
-        const int kn = k - PF >= 0 ? k - PF : 0;
-        yq[u] = ld((size_t)kn * stride + sid);
-        dq[u] = invd[(size_t)kn * ncol + col];
-        x = fma(-g.zc[k], x, yy) * d;
-        stv((size_t)k * stride + sid, x);
-      }
-    }
-  }
-}
-
-// One column of a PP_MIXED_Z64 plan (TriZ64), both components in one thread
-// (two independent FP64 chains sharing the table loads): both sweeps are
-// FP64 recurrences with one FMA per row and component; the spectrum keeps
-// its FP32 storage, so the forward values are stored as s_k = (1/d_k) y_k,
-// rounded to FP32 and multiplied by the FP32 inverse pivot (the same 2^-24
-// relative perturbation per value as storing y_k itself).  ZERO: the
-// singular column 0, whose right-hand side first loses its dzf-weighted z
-// mean (m0x, m0y).  Loads run PF rows ahead.  32-bit offsets: the plan keeps
-// nx ny (nz + 1) below 2^31.
-template <bool ZERO>
-__device__ __forceinline__ void stage_tridiag_z64(const Geo& g, const TriZ64& t, float2* __restrict__ spec,
-                                                  unsigned col, unsigned ncol, unsigned tc, unsigned ntc,
-                                                  double m0x, double m0y) {
-  constexpr int PF = 4;
-  const int nz = g.nz;
-  const double* __restrict__ tm = t.m;
-  const double* __restrict__ te = t.e;
-  const float* __restrict__ td = t.d;
-  float2 fq[PF];
-  float dq[PF];
-  double mq[PF];
-#pragma unroll
-  for (int u = 0; u < PF; ++u) {
-    const unsigned k = u < nz ? u : nz - 1;
-    fq[u] = spec[k * ncol + col];
-    mq[u] = tm[k * ntc + tc];
-    dq[u] = td[k * ntc + tc];
-  }
-  double yx = 0.0, yy = 0.0;
-  float2 s = make_float2(0.f, 0.f);
-  for (int k0 = 0; k0 < nz; k0 += PF) {
-#pragma unroll
-    for (int u = 0; u < PF; ++u) {
-      const int k = k0 + u;
-      if (k < nz) {
-        const double fx = widen_f32(fq[u].x), fy = widen_f32(fq[u].y);
-        const double m = mq[u];
-        const float dk = dq[u];
-        const unsigned kn = k + PF < nz ? k + PF : nz - 1;
-        fq[u] = spec[kn * ncol + col];
-        mq[u] = tm[kn * ntc + tc];
-        dq[u] = td[kn * ntc + tc];
-        yx = fma(-m, yx, ZERO ? fx - m0x : fx);
-        yy = fma(-m, yy, ZERO ? fy - m0y : fy);
-        s = make_float2(narrow_f64(yx) * dk, narrow_f64(yy) * dk);
-        spec[(unsigned)k * ncol + col] = s;
-      }
-    }
-  }
-  // x_{nz-1} = s_{nz-1} (already stored); backward from row nz - 2
-  double xx = widen_f32(s.x), xy = widen_f32(s.y);
-  float2 sq[PF];
-  double eq[PF];
-#pragma unroll
-  for (int u = 0; u < PF; ++u) {
-    const unsigned k = nz - 2 - u >= 0 ? nz - 2 - u : 0;
-    sq[u] = spec[k * ncol + col];
-    eq[u] = te[k * ntc + tc];
-  }
-  for (int k0 = nz - 2; k0 >= 0; k0 -= PF) {
-#pragma unroll
-    for (int u = 0; u < PF; ++u) {
-      const int k = k0 - u;
-      if (k >= 0) {
-        const double sx = widen_f32(sq[u].x), sy = widen_f32(sq[u].y);
-        const double e = eq[u];
-        const unsigned kn = k - PF >= 0 ? k - PF : 0;
-        sq[u] = spec[kn * ncol + col];
-        eq[u] = te[kn * ntc + tc];
-        xx = fma(-e, xx, sx);
-        xy = fma(-e, xy, sy);
-        spec[(unsigned)k * ncol + col] = make_float2(narrow_f64(xx), narrow_f64(xy));
-      }
-    }
-  }
-}
-
 // One ill-conditioned column of a mixed plan, solved by a whole warp in
 // FP64.  Both sweeps of the Thomas elimination are first-order affine
 // recurrences,
@@ -1070,7 +899,7 @@ __device__ __forceinline__ void stage_tridiag_z64(const Geo& g, const TriZ64& t,
 // so each lane composes the maps of its R = ceil(nz/32) consecutive rows, a
 // shuffle scan combines the lanes' maps, and each lane replays its rows from
 // the value entering its segment.  The values stay FP32 in memory (the
-// intermediate y too, as in stage_tridiag_split); the recurrences run in
+// intermediate y too); the recurrences run in
 // FP64.  Column 0 (the singular (0, 0) system, its last pivot pinned) first
 // loses its dzf-weighted z mean.
 __device__ __forceinline__ void tridiag_col_warp64(const Geo& g, const double* __restrict__ mtab,
@@ -1165,69 +994,19 @@ __device__ __forceinline__ void tridiag_col_warp64(const Geo& g, const double* _
 }
 
 // Mixed plans, one thread per (kx, ky) column holding both components, in
-// FP32 with FP32 tables (float2 loads and stores of the spectrum).  Only the well-conditioned columns (TriF32) take this path;
-// column 0 and the other ill-conditioned columns are left to
+// FP32 with FP32 tables.  Only the well-conditioned columns (TriF32) take
+// this path; column 0 and the other ill-conditioned columns are left to
 // tridiag_col_warp64.
-__device__ __forceinline__ void stage_tridiag_col32(const Geo& g, const TriF32& f, float2* spec, size_t col) {
-  constexpr int PF = 1;  // deeper register prefetch (2-16 rows) measured slower at 512^3
+__device__ __forceinline__ void stage_tridiag_col32(const Geo& g, const TriF32& f, float2* spec, size_t col,
+                                                    unsigned char* smem) {
   const size_t ncol = (size_t)g.ny * g.nxh;
   if (col >= ncol) return;
-  const int j = (int)(col / (size_t)g.nxh);
+  const int j = (int)((unsigned)col / (unsigned)g.nxh);
   const int kx = (int)(col - (size_t)j * g.nxh);
   if (col == 0 || fabs(f.lamx[kx] + f.lamy[j]) < f.thr) return;
-  const int nz = g.nz;
-  float2 fq[PF];
-  float mq[PF];
-#pragma unroll
-  for (int u = 0; u < PF; ++u) {
-    const int k = u < nz ? u : nz - 1;
-    fq[u] = spec[(size_t)k * ncol + col];
-    mq[u] = f.mtab[(size_t)k * ncol + col];
-  }
-  float2 y = make_float2(0.f, 0.f);
-  for (int k0 = 0; k0 < nz; k0 += PF) {
-#pragma unroll
-    for (int u = 0; u < PF; ++u) {
-      const int k = k0 + u;
-      if (k < nz) {
-        const float2 fv = fq[u];
-        const float m = mq[u];
-        const int kn = k + PF < nz ? k + PF : nz - 1;
-        fq[u] = spec[(size_t)kn * ncol + col];
-        mq[u] = f.mtab[(size_t)kn * ncol + col];
-        y.x = fmaf(-m, y.x, fv.x);
-        y.y = fmaf(-m, y.y, fv.y);
-        if (k < nz - 1) spec[(size_t)k * ncol + col] = y;
-      }
-    }
-  }
-  const float dl = f.invd[(size_t)(nz - 1) * ncol + col];
-  float2 x = make_float2(y.x * dl, y.y * dl);
-  spec[(size_t)(nz - 1) * ncol + col] = x;
-  float2 yq[PF];
-  float dq[PF];
-#pragma unroll
-  for (int u = 0; u < PF; ++u) {
-    const int k = nz - 2 - u >= 0 ? nz - 2 - u : 0;
-    yq[u] = spec[(size_t)k * ncol + col];
-    dq[u] = f.invd[(size_t)k * ncol + col];
-  }
-  for (int k0 = nz - 2; k0 >= 0; k0 -= PF) {
-#pragma unroll
-    for (int u = 0; u < PF; ++u) {
-      const int k = k0 - u;
-      if (k >= 0) {
-        const float2 yy = yq[u];
-        const float d = dq[u], c = f.zc[k];
-        const int kn = k - PF >= 0 ? k - PF : 0;
-        yq[u] = spec[(size_t)kn * ncol + col];
-        dq[u] = f.invd[(size_t)kn * ncol + col];
-        x.x = fmaf(-c, x.x, yy.x) * d;
-        x.y = fmaf(-c, x.y, yy.y) * d;
-        spec[(size_t)k * ncol + col] = x;
-      }
-    }
-  }
+  const ZForm32 form{f.mtab, nullptr, f.invd};
+  float2* const vals[1] = {spec + col};
+  zsweep<ZForm32, 1, false>(form, vals, ncol, col, ncol, g.nz, f.zc, smem, 0.0, 0.0);
 }
 
 // Block b of the mixed z solve: the first nblk_low blocks give one warp to
@@ -1235,14 +1014,15 @@ __device__ __forceinline__ void stage_tridiag_col32(const Geo& g, const TriF32& 
 // the longest), the rest one thread to each column.  Block-uniform branch.
 __device__ __forceinline__ void stage_tridiag_mixed(const Geo& g, const double* __restrict__ mtab,
                                                     const double* __restrict__ invd, const TriF32& f,
-                                                    float2* spec, int b) {
-  const int nblk_low = (f.nlow + 3) >> 2;
+                                                    float2* spec, int b, unsigned char* smem) {
+  constexpr int kWarps = kZThreads / 32;
+  const int nblk_low = (f.nlow + kWarps - 1) / kWarps;
   if (b < nblk_low) {
-    const int w = b * 4 + (threadIdx.x >> 5);
+    const int w = b * kWarps + (threadIdx.x >> 5);
     if (w < f.nlow) tridiag_col_warp64(g, mtab, invd, spec, (size_t)f.low[w], (size_t)g.ny * g.nxh);
     return;
   }
-  stage_tridiag_col32(g, f, spec, (size_t)(b - nblk_low) * blockDim.x + threadIdx.x);
+  stage_tridiag_col32(g, f, spec, (size_t)(b - nblk_low) * kZThreads + threadIdx.x, smem);
 }
 
 // Inverse x transform of two half spectra per complex sequence, then
