@@ -277,7 +277,7 @@ pp_status solve_pass(pp_plan_s* P, double* p, int p_zero, T* delta = nullptr, fl
   const bool ytc = P->ystretch && std::is_same<T, float>::value;
   C2<T>* zs = ytc ? (C2<T>*)P->d_spec2 : spec;
   // the dense y step of a stretched y is W-orthonormal: no 1/ny on the way back
-  const double scale = 1.0 / ((double)P->nx * (P->ystretch ? 1.0 : (double)P->ny));
+  const double scale = kSpecScale / ((double)P->nx * (P->ystretch ? 1.0 : (double)P->ny));
   const C2<T>* dct = (const C2<T>*)P->d_dcty;  // null: periodic y
   auto ytc_args = [&](const void* x, void* y, const unsigned char* mat) {
     DenseTcArgs a{};

@@ -12,8 +12,9 @@
 #include <new>
 #include <vector>
 
+#include "pp_batch.cuh"
 #include "pp_cells.cuh"
-#include "pp_stages.cuh"
+#include "pp_wfft.cuh"
 
 using namespace pp;
 
@@ -21,33 +22,6 @@ namespace {
 
 constexpr int kChunk = 2048;  // cells per block of the elementwise grouped kernels
 constexpr int kExactEveryBatch = 40;
-
-struct GridDev {
-  Geo g;
-  Faces fc;
-  FftDesc fx, fy;
-  const float2* twx;
-  const float2* twy;
-  const float2* dcty;  // walls in y: exp(-i pi m / (2 ny)); null: periodic y
-  const double* invd;
-  const double* mtab;
-  TriF32 tri;  // FP32 tables of the well-conditioned z columns
-  float2* spec;
-  float* E;
-  float* delta;
-  float* sdelta;  // increments not yet added to p (lazy update, stage_fftx_inv)
-  double* b;
-  double* red;
-  DevStatus* st;
-  // per call: this grid's fields inside the caller's packed buffers
-  const double *us, *vs, *ws, *rho, *S;
-  double *p, *u, *v, *w;
-  double dt, inv_dt, scale;
-  int rpb, nblk_x;  // x kernels: rows per block, blocks
-  int tx, ntx;      // y kernels: kx tile, tiles per plane
-  int nchunk;       // elementwise chunks
-  long long ncell;
-};
 
 struct BatchCtl {
   double rtol;
@@ -260,6 +234,10 @@ struct pp_batch_s {
   int2 *w_cells = nullptr, *w_x = nullptr, *w_y = nullptr, *w_z = nullptr;
   int n_cells = 0, n_x = 0, n_y = 0, n_z = 0;
   size_t smem_x = 0, smem_y = 0;
+  // the grids whose x (y) length has a register transform (pp_wfft.cuh)
+  int2 *w_xw = nullptr, *w_yw = nullptr;
+  int n_xw = 0, n_yw = 0;
+  size_t smem_xw = 0, smem_yw = 0;
   int ept_x = kEpt, ept_y = kEpt;  // chosen by the tuner
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -276,7 +254,7 @@ void free_batch(pp_batch_s* B) {
   if (B->d_low) cudaFree(B->d_low);
   if (B->d_dev) cudaFree(B->d_dev);
   if (B->d_ctl) cudaFree(B->d_ctl);
-  int2* ws[] = {B->w_cells, B->w_x, B->w_y, B->w_z};
+  int2* ws[] = {B->w_cells, B->w_x, B->w_y, B->w_z, B->w_xw, B->w_yw};
   for (int2* w : ws) if (w) cudaFree(w);
   if (B->h_dev) cudaFreeHost(B->h_dev);
   if (B->h_ctl) cudaFreeHost(B->h_ctl);
@@ -295,24 +273,39 @@ pp_status upload_list(const std::vector<int2>& h, int2** d, int* n) {
 }
 
 // Work lists for the x kernels (rows) and y kernels (tiles) for given
-// elements-per-thread choices; updates rpb/nblk_x/tx/ntx in the mirror.
+// elements-per-thread choices; updates rpb/nblk_x/tx/ntx in the mirror.  Grids
+// with a register transform in x (y) go to the lists w_xw (w_yw), which the
+// choices do not touch.
 pp_status build_fft_lists(pp_batch_s* B, int ept_x, int ept_y) {
-  std::vector<int2> wx, wy;
+  std::vector<int2> wx, wy, wxw, wyw;
   size_t sx = 0, sy = 0;
+  B->smem_xw = B->smem_yw = 0;
   for (int i = 0; i < B->n; ++i) {
     GridDev& d = B->h_dev[i];
-    d.rpb = rows_per_block(d.g.nx, ept_x);
     const int nrows = d.g.nz * d.g.ny;
-    d.nblk_x = (nrows + d.rpb - 1) / d.rpb;
-    for (int b = 0; b < d.nblk_x; ++b) wx.push_back(make_int2(i, b));
-    {  // buffer A, buffer B written padded, twiddle table
+    BatchWShape sh;
+    if (wfft_length(d.g.nx)) {
+      batch_wfft_x(d.g.nx, nrows, &sh);
+      d.rpb = 0;
+      d.nblk_x = sh.nred;
+      for (int b = 0; b < sh.nblk_x; ++b) wxw.push_back(make_int2(i, b));
+      B->smem_xw = std::max(B->smem_xw, sh.smem_x);
+    } else {
+      d.rpb = rows_per_block(d.g.nx, ept_x);
+      d.nblk_x = (nrows + d.rpb - 1) / d.rpb;
+      for (int b = 0; b < d.nblk_x; ++b) wx.push_back(make_int2(i, b));
+      // buffer A, buffer B written padded, twiddle table
       const int nbuf = (d.rpb / 2) * d.g.nx;
       sx = std::max(sx, (size_t)(nbuf + fft_pad_elems(nbuf) + d.g.nx) * sizeof(float2));
     }
-    d.tx = ffty_tile(d.g.ny, sizeof(float2), ept_y);
-    d.ntx = (d.g.nxh + d.tx - 1) / d.tx;
-    for (int b = 0; b < d.ntx * d.g.nz; ++b) wy.push_back(make_int2(i, b));
-    {
+    if (wfft_length(d.g.ny)) {
+      batch_wfft_y(d.g.ny, d.g.nxh, d.g.nz, &sh);
+      for (int b = 0; b < sh.ngroups_y; ++b) wyw.push_back(make_int2(i, b));
+      B->smem_yw = std::max(B->smem_yw, sh.smem_y);
+    } else {
+      d.tx = ffty_tile(d.g.ny, sizeof(float2), ept_y);
+      d.ntx = (d.g.nxh + d.tx - 1) / d.tx;
+      for (int b = 0; b < d.ntx * d.g.nz; ++b) wy.push_back(make_int2(i, b));
       const int tsz = d.g.ny * d.tx;
       sy = std::max(sy, (size_t)(tsz + fft_pad_elems(tsz) + d.g.ny) * sizeof(float2));
     }
@@ -320,19 +313,25 @@ pp_status build_fft_lists(pp_batch_s* B, int ept_x, int ept_y) {
   B->smem_x = sx;
   B->smem_y = sy;
   pp_status s;
-  if ((s = upload_list(wx, &B->w_x, &B->n_x)) != PP_OK) return s;
-  if ((s = upload_list(wy, &B->w_y, &B->n_y)) != PP_OK) return s;
+  if ((s = upload_list(wx, &B->w_x, &B->n_x)) != PP_OK || (s = upload_list(wy, &B->w_y, &B->n_y)) != PP_OK ||
+      (s = upload_list(wxw, &B->w_xw, &B->n_xw)) != PP_OK || (s = upload_list(wyw, &B->w_yw, &B->n_yw)) != PP_OK)
+    return s;
   return cudaMemcpy(B->d_dev, B->h_dev, B->n * sizeof(GridDev), cudaMemcpyHostToDevice) == cudaSuccess
              ? PP_OK : PP_ERR_CUDA;
 }
 
 cudaError_t launch_pass(pp_batch_s* B, cudaStream_t s) {
-  kb_resid<<<B->n_x, kThreads, B->smem_x, s>>>(B->d_dev, B->w_x);
+  cudaError_t e;
+  if (B->n_x) kb_resid<<<B->n_x, kThreads, B->smem_x, s>>>(B->d_dev, B->w_x);
+  if (B->n_xw && (e = launch_batch_resid_w(B->d_dev, B->w_xw, B->n_xw, B->smem_xw, s)) != cudaSuccess) return e;
   kb_check<<<B->n, 1024, 0, s>>>(B->d_dev, B->d_ctl, kExactEveryBatch);
-  kb_ffty<-1><<<B->n_y, kThreads, B->smem_y, s>>>(B->d_dev, B->w_y);
+  if (B->n_y) kb_ffty<-1><<<B->n_y, kThreads, B->smem_y, s>>>(B->d_dev, B->w_y);
+  if (B->n_yw && (e = launch_batch_ffty_w(B->d_dev, B->w_yw, B->n_yw, B->smem_yw, 0, s)) != cudaSuccess) return e;
   kb_tridiag<<<B->n_z, kZThreads, zsweep_smem<ZForm32, 1>(), s>>>(B->d_dev, B->w_z);
-  kb_ffty<1><<<B->n_y, kThreads, B->smem_y, s>>>(B->d_dev, B->w_y);
-  kb_fftx_inv<<<B->n_x, kThreads, B->smem_x, s>>>(B->d_dev, B->w_x);
+  if (B->n_y) kb_ffty<1><<<B->n_y, kThreads, B->smem_y, s>>>(B->d_dev, B->w_y);
+  if (B->n_yw && (e = launch_batch_ffty_w(B->d_dev, B->w_yw, B->n_yw, B->smem_yw, 1, s)) != cudaSuccess) return e;
+  if (B->n_x) kb_fftx_inv<<<B->n_x, kThreads, B->smem_x, s>>>(B->d_dev, B->w_x);
+  if (B->n_xw && (e = launch_batch_fftx_inv_w(B->d_dev, B->w_xw, B->n_xw, B->smem_xw, s)) != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
@@ -357,9 +356,14 @@ cudaError_t launch_post(pp_batch_s* B, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// Time `reps` launches of the transform kernels for each candidate and keep
-// the fastest (x kernels and y kernels are chosen independently).
+// Time `reps` launches of the shared-memory transform kernels for each
+// candidate and keep the fastest (x kernels and y kernels are chosen
+// independently).  Nothing to choose where every grid has register transforms.
 pp_status autotune(pp_batch_s* B) {
+  bool any = false;
+  for (int i = 0; i < B->n; ++i)
+    any = any || !wfft_length(B->h_dev[i].g.nx) || !wfft_length(B->h_dev[i].g.ny);
+  if (!any) return build_fft_lists(B, kEpt, kEpt);
   const int cands[3] = {4, 8, 16};
   cudaEvent_t a, b;
   if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess) return PP_ERR_CUDA;
@@ -372,14 +376,18 @@ pp_status autotune(pp_batch_s* B) {
     for (int rep = 0; rep < 2; ++rep) {  // first repetition warms up
       float tx = 0.f, ty = 0.f;
       cudaEventRecord(a, B->cap);
-      kb_resid<<<B->n_x, kThreads, B->smem_x, B->cap>>>(B->d_dev, B->w_x);
-      kb_fftx_inv<<<B->n_x, kThreads, B->smem_x, B->cap>>>(B->d_dev, B->w_x);
+      if (B->n_x) {
+        kb_resid<<<B->n_x, kThreads, B->smem_x, B->cap>>>(B->d_dev, B->w_x);
+        kb_fftx_inv<<<B->n_x, kThreads, B->smem_x, B->cap>>>(B->d_dev, B->w_x);
+      }
       cudaEventRecord(b, B->cap);
       if (cudaEventSynchronize(b) != cudaSuccess) { s = PP_ERR_CUDA; break; }
       cudaEventElapsedTime(&tx, a, b);
       cudaEventRecord(a, B->cap);
-      kb_ffty<-1><<<B->n_y, kThreads, B->smem_y, B->cap>>>(B->d_dev, B->w_y);
-      kb_ffty<1><<<B->n_y, kThreads, B->smem_y, B->cap>>>(B->d_dev, B->w_y);
+      if (B->n_y) {
+        kb_ffty<-1><<<B->n_y, kThreads, B->smem_y, B->cap>>>(B->d_dev, B->w_y);
+        kb_ffty<1><<<B->n_y, kThreads, B->smem_y, B->cap>>>(B->d_dev, B->w_y);
+      }
       cudaEventRecord(b, B->cap);
       if (cudaEventSynchronize(b) != cudaSuccess) { s = PP_ERR_CUDA; break; }
       cudaEventElapsedTime(&ty, a, b);
@@ -595,7 +603,7 @@ pp_status pressure_batch_create(const pp_grid* grids, int ngrids, pp_precision p
     d.b = (double*)(P + o.b); d.red = (double*)(P + o.red); d.st = (DevStatus*)(P + o.st);
     d.ncell = (long long)nx * ny * nz;
     d.nchunk = (int)((d.ncell + kChunk - 1) / kChunk);
-    d.scale = 1.0 / ((double)nx * ny);
+    d.scale = kSpecScale / ((double)nx * ny);
     for (int c = 0; c < d.nchunk; ++c) wc.push_back(make_int2(i, c));
     const size_t ncol = (size_t)nxh * ny;
     const std::vector<int> lowi = tri_low_columns(lamx, lamy, 2.0 * dmax / 512.0);

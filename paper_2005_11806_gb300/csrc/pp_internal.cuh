@@ -11,6 +11,10 @@
 namespace pp {
 
 constexpr int kMaxStages = 16;
+// The forward x transform leaves every spectrum doubled (it separates two rows
+// without the halving products); the scale of the inverse x transform carries
+// this factor.
+constexpr double kSpecScale = 0.5;
 
 // Mixed-radix factorisation of one FFT length (radices 8, 4, 2, 3, 5).
 struct FftDesc {
@@ -103,9 +107,17 @@ __device__ __forceinline__ double widen_f32(float f) {
   return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)lo);
 }
 
+// 1 / x to 1 ulp, one instruction (no range checks: x is a sum of two
+// densities; Inf gives 0).
+__device__ __forceinline__ float rcp_f32(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // 1 / rho_f of a face from its two cells' FP32 densities (arithmetic face
-// density, as the FP64 coefficients): 2 / (a + b), fast FP32 division.
-__device__ __forceinline__ float face_beta_f(float a, float b) { return __fdividef(2.f, a + b); }
+// density, as the FP64 coefficients): 2 / (a + b).
+__device__ __forceinline__ float face_beta_f(float a, float b) { return 2.f * rcp_f32(a + b); }
 
 // Host: whether the n + 1 face coordinates f[0..n] are finite and strictly
 // increasing (the grid descriptor's zfaces / yfaces).
@@ -157,6 +169,28 @@ cudaError_t launch_resid_fftx(const Geo& g, const Faces& fc, const FftDesc& fx, 
                               int p_zero, int scale_rho, C2<T>* spec, double* red, int* nblk_out,
                               const DevStatus* st, cudaStream_t s, float* E = nullptr,
                               const float* delta = nullptr);
+// The same steps for the lengths of PP_WFFT_LENGTHS (pp_wfft.cuh); the
+// launchers route such plans to them.
+template <typename T>
+cudaError_t launch_resid_w(const Geo& g, const Faces& fc, const C2<T>* twx, const double* b, const double* rho,
+                           const double* p, int p_zero, int scale_rho, C2<T>* spec, double* red, int* nblk_out,
+                           const DevStatus* st, cudaStream_t s, float* E, const float* delta);
+template <typename T>
+cudaError_t launch_ffty_w(const Geo& g, const C2<T>* twy, C2<T>* spec, int inverse, const DevStatus* st,
+                          cudaStream_t s, const C2<T>* dct);
+template <typename T>
+cudaError_t launch_fftx_inv_w(const Geo& g, const C2<T>* twx, const C2<T>* spec, double scale, double* p, int p_zero,
+                              const DevStatus* st, cudaStream_t s, T* delta, float* sdelta);
+template <> cudaError_t launch_resid_w<float>(const Geo&, const Faces&, const C2<float>*, const double*, const double*,
+                                            const double*, int, int, C2<float>*, double*, int*, const DevStatus*,
+                                            cudaStream_t, float*, const float*);
+template <> cudaError_t launch_ffty_w<float>(const Geo&, const C2<float>*, C2<float>*, int, const DevStatus*, cudaStream_t,
+                                           const C2<float>*);
+template <> cudaError_t launch_resid_w<double>(const Geo&, const Faces&, const C2<double>*, const double*, const double*,
+                                            const double*, int, int, C2<double>*, double*, int*, const DevStatus*,
+                                            cudaStream_t, float*, const float*);
+template <> cudaError_t launch_ffty_w<double>(const Geo&, const C2<double>*, C2<double>*, int, const DevStatus*, cudaStream_t,
+                                           const C2<double>*);
 // z solve of a uniform walled z by the cosine basis (FP64 plans): forward
 // transform with the eigenvalue divide (inverse = 0), then the inverse
 // transform (inverse = 1).  dct: exp(-i pi m / (2 nz)); zd: the eigenvalues.

@@ -3,6 +3,7 @@
 #include <cmath>
 
 #include "pp_stages.cuh"
+#include "pp_wfft.cuh"
 
 namespace pp {
 
@@ -145,6 +146,8 @@ cudaError_t launch_resid_fftx(const Geo& g, const Faces& fc, const FftDesc& fx, 
                               const double* b, double inv_dt, const double* rho, const double* p,
                               int p_zero, int scale_rho, C2<T>* spec, double* red, int* nblk_out,
                               const DevStatus* st, cudaStream_t s, float* E, const float* delta) {
+  if (wfft_length(g.nx))
+    return launch_resid_w<T>(g, fc, twx, b, rho, p, p_zero, scale_rho, spec, red, nblk_out, st, s, E, delta);
   const int rpb = rows_per_block(g.nx, kEpt);
   const long nrows = (long)g.nz * g.ny;
   const int nblk = (int)((nrows + rpb - 1) / rpb);
@@ -172,6 +175,7 @@ cudaError_t launch_ffty(const Geo& g, const FftDesc& fy, const C2<T>* twy, C2<T>
     if (g.ny == 512 && dct == nullptr)
       return launch_ffty512(g, reinterpret_cast<const float2*>(twy), reinterpret_cast<float2*>(spec), inverse, st, s);
   }
+  if (wfft_length(g.ny)) return launch_ffty_w<T>(g, twy, spec, inverse, st, s, dct);
   const int tx = ffty_tile(g.ny, sizeof(C2<T>), kEpt);
   const int tsz = g.ny * tx;
   const size_t smem = (sizeof(T) == sizeof(float))
@@ -304,6 +308,7 @@ cudaError_t launch_fftx_inv(const Geo& g, const FftDesc& fx, const C2<T>* twx, c
       return launch_fftx512_inv(g, reinterpret_cast<const float2*>(twx), reinterpret_cast<const float2*>(spec),
                                 scale, p, p_zero, st, s, delta, sdelta);
   }
+  if (wfft_length(g.nx)) return launch_fftx_inv_w<T>(g, twx, spec, scale, p, p_zero, st, s, delta, sdelta);
   const int rpb = rows_per_block(g.nx, kEpt);
   const long nrows = (long)g.nz * g.ny;
   const int nblk = (int)((nrows + rpb - 1) / rpb);

@@ -249,7 +249,7 @@ extern "C" pp_status pressure_solve_noalloc(const pp_grid* grid, const double* f
   double* red = (double*)(S + o_red);
   DevStatus* st = (DevStatus*)(S + o_st);
   Faces none{nullptr, nullptr, nullptr};
-  const double scale = 1.0 / ((double)nx * (double)ny);
+  const double scale = kSpecScale / ((double)nx * (double)ny);
   // The status word starts cleared and the pivots are rebuilt: the array
   // still holds whatever the previous call left in it.
   if (launch_init_status(st, s) != cudaSuccess ||

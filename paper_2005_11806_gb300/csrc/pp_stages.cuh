@@ -123,20 +123,104 @@ __device__ __forceinline__ void load_twiddles_smem(const float2* __restrict__ tw
 // ---------------------------------------------------------------------------
 // Update pass of the mixed residual for nx % 4 == 0, vectorised: each thread
 // takes the two rows of one complex sequence and four consecutive cells of
-// each (16-byte loads of E, delta and the FP32 coefficients, all issued
-// before the arithmetic), subtracts A delta = sum_nb c_nb (delta_nb -
-// delta_c) from E, and writes the scaled residual of both rows as two
-// interleaved complex pairs.  Same per-cell arithmetic as the scalar path.
+// each (16-byte loads of E, delta and the FP32 density), subtracts A delta
+// from E, and writes the scaled residual of both rows as two interleaved
+// complex pairs.
+//
+// A delta is formed from half fluxes G = (delta_b - delta_a) / (rho_a +
+// rho_b), one per face: an add, an add, a reciprocal and a multiply, shared
+// by the face's two cells where both are in the thread (5 x faces for 4
+// cells; with two rows taken together 3 y faces for 2 cells), then
+//   A delta = 2 [w_x (G_x+ - G_x-) + w_y+ G_y+ - w_y- G_y- + w_z+ G_z+ - w_z- G_z-]
+// with the layer (and row) factors w.  Coefficients formed per cell and face
+// took 131 instructions a cell, 35 of them range checks and selects of the
+// division; this form takes about 80.
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float half_flux(float da, float db, float ha, float hb) {
+  return (db - da) * rcp_f32(ha + hb);
+}
+__device__ __forceinline__ float4 half_flux4(float4 da, float4 db, float4 ha, float4 hb) {
+  return make_float4(half_flux(da.x, db.x, ha.x, hb.x), half_flux(da.y, db.y, ha.y, hb.y),
+                     half_flux(da.z, db.z, ha.z, hb.z), half_flux(da.w, db.w, ha.w, hb.w));
+}
 
+// Factors of one row (all carry the 2 of the fluxes): x faces, y faces below
+// and above, z faces below and above, 1 / dzf (1 / (dzf s_j) on a stretched
+// y), the scaling of the residual where it is constant.
+struct RowW {
+  float x, yl, yh, zd, zu, iv;
+};
+
+// The four cells of a row at offset c: their E updated in place, their
+// scaled residuals returned, e^2 and |e| added to s2 and s1.  Gl, Gh: the
+// half fluxes of the y faces below and above.
+__device__ __forceinline__ float4 resid_row4(const RowW& w, float* __restrict__ E, const float* __restrict__ delta,
+                                             const float* __restrict__ rhof, unsigned c, unsigned il, unsigned ir,
+                                             unsigned plane, bool up, bool dn, float4 d, float4 h, float4 Gl,
+                                             float4 Gh, bool scale, bool own, float rt_f, float& s2, float& s1) {
+  const float dl = delta[il], dr = delta[ir], hl = rhof[il], hr = rhof[ir];
+  float4 du = d, dd = d, hu = h, hd = h;
+  if (up) { du = ld4(delta + c + plane); hu = ld4(rhof + c + plane); }
+  if (dn) { dd = ld4(delta + c - plane); hd = ld4(rhof + c - plane); }
+  float4 e = ld4(E + c);
+  const float x0 = half_flux(dl, d.x, hl, h.x), x1 = half_flux(d.x, d.y, h.x, h.y), x2 = half_flux(d.y, d.z, h.y, h.z),
+              x3 = half_flux(d.z, d.w, h.z, h.w), x4 = half_flux(d.w, dr, h.w, hr);
+  const float4 Gu = half_flux4(d, du, h, hu), Gd = half_flux4(dd, d, hd, h);
+  auto cell = [&](float xm, float xp, float gl, float gh, float gd, float gu, float& ev, float hv) -> float {
+    float t = w.x * (xp - xm);
+    t = fmaf(w.yh, gh, t);
+    t = fmaf(-w.yl, gl, t);
+    t = fmaf(w.zu, gu, t);
+    t = fmaf(-w.zd, gd, t);
+    ev = ev - t;
+    const float ee = ev * w.iv;
+    s2 = fmaf(ee, ee, s2);
+    s1 += fabsf(ee);
+    return scale ? (own ? hv : rt_f) * ee : ee;
+  };
+  float4 r;
+  r.x = cell(x0, x1, Gl.x, Gh.x, Gd.x, Gu.x, e.x, h.x);
+  r.y = cell(x1, x2, Gl.y, Gh.y, Gd.y, Gu.y, e.y, h.y);
+  r.z = cell(x2, x3, Gl.z, Gh.z, Gd.z, Gu.z, e.z, h.z);
+  r.w = cell(x3, x4, Gl.w, Gh.w, Gd.w, Gu.w, e.w, h.w);
+  *reinterpret_cast<float4*>(E + c) = e;
+  return r;
+}
+
+// Factors of row j of layer k.  The y faces of the walls are 0; a stretched y
+// (YS) scales the x and z faces by s_j, the y faces below and above by t_j
+// and t_{j+1}, the cell's value by 1 / s_j.
+template <bool YS>
+__device__ __forceinline__ RowW row_factors(const Geo& g, int k, int j) {
+  const int nz1 = g.nz + 1, ny = g.ny;
+  RowW w;
+  w.x = 2.f * g.cw_f[k];
+  w.yl = (g.ywall && j == 0) ? 0.f : 2.f * g.cw_f[nz1 + k];
+  w.yh = (g.ywall && j + 1 == ny) ? 0.f : 2.f * g.cw_f[nz1 + k];
+  w.zd = 2.f * g.cw_f[2 * nz1 + k];
+  w.zu = 2.f * g.cw_f[2 * nz1 + k + 1];
+  w.iv = g.inv_dzf_f[k];
+  if constexpr (YS) {
+    const float sj = g.ym_f[j];
+    w.x *= sj;
+    w.zd *= sj;
+    w.zu *= sj;
+    w.yl *= g.ym_f[ny + j];
+    w.yh = (j + 1 < ny) ? w.yh * g.ym_f[ny + j + 1] : 0.f;
+    w.iv *= g.ym_f[2 * ny + j];
+  }
+  return w;
+}
+
+// Odd ny: the two rows of a sequence one after the other.
 template <bool YS>
 __device__ __forceinline__ void resid_update_vec4(const Geo& g, const Faces& fc, float* __restrict__ E,
-                                                  const float* __restrict__ delta, int scale_rho,
-                                                  bool const_scale, float rt_f, long row0, int rpb,
-                                                  float2* bufA, int seq_stride, float& s2, float& s1) {
-  // 32-bit cell offsets (grids keep nx ny (nz + 1) below 2^31); the block's
-  // first row is split into (layer, row in layer) once, the others step
-  // from it (no 64-bit division per cell group)
+                                                  const float* __restrict__ delta, bool scale, bool own, float rt_f,
+                                                  long row0, int rpb, float2* bufA, int seq_stride, float& s2,
+                                                  float& s1, int tid, int nth) {
+  // 32-bit cell offsets (grids keep nx ny (nz + 1) below 2^31); the first row
+  // is split into (layer, row in layer) once, the others step from it (no
+  // 64-bit division per cell group)
   const int nx = g.nx, ny = g.ny, nz = g.nz;
   const int nrows = nz * ny;
   const unsigned plane = (unsigned)nx * ny;
@@ -145,92 +229,27 @@ __device__ __forceinline__ void resid_update_vec4(const Geo& g, const Faces& fc,
   const int lg4 = ((t4 & (t4 - 1)) == 0) ? 31 - __clz(t4) : -1;
   const int r0 = (int)row0;
   const int k0 = r0 / ny, j0 = r0 - k0 * ny;
-  for (int w = threadIdx.x; w < npairs * t4; w += blockDim.x) {
+  for (int w = tid; w < npairs * t4; w += nth) {
     const int qp = lg4 >= 0 ? (w >> lg4) : w / t4;
     const int i = (w - qp * t4) << 2;
     float4 rr[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int row = r0 + 2 * qp + h;
-      float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+      rr[h] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (row < nrows) {
         int k = k0, j = j0 + 2 * qp + h;
         while (j >= ny) { j -= ny; ++k; }
         const int jp = (j + 1 == ny) ? 0 : j + 1, jm = (j == 0) ? ny - 1 : j - 1;
-        const unsigned rowoff = (unsigned)row * nx;
-        const unsigned kp = (unsigned)k * plane;
-        const unsigned c = rowoff + i;
+        const unsigned rowoff = (unsigned)row * nx, kp = (unsigned)k * plane, c = rowoff + i;
         const unsigned cyp = kp + (unsigned)jp * nx + i, cym = kp + (unsigned)jm * nx + i;
-        const int il = (i == 0) ? nx - 1 : i - 1, ir = (i + 4 == nx) ? 0 : i + 4;
-        const float4 d = ld4(delta + c);
-        const float dl = delta[rowoff + il], dr = delta[rowoff + ir];
-        const float4 dyp = ld4(delta + cyp), dym = ld4(delta + cym);
-        const bool up = k + 1 < nz, dn = k > 0;
-        float4 dzp = d, dzm = d;
-        if (up) dzp = ld4(delta + c + plane);
-        if (dn) dzm = ld4(delta + c - plane);
-        // FP32 face coefficients from the FP32 density of the cell and its
-        // six neighbours and the layer factors (z walls: factor 0; y walls:
-        // the wall faces of rows 0 and ny - 1 are 0)
-        const float4 rc = ld4(fc.rhof + c);
-        const float rl = fc.rhof[rowoff + il], rr = fc.rhof[rowoff + ir];
-        const float4 ryp = ld4(fc.rhof + cyp), rym = ld4(fc.rhof + cym);
-        float4 rzp = rc, rzm = rc;
-        if (up) rzp = ld4(fc.rhof + c + plane);
-        if (dn) rzm = ld4(fc.rhof + c - plane);
-        const int nz1 = nz + 1;
-        // stretched y: row factor s_j on the x and z faces, t_j and t_{j+1}
-        // on the y faces below and above, 1 / s_j on the cell's value
-        // (a separate instantiation: the uniform one keeps its registers)
-        float wx = g.cw_f[k];
-        float wyl = (g.ywall && j == 0) ? 0.f : g.cw_f[nz1 + k];
-        float wyh = (g.ywall && j + 1 == ny) ? 0.f : g.cw_f[nz1 + k];
-        float wzp = g.cw_f[2 * nz1 + k + 1], wzm = g.cw_f[2 * nz1 + k];
-        if constexpr (YS) {
-          const float sj = g.ym_f[j];
-          wx *= sj;
-          wzp *= sj;
-          wzm *= sj;
-          wyl *= g.ym_f[ny + j];
-          wyh = (j + 1 < ny) ? wyh * g.ym_f[ny + j + 1] : 0.f;
-        }
-        const float4 cx = make_float4(wx * face_beta_f(rl, rc.x), wx * face_beta_f(rc.x, rc.y),
-                                      wx * face_beta_f(rc.y, rc.z), wx * face_beta_f(rc.z, rc.w));
-        const float cxr = wx * face_beta_f(rc.w, rr);
-        const float4 cyp4 = make_float4(wyh * face_beta_f(rc.x, ryp.x), wyh * face_beta_f(rc.y, ryp.y),
-                                        wyh * face_beta_f(rc.z, ryp.z), wyh * face_beta_f(rc.w, ryp.w));
-        const float4 cym4 = make_float4(wyl * face_beta_f(rc.x, rym.x), wyl * face_beta_f(rc.y, rym.y),
-                                        wyl * face_beta_f(rc.z, rym.z), wyl * face_beta_f(rc.w, rym.w));
-        const float4 czp = make_float4(wzp * face_beta_f(rc.x, rzp.x), wzp * face_beta_f(rc.y, rzp.y),
-                                       wzp * face_beta_f(rc.z, rzp.z), wzp * face_beta_f(rc.w, rzp.w));
-        const float4 czm = make_float4(wzm * face_beta_f(rc.x, rzm.x), wzm * face_beta_f(rc.y, rzm.y),
-                                       wzm * face_beta_f(rc.z, rzm.z), wzm * face_beta_f(rc.w, rzm.w));
-        float4 e = ld4(E + c);
-        const float4 rh = scale_rho && !const_scale ? rc : make_float4(rt_f, rt_f, rt_f, rt_f);
-        float idzf = g.inv_dzf_f[k];
-        if constexpr (YS) idzf *= g.ym_f[2 * ny + j];
-        auto cell = [&](float dc, float dxm, float dxp, float cxm, float cxp, float dypv, float cypv,
-                        float dymv, float cymv, float dzpv, float czpv, float dzmv, float czmv, float& ev,
-                        float rhv) -> float {
-          float t = cxp * (dxp - dc);
-          t = fmaf(cxm, dxm - dc, t);
-          t = fmaf(cypv, dypv - dc, t);
-          t = fmaf(cymv, dymv - dc, t);
-          t = fmaf(czpv, dzpv - dc, t);
-          t = fmaf(czmv, dzmv - dc, t);
-          ev = ev - t;
-          const float ee = ev * idzf;
-          s2 = fmaf(ee, ee, s2);
-          s1 += fabsf(ee);
-          return scale_rho ? rhv * ee : ee;
-        };
-        r.x = cell(d.x, dl, d.y, cx.x, cx.y, dyp.x, cyp4.x, dym.x, cym4.x, dzp.x, czp.x, dzm.x, czm.x, e.x, rh.x);
-        r.y = cell(d.y, d.x, d.z, cx.y, cx.z, dyp.y, cyp4.y, dym.y, cym4.y, dzp.y, czp.y, dzm.y, czm.y, e.y, rh.y);
-        r.z = cell(d.z, d.y, d.w, cx.z, cx.w, dyp.z, cyp4.z, dym.z, cym4.z, dzp.z, czp.z, dzm.z, czm.z, e.z, rh.z);
-        r.w = cell(d.w, d.z, dr, cx.w, cxr, dyp.w, cyp4.w, dym.w, cym4.w, dzp.w, czp.w, dzm.w, czm.w, e.w, rh.w);
-        *reinterpret_cast<float4*>(E + c) = e;
+        const float4 d = ld4(delta + c), hc = ld4(fc.rhof + c);
+        const float4 Gl = half_flux4(ld4(delta + cym), d, ld4(fc.rhof + cym), hc);
+        const float4 Gh = half_flux4(d, ld4(delta + cyp), hc, ld4(fc.rhof + cyp));
+        rr[h] = resid_row4(row_factors<YS>(g, k, j), E, delta, fc.rhof, c, rowoff + (i == 0 ? nx - 1 : i - 1),
+                           rowoff + (i + 4 == nx ? 0 : i + 4), plane, k + 1 < nz, k > 0, d, hc, Gl, Gh, scale, own,
+                           rt_f, s2, s1);
       }
-      rr[h] = r;
     }
     float4* dst = reinterpret_cast<float4*>(bufA + qp * seq_stride + i);
     dst[0] = make_float4(rr[0].x, rr[1].x, rr[0].y, rr[1].y);
@@ -239,16 +258,15 @@ __device__ __forceinline__ void resid_update_vec4(const Geo& g, const Faces& fc,
 }
 
 // The same update with the two rows of a sequence taken together.  With ny
-// even, rows 2q and 2q + 1 of a block (its first row is even) lie in one
-// layer and are y neighbours of each other: the rows j - 1 .. j + 2 of delta
-// and of the density are loaded once each (four float4 loads fewer per
-// pair) and the face between the two rows is formed once (four reciprocals
-// fewer).  Same per-cell arithmetic as resid_update_vec4.
+// even, rows 2q and 2q + 1 (the first row is even) lie in one layer and are y
+// neighbours of each other: the rows j - 1 .. j + 2 of delta and of the
+// density are loaded once each and the face between the two rows is formed
+// once.
 template <bool YS>
 __device__ __forceinline__ void resid_update_pair4(const Geo& g, const Faces& fc, float* __restrict__ E,
-                                                   const float* __restrict__ delta, int scale_rho,
-                                                   bool const_scale, float rt_f, long row0, int rpb,
-                                                   float2* bufA, int seq_stride, float& s2, float& s1) {
+                                                   const float* __restrict__ delta, bool scale, bool own, float rt_f,
+                                                   long row0, int rpb, float2* bufA, int seq_stride, float& s2,
+                                                   float& s1, int tid, int nth) {
   const int nx = g.nx, ny = g.ny, nz = g.nz;
   const int nrows = nz * ny;
   const unsigned plane = (unsigned)nx * ny;
@@ -257,8 +275,7 @@ __device__ __forceinline__ void resid_update_pair4(const Geo& g, const Faces& fc
   const int lg4 = ((t4 & (t4 - 1)) == 0) ? 31 - __clz(t4) : -1;
   const int r0 = (int)row0;
   const int k0 = r0 / ny, j0 = r0 - k0 * ny;
-  const int nz1 = nz + 1;
-  for (int w = threadIdx.x; w < npairs * t4; w += blockDim.x) {
+  for (int w = tid; w < npairs * t4; w += nth) {
     const int qp = lg4 >= 0 ? (w >> lg4) : w / t4;
     const int i = (w - qp * t4) << 2;
     const int row = r0 + 2 * qp;  // row A; row B = row + 1, same layer
@@ -274,95 +291,87 @@ __device__ __forceinline__ void resid_update_pair4(const Geo& g, const Faces& fc
       const unsigned cm = kp + (unsigned)jm * nx + i, cp = kp + (unsigned)jpp * nx + i;
       const int il = (i == 0) ? nx - 1 : i - 1, ir = (i + 4 == nx) ? 0 : i + 4;
       const bool up = k + 1 < nz, dn = k > 0;
-      const bool own = scale_rho && !const_scale;
-      // layer factors; the y faces below A (face j), between A and B (face
-      // j + 1) and above B (face j + 2); walls in y zero the faces of rows
-      // 0 and ny - 1
-      float wxA = g.cw_f[k], wxB = wxA;
-      const float wy = g.cw_f[nz1 + k];
-      float wlo = (g.ywall && j == 0) ? 0.f : wy, wmid = wy, whi = (g.ywall && j + 2 == ny) ? 0.f : wy;
-      float wuA = g.cw_f[2 * nz1 + k + 1], wdA = g.cw_f[2 * nz1 + k], wuB = wuA, wdB = wdA;
-      float idA = g.inv_dzf_f[k], idB = idA;
-      if constexpr (YS) {
-        const float sA = g.ym_f[j], sB = g.ym_f[j + 1];
-        wxA *= sA; wuA *= sA; wdA *= sA;
-        wxB *= sB; wuB *= sB; wdB *= sB;
-        wlo *= g.ym_f[ny + j];
-        wmid *= g.ym_f[ny + j + 1];
-        whi = (j + 2 < ny) ? whi * g.ym_f[ny + j + 2] : 0.f;
-        idA *= g.ym_f[2 * ny + j];
-        idB *= g.ym_f[2 * ny + j + 1];
-      }
-      auto cell = [&](float dc, float dxm, float dxp, float cxm, float cxp, float dypv, float cypv,
-                      float dymv, float cymv, float dzpv, float czpv, float dzmv, float czmv, float& ev,
-                      float rhv, float idzf) -> float {
-        float t = cxp * (dxp - dc);
-        t = fmaf(cxm, dxm - dc, t);
-        t = fmaf(cypv, dypv - dc, t);
-        t = fmaf(cymv, dymv - dc, t);
-        t = fmaf(czpv, dzpv - dc, t);
-        t = fmaf(czmv, dzmv - dc, t);
-        ev = ev - t;
-        const float ee = ev * idzf;
-        s2 = fmaf(ee, ee, s2);
-        s1 += fabsf(ee);
-        return scale_rho ? (own ? rhv : rt_f) * ee : ee;
-      };
-      // the two centre rows (A's y+ neighbour is B, B's y- neighbour is A)
+      RowW wa = row_factors<YS>(g, k, j), wb = wa;
+      if constexpr (YS) wb = row_factors<YS>(g, k, j + 1);
+      else { wb.yl = wa.yh; wb.yh = (g.ywall && j + 2 == ny) ? 0.f : wa.yh; }
       const float4 dA = ld4(delta + ca), dB = ld4(delta + cb);
       const float4 hA = ld4(fc.rhof + ca), hB = ld4(fc.rhof + cb);
-      const float4 cym = make_float4(wmid * face_beta_f(hA.x, hB.x), wmid * face_beta_f(hA.y, hB.y),
-                                     wmid * face_beta_f(hA.z, hB.z), wmid * face_beta_f(hA.w, hB.w));
-      {  // row A: y- neighbour row j - 1 (face j)
-        const float4 dM = ld4(delta + cm), hM = ld4(fc.rhof + cm);
-        const float dAl = delta[oa + il], dAr = delta[oa + ir];
-        const float hAl = fc.rhof[oa + il], hAr = fc.rhof[oa + ir];
-        float4 dAu = dA, dAd = dA, hAu = hA, hAd = hA;
-        if (up) { dAu = ld4(delta + ca + plane); hAu = ld4(fc.rhof + ca + plane); }
-        if (dn) { dAd = ld4(delta + ca - plane); hAd = ld4(fc.rhof + ca - plane); }
-        float4 eA = ld4(E + ca);
-        const float4 cxA = make_float4(wxA * face_beta_f(hAl, hA.x), wxA * face_beta_f(hA.x, hA.y),
-                                       wxA * face_beta_f(hA.y, hA.z), wxA * face_beta_f(hA.z, hA.w));
-        const float cxAr = wxA * face_beta_f(hA.w, hAr);
-        const float4 cyl = make_float4(wlo * face_beta_f(hA.x, hM.x), wlo * face_beta_f(hA.y, hM.y),
-                                       wlo * face_beta_f(hA.z, hM.z), wlo * face_beta_f(hA.w, hM.w));
-        const float4 cuA = make_float4(wuA * face_beta_f(hA.x, hAu.x), wuA * face_beta_f(hA.y, hAu.y),
-                                       wuA * face_beta_f(hA.z, hAu.z), wuA * face_beta_f(hA.w, hAu.w));
-        const float4 cdA = make_float4(wdA * face_beta_f(hA.x, hAd.x), wdA * face_beta_f(hA.y, hAd.y),
-                                       wdA * face_beta_f(hA.z, hAd.z), wdA * face_beta_f(hA.w, hAd.w));
-        ra.x = cell(dA.x, dAl, dA.y, cxA.x, cxA.y, dB.x, cym.x, dM.x, cyl.x, dAu.x, cuA.x, dAd.x, cdA.x, eA.x, hA.x, idA);
-        ra.y = cell(dA.y, dA.x, dA.z, cxA.y, cxA.z, dB.y, cym.y, dM.y, cyl.y, dAu.y, cuA.y, dAd.y, cdA.y, eA.y, hA.y, idA);
-        ra.z = cell(dA.z, dA.y, dA.w, cxA.z, cxA.w, dB.z, cym.z, dM.z, cyl.z, dAu.z, cuA.z, dAd.z, cdA.z, eA.z, hA.z, idA);
-        ra.w = cell(dA.w, dA.z, dAr, cxA.w, cxAr, dB.w, cym.w, dM.w, cyl.w, dAu.w, cuA.w, dAd.w, cdA.w, eA.w, hA.w, idA);
-        *reinterpret_cast<float4*>(E + ca) = eA;
-      }
-      {  // row B: y+ neighbour row j + 2 (face j + 2)
-        const float4 dP = ld4(delta + cp), hP = ld4(fc.rhof + cp);
-        const float dBl = delta[ob + il], dBr = delta[ob + ir];
-        const float hBl = fc.rhof[ob + il], hBr = fc.rhof[ob + ir];
-        float4 dBu = dB, dBd = dB, hBu = hB, hBd = hB;
-        if (up) { dBu = ld4(delta + cb + plane); hBu = ld4(fc.rhof + cb + plane); }
-        if (dn) { dBd = ld4(delta + cb - plane); hBd = ld4(fc.rhof + cb - plane); }
-        float4 eB = ld4(E + cb);
-        const float4 cxB = make_float4(wxB * face_beta_f(hBl, hB.x), wxB * face_beta_f(hB.x, hB.y),
-                                       wxB * face_beta_f(hB.y, hB.z), wxB * face_beta_f(hB.z, hB.w));
-        const float cxBr = wxB * face_beta_f(hB.w, hBr);
-        const float4 cyh = make_float4(whi * face_beta_f(hB.x, hP.x), whi * face_beta_f(hB.y, hP.y),
-                                       whi * face_beta_f(hB.z, hP.z), whi * face_beta_f(hB.w, hP.w));
-        const float4 cuB = make_float4(wuB * face_beta_f(hB.x, hBu.x), wuB * face_beta_f(hB.y, hBu.y),
-                                       wuB * face_beta_f(hB.z, hBu.z), wuB * face_beta_f(hB.w, hBu.w));
-        const float4 cdB = make_float4(wdB * face_beta_f(hB.x, hBd.x), wdB * face_beta_f(hB.y, hBd.y),
-                                       wdB * face_beta_f(hB.z, hBd.z), wdB * face_beta_f(hB.w, hBd.w));
-        rb.x = cell(dB.x, dBl, dB.y, cxB.x, cxB.y, dP.x, cyh.x, dA.x, cym.x, dBu.x, cuB.x, dBd.x, cdB.x, eB.x, hB.x, idB);
-        rb.y = cell(dB.y, dB.x, dB.z, cxB.y, cxB.z, dP.y, cyh.y, dA.y, cym.y, dBu.y, cuB.y, dBd.y, cdB.y, eB.y, hB.y, idB);
-        rb.z = cell(dB.z, dB.y, dB.w, cxB.z, cxB.w, dP.z, cyh.z, dA.z, cym.z, dBu.z, cuB.z, dBd.z, cdB.z, eB.z, hB.z, idB);
-        rb.w = cell(dB.w, dB.z, dBr, cxB.w, cxBr, dP.w, cyh.w, dA.w, cym.w, dBu.w, cuB.w, dBd.w, cdB.w, eB.w, hB.w, idB);
-        *reinterpret_cast<float4*>(E + cb) = eB;
-      }
+      const float4 Gm = half_flux4(dA, dB, hA, hB);
+      const float4 Gl = half_flux4(ld4(delta + cm), dA, ld4(fc.rhof + cm), hA);
+      ra = resid_row4(wa, E, delta, fc.rhof, ca, oa + il, oa + ir, plane, up, dn, dA, hA, Gl, Gm, scale, own, rt_f,
+                      s2, s1);
+      const float4 Gh = half_flux4(dB, ld4(delta + cp), hB, ld4(fc.rhof + cp));
+      rb = resid_row4(wb, E, delta, fc.rhof, cb, ob + il, ob + ir, plane, up, dn, dB, hB, Gm, Gh, scale, own, rt_f,
+                      s2, s1);
     }
     float4* dst = reinterpret_cast<float4*>(bufA + qp * seq_stride + i);
     dst[0] = make_float4(ra.x, rb.x, ra.y, rb.y);
     dst[1] = make_float4(ra.z, rb.z, ra.w, rb.w);
+  }
+}
+
+// FP64 residual with the two rows of a sequence taken together (ny even: rows
+// 2q and 2q + 1 are y neighbours in one layer): the y neighbours and the y
+// coefficients between them are loaded once, and a thread has 23 loads in
+// flight for two cells.  Per cell: seven FMAs, then the scaling and the norms.
+template <bool YS>
+__device__ __forceinline__ void resid_exact_pair(const Geo& g, const Faces& fc, const double* __restrict__ b,
+                                                 const double* __restrict__ rho, const double* __restrict__ p,
+                                                 bool scale, bool const_scale, double rt, long row0, int rpb,
+                                                 double2* bufA, int seq_stride, double& s2, double& s1, int tid,
+                                                 int nth) {
+  const int nx = g.nx, ny = g.ny, nz = g.nz;
+  const int nrows = nz * ny;
+  const unsigned plane = (unsigned)nx * ny;
+  const int npairs = rpb >> 1;
+  const int r0 = (int)row0;
+  const int k0 = r0 / ny, j0 = r0 - k0 * ny;
+  const int tpr = nx < nth ? nx : nth, par = nth / tpr;
+  const int q0 = tid / tpr, i0 = tid - q0 * tpr;
+  for (int q = q0; q < npairs && q0 < par; q += par) {
+    const int row = r0 + 2 * q;
+    if (row >= nrows) {
+      for (int i = i0; i < nx; i += tpr) bufA[(size_t)q * seq_stride + i] = make_double2(0.0, 0.0);
+      continue;
+    }
+    int k = k0, j = j0 + 2 * q;
+    while (j >= ny) { j -= ny; ++k; }
+    const unsigned kp = (unsigned)k * plane;
+    const unsigned oa = (unsigned)row * nx, ob = oa + nx;
+    const unsigned om = kp + (unsigned)(j == 0 ? ny - 1 : j - 1) * nx, op = kp + (unsigned)(j + 2 == ny ? 0 : j + 2) * nx;
+    const bool up = k + 1 < nz, dn = k > 0;
+    const double iva = g.inv_dzf[k] * (YS ? g.ym[2 * ny + j] : 1.0), ivb = YS ? g.inv_dzf[k] * g.ym[2 * ny + j + 1] : iva;
+    for (int i = i0; i < nx; i += tpr) {
+      const int ip = (i + 1 == nx) ? 0 : i + 1, im = (i == 0) ? nx - 1 : i - 1;
+      const unsigned ca = oa + i, cb = ob + i;
+      const double pa = p[ca], pb = p[cb], pm = p[om + i], pp = p[op + i];
+      const double pal = p[oa + im], par_ = p[oa + ip], pbl = p[ob + im], pbr = p[ob + ip];
+      const double xa = fc.cx[ca], xar = fc.cx[oa + ip], xb = fc.cx[cb], xbr = fc.cx[ob + ip];
+      const double ya = fc.cy[ca], yb = fc.cy[cb], yp = fc.cy[op + i];
+      const double za = fc.cz[ca], zau = fc.cz[ca + plane], zb = fc.cz[cb], zbu = fc.cz[cb + plane];
+      double pau = 0.0, pbu = 0.0, pad = 0.0, pbd = 0.0;  // the wall faces' coefficients are 0
+      if (up) { pau = p[ca + plane]; pbu = p[cb + plane]; }
+      if (dn) { pad = p[ca - plane]; pbd = p[cb - plane]; }
+      double ea = fma(fc.diag[ca], pa, b[ca]), eb = fma(fc.diag[cb], pb, b[cb]);
+      const double ha = scale ? (const_scale ? rt : rho[ca]) : 1.0, hb = scale ? (const_scale ? rt : rho[cb]) : 1.0;
+      ea = fma(-xar, par_, ea);
+      eb = fma(-xbr, pbr, eb);
+      ea = fma(-xa, pal, ea);
+      eb = fma(-xb, pbl, eb);
+      ea = fma(-yb, pb, ea);
+      eb = fma(-yp, pp, eb);
+      ea = fma(-ya, pm, ea);
+      eb = fma(-yb, pa, eb);
+      if (up) { ea = fma(-zau, pau, ea); eb = fma(-zbu, pbu, eb); }
+      if (dn) { ea = fma(-za, pad, ea); eb = fma(-zb, pbd, eb); }
+      ea *= iva;
+      eb *= ivb;
+      s2 = fma(ea, ea, s2);
+      s1 += fabs(ea);
+      s2 = fma(eb, eb, s2);
+      s1 += fabs(eb);
+      bufA[(size_t)q * seq_stride + i] = make_double2(scale ? ha * ea : ea, scale ? hb * eb : eb);
+    }
   }
 }
 
@@ -381,13 +390,14 @@ __device__ __forceinline__ void resid_update_pair4(const Geo& g, const Faces& fc
 // The rows [row0, row0 + rpb) of the residual (the first step of the stage
 // below) into bufA: complex sequence q = (row - row0) / 2 at element offset
 // q * seq_stride (re = even row, im = odd row); s2, s1 accumulate e^2 and
-// |e| of the thread's cells.  Every thread of the block calls it.
+// |e| of the thread's cells.  Called by nth threads (a block, or a warp), tid
+// their index.
 template <typename T, bool YS>
 __device__ __forceinline__ void resid_rows(const Geo& g, const Faces& fc, const double* __restrict__ b,
                                            const double* __restrict__ rho, const double* __restrict__ p, int mode,
                                            int p_zero, int scale_rho, long row0, int rpb, bool need_exact,
                                            float* __restrict__ E, const float* __restrict__ delta, C2<T>* bufA,
-                                           int seq_stride, T& s2, T& s1) {
+                                           int seq_stride, T& s2, T& s1, int tid, int nth) {
   const int nx = g.nx, ny = g.ny, nz = g.nz;
   const bool update = (E != nullptr) && !p_zero && !need_exact;
   const int nrows = nz * ny;
@@ -397,20 +407,27 @@ __device__ __forceinline__ void resid_rows(const Geo& g, const Faces& fc, const 
   const double rt = (const_scale && mode != 0) ? *fc.rho_tilde : 0.0;
   const float rt_f = (float)rt;
   // thread -> (row offset, first column); index math is done once per row
-  const int tpr = nx < (int)blockDim.x ? nx : (int)blockDim.x;
-  const int rows_par = blockDim.x / tpr;
-  const int qoff = threadIdx.x / tpr, i0 = threadIdx.x - qoff * tpr;
-  const bool vec = update && sizeof(T) == sizeof(float) && (nx & 3) == 0;
+  const int tpr = nx < nth ? nx : nth;
+  const int rows_par = nth / tpr;
+  const int qoff = tid / tpr, i0 = tid - qoff * tpr;
+  bool vec = update && sizeof(T) == sizeof(float) && (nx & 3) == 0;
   if (vec) {
     float a2 = 0.f, a1 = 0.f;
     if ((ny & 1) == 0)  // the two rows of a sequence share a layer
-      resid_update_pair4<YS>(g, fc, E, delta, scale_rho, const_scale, rt_f, row0, rpb,
-                             reinterpret_cast<float2*>(bufA), seq_stride, a2, a1);
+      resid_update_pair4<YS>(g, fc, E, delta, scale_rho != 0, !const_scale, rt_f, row0, rpb,
+                             reinterpret_cast<float2*>(bufA), seq_stride, a2, a1, tid, nth);
     else
-      resid_update_vec4<YS>(g, fc, E, delta, scale_rho, const_scale, rt_f, row0, rpb,
-                            reinterpret_cast<float2*>(bufA), seq_stride, a2, a1);
+      resid_update_vec4<YS>(g, fc, E, delta, scale_rho != 0, !const_scale, rt_f, row0, rpb,
+                            reinterpret_cast<float2*>(bufA), seq_stride, a2, a1, tid, nth);
     s2 += (T)a2;
     s1 += (T)a1;
+  }
+  if constexpr (sizeof(T) == sizeof(double)) {
+    if (mode != 0 && !p_zero && (ny & 1) == 0) {
+      resid_exact_pair<YS>(g, fc, b, rho, p, scale_rho != 0, const_scale, rt, row0, rpb,
+                           reinterpret_cast<double2*>(bufA), seq_stride, s2, s1, tid, nth);
+      vec = true;
+    }
   }
   for (int q = qoff; !vec && q < rpb && qoff < rows_par; q += rows_par) {
     const int row = (int)row0 + q;
@@ -459,15 +476,14 @@ __device__ __forceinline__ void resid_rows(const Geo& g, const Faces& fc, const 
             E[c] = ev;
           } else {
             ep = b[c];
-            if (!p_zero) {
-              double t = -fc.diag[c] * p[c];
-              t = fma(fc.cx[rowoff + ip], p[rowoff + ip], t);
-              t = fma(fc.cx[c], p[rowoff + im], t);
-              t = fma(fc.cy[rowp + i], p[rowp + i], t);
-              t = fma(fc.cy[c], p[rowm + i], t);
-              if (k + 1 < nz) t = fma(fc.cz[c + plane], p[c + plane], t);
-              if (k > 0) t = fma(fc.cz[c], p[c - plane], t);
-              ep -= t;
+            if (!p_zero) {  // b - (sum_nb c_nb p_nb - diag p_c), seven FMAs
+              ep = fma(fc.diag[c], p[c], ep);
+              ep = fma(-fc.cx[rowoff + ip], p[rowoff + ip], ep);
+              ep = fma(-fc.cx[c], p[rowoff + im], ep);
+              ep = fma(-fc.cy[rowp + i], p[rowp + i], ep);
+              ep = fma(-fc.cy[c], p[rowm + i], ep);
+              if (k + 1 < nz) ep = fma(-fc.cz[c + plane], p[c + plane], ep);
+              if (k > 0) ep = fma(-fc.cz[c], p[c - plane], ep);
             }
             if (sizeof(T) == sizeof(float)) {
               ev = narrow_f64(ep);
@@ -520,7 +536,8 @@ __device__ __forceinline__ void stage_resid_fftx(const Geo& g, const Faces& fc, 
   if constexpr (F32) {
     if (fast) load_twiddles_smem(twx, nx, twb);
   }
-  resid_rows<T, YS>(g, fc, b, rho, p, mode, p_zero, scale_rho, row0, rpb, need_exact, E, delta, bufA, nx, s2, s1);
+  resid_rows<T, YS>(g, fc, b, rho, p, mode, p_zero, scale_rho, row0, rpb, need_exact, E, delta, bufA, nx, s2, s1,
+                    threadIdx.x, blockDim.x);
   if (mode != 0) {
     // block partial sums of e^2 and |e|: in the arithmetic's own precision
     // (FP32 shuffles on mixed plans: the FP64 pipe is the scarce one)
@@ -545,10 +562,11 @@ __device__ __forceinline__ void stage_resid_fftx(const Geo& g, const Faces& fc, 
     const C2<T> Z = res[(size_t)q * nx + kx];
     const int km = (kx == 0) ? 0 : nx - kx;
     const C2<T> W = res[(size_t)q * nx + km];
-    // A = (Z + conj W)/2, B = (Z - conj W)/(2i)
+    // 2 A = Z + conj W, 2 B = (Z - conj W)/i: the spectra are kept doubled,
+    // the scale of the inverse x transform halves them (kSpecScale)
     C2<T> A, B;
-    A.x = (T)0.5 * (Z.x + W.x); A.y = (T)0.5 * (Z.y - W.y);
-    B.x = (T)0.5 * (Z.y + W.y); B.y = (T)-0.5 * (Z.x - W.x);
+    A.x = Z.x + W.x; A.y = Z.y - W.y;
+    B.x = Z.y + W.y; B.y = W.x - Z.x;
     const long ra = row0 + 2 * q;
     if (ra < nrows) spec[(size_t)ra * nxh + kx] = A;
     if (ra + 1 < nrows) spec[(size_t)(ra + 1) * nxh + kx] = B;
