@@ -22,7 +22,7 @@ const char* const kNames[K_COUNT] = {
     "prep_faces", "mean_S", "rhs_b", "remove_mean", "correct", "mixture_density", "adj_rhs",
     "adj_finish", "adj_grho", "rho_tilde", "fold_pending", "p0_rate", "divergence_source", "predictor",
     "zdct_fwd", "zdct_inv"};
-const int kLaunches[K_COUNT] = {1, 1, 1, 1, 1, 1, 1, 2, 2, 2, 3, 1, 1, 1, 1, 1, 2, 1, 2, 1, 2, 1, 1};
+const int kLaunches[K_COUNT] = {1, 1, 1, 1, 1, 1, 1, 2, 2, 2, 3, 1, 1, 1, 1, 1, 2, 1, 2, 1, 1, 1, 1};
 struct Rec { int kid; cudaEvent_t a, b; };
 struct Prof {
   bool on = false;
@@ -47,7 +47,8 @@ struct pp_plan_s {
   double *d_inv_dzf = nullptr, *d_inv_dzc = nullptr, *d_dzf = nullptr, *d_za = nullptr, *d_zc = nullptr;
   double *d_lamx = nullptr, *d_lamy = nullptr, *d_invd = nullptr, *d_mtab = nullptr;
   float* d_inv_dzf_f = nullptr;
-  float* d_cw_f = nullptr;  // [3][nz + 1] FP32 layer factors of the face coefficients
+  float* d_cw_f = nullptr;   // [3][nz + 1] FP32 layer factors of the face coefficients
+  double* d_cw_d = nullptr;  // the same in FP64, doubled (Geo::cw_d)
   void *d_twx = nullptr, *d_twy = nullptr;
   void* d_dcty = nullptr;  // walls in y: exp(-i pi m / (2 ny)), m < ny (C2 of the plan's FFT type)
   // stretched y between walls: row factors (Geo::ym, ym_f) and the transposed
@@ -442,7 +443,7 @@ void free_plan(pp_plan_s* P) {
   if (!P) return;
   double* dptrs[] = {P->d_inv_dzf, P->d_inv_dzc, P->d_dzf, P->d_za, P->d_zc, P->d_lamx, P->d_lamy,
                      P->d_invd, P->d_mtab, P->d_b, P->d_red, P->faces.cx, P->faces.cy, P->faces.cz,
-                     P->faces.diag, P->d_rho_tilde, P->d_delta64, P->d_thermo};
+                     P->faces.diag, P->d_rho_tilde, P->d_delta64, P->d_thermo, P->d_cw_d};
   if (P->faces.rhof) cudaFree(P->faces.rhof);
   if (P->d_low) cudaFree(P->d_low);
   float* fptrs[] = {P->faces.diagf, P->d_delta, P->d_sdelta, P->d_mtab_f, P->d_invd_f, P->d_zc_f,
@@ -612,6 +613,11 @@ pp_status pressure_plan_create(const pp_grid* grid, pp_precision prec, void* str
     free_plan(P);
     return st;
   }
+  if ((st = up(&P->d_cw_d, layer_factors_f64(nz, dzf, inv_dzc, 1.0 / (P->dx * P->dx), 1.0 / (P->dy * P->dy)))) !=
+      PP_OK) {
+    free_plan(P);
+    return st;
+  }
   if (ystretch) {
     std::vector<float> ymf(ymet.begin(), ymet.end());
     const int ny = G.ny;
@@ -729,7 +735,10 @@ pp_status pressure_plan_create(const pp_grid* grid, pp_precision prec, void* str
   g.nx = G.nx; g.ny = G.ny; g.nz = nz; g.nxh = P->nxh;
   g.inv_dzf_f = P->d_inv_dzf_f;
   g.cw_f = P->d_cw_f;
+  g.cw_d = P->d_cw_d;
   g.dx = P->dx; g.dy = P->dy;
+  g.inv_dx = 1.0 / g.dx;
+  g.inv_dy = 1.0 / g.dy;
   g.inv_dx2 = 1.0 / (P->dx * P->dx);
   g.inv_dy2 = 1.0 / (P->dy * P->dy);
   g.inv_dzf = P->d_inv_dzf; g.inv_dzc = P->d_inv_dzc; g.dzf = P->d_dzf;
@@ -922,9 +931,7 @@ pp_status pressure_predictor(pp_plan P, const double* u, const double* v, const 
     if (q != nullptr && !is_device_ptr(q)) return PP_ERR_INVALID_ARG;
   const double r = ab2 ? dt_new / dt_old : 0.0;
   const double a = ab2 ? 1.0 + 0.5 * r : 1.0, b = ab2 ? 0.5 * r : 0.0;
-  // the cell divergence goes to the plan's right-hand-side workspace (free
-  // between projections)
-  PP_K(P, K_PRED, launch_predictor(P->geo, u, v, w, rho, mu, f, prev, gravity, dt_new, a, b, P->d_b, u_star, ru,
+  PP_K(P, K_PRED, launch_predictor(P->geo, u, v, w, rho, mu, f, prev, gravity, dt_new, a, b, u_star, ru,
                                    P->stream));
   return PP_OK;
 }

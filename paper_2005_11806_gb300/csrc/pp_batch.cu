@@ -61,10 +61,10 @@ __global__ void kb_weighted_partial(GridDev* G, const int2* __restrict__ work, i
   const int2 w = work[blockIdx.x];
   const GridDev& d = G[w.x];
   const double* f = use_p ? d.p : d.S;
-  const size_t plane = (size_t)d.g.nx * d.g.ny;
   double s = 0.0;
   if (f != nullptr) {
-    PP_CHUNK_LOOP(d, w) s += d.g.dzf[c / plane] * f[c];
+    const unsigned plane = (unsigned)d.g.nx * (unsigned)d.g.ny;
+    PP_CHUNK_LOOP(d, w) s += d.g.dzf[(unsigned)c / plane] * f[c];
   }
   s = block_sum<double>(s, sh);
   if (threadIdx.x == 0) d.red[w.y] = s;
@@ -495,7 +495,7 @@ pp_status pressure_batch_create(const pp_grid* grids, int ngrids, pp_precision p
   // pool layout: per grid, every buffer and table
   struct Off {
     size_t spec, E, delta, sdelta, b, red, st, cx, cy, cz, diag, rhof, invd, mtab,
-        twx, twy, dcty, idzf, idzc, dzf, za, zc, idzff, cwf, lamx, lamy, mtabf, invdf, zcf;
+        twx, twy, dcty, idzf, idzc, dzf, za, zc, idzff, cwf, cwd, lamx, lamy, mtabf, invdf, zcf;
   };
   std::vector<Off> off(ngrids);
   Carve cv;
@@ -523,7 +523,7 @@ pp_status pressure_batch_create(const pp_grid* grids, int ngrids, pp_precision p
     o.dcty = cv.take((size_t)G.ny * sizeof(float2));
     o.idzf = cv.take((size_t)G.nz * 8); o.idzc = cv.take((size_t)(G.nz + 1) * 8); o.dzf = cv.take((size_t)G.nz * 8);
     o.za = cv.take((size_t)G.nz * 8); o.zc = cv.take((size_t)G.nz * 8); o.idzff = cv.take((size_t)G.nz * 4);
-    o.cwf = cv.take(3 * (size_t)(G.nz + 1) * 4);
+    o.cwf = cv.take(3 * (size_t)(G.nz + 1) * 4); o.cwd = cv.take(3 * (size_t)(G.nz + 1) * 8);
     o.lamx = cv.take((size_t)(G.nx / 2 + 1) * 8); o.lamy = cv.take((size_t)G.ny * 8);
     o.mtabf = cv.take(nsp * 4); o.invdf = cv.take(nsp * 4); o.zcf = cv.take((size_t)G.nz * 4);
   }
@@ -570,6 +570,7 @@ pp_status pressure_batch_create(const pp_grid* grids, int ngrids, pp_precision p
     for (int m = 0; m < ny; ++m)
       dcty[m] = make_float2((float)std::cos(pi * m / (2.0 * ny)), (float)(-std::sin(pi * m / (2.0 * ny))));
     const std::vector<float> cwf = layer_factors_f32(nz, dzf, idzc, 1.0 / (dx * dx), 1.0 / (dy * dy));
+    const std::vector<double> cwd = layer_factors_f64(nz, dzf, idzc, 1.0 / (dx * dx), 1.0 / (dy * dy));
     std::vector<float2> twx(nx), twy(ny);
     for (int m = 0; m < nx; ++m) twx[m] = make_float2((float)std::cos(two_pi * m / nx), (float)std::sin(two_pi * m / nx));
     for (int m = 0; m < ny; ++m) twy[m] = make_float2((float)std::cos(two_pi * m / ny), (float)std::sin(two_pi * m / ny));
@@ -579,15 +580,16 @@ pp_status pressure_batch_create(const pp_grid* grids, int ngrids, pp_precision p
         {o.idzc, idzc.data(), idzc.size() * 8}, {o.za, za.data(), za.size() * 8}, {o.zc, zc.data(), zc.size() * 8},
         {o.idzff, idzff.data(), idzff.size() * 4}, {o.lamx, lamx.data(), lamx.size() * 8},
         {o.lamy, lamy.data(), lamy.size() * 8}, {o.zcf, zcf.data(), zcf.size() * 4},
-        {o.cwf, cwf.data(), cwf.size() * 4}, {o.dcty, dcty.data(), dcty.size() * sizeof(float2)}};
+        {o.cwf, cwf.data(), cwf.size() * 4}, {o.cwd, cwd.data(), cwd.size() * 8}, {o.dcty, dcty.data(), dcty.size() * sizeof(float2)}};
     for (const Up& u : ups)
       if (cudaMemcpy(P + u.off, u.src, u.bytes, cudaMemcpyHostToDevice) != cudaSuccess) { free_batch(B); return PP_ERR_CUDA; }
     Geo& g = d.g;
     g.nx = nx; g.ny = ny; g.nz = nz; g.nxh = nxh; g.dx = dx; g.dy = dy;
+    g.inv_dx = 1.0 / dx; g.inv_dy = 1.0 / dy;
     g.inv_dx2 = 1.0 / (dx * dx); g.inv_dy2 = 1.0 / (dy * dy);
     g.inv_dzf = (const double*)(P + o.idzf); g.inv_dzc = (const double*)(P + o.idzc);
     g.dzf = (const double*)(P + o.dzf); g.za = (const double*)(P + o.za); g.zc = (const double*)(P + o.zc);
-    g.inv_dzf_f = (const float*)(P + o.idzff); g.cw_f = (const float*)(P + o.cwf); g.lz = zf[nz] - zf[0];
+    g.inv_dzf_f = (const float*)(P + o.idzff); g.cw_f = (const float*)(P + o.cwf); g.cw_d = (const double*)(P + o.cwd); g.lz = zf[nz] - zf[0];
     g.ywall = ywall ? 1 : 0;
     g.ym = nullptr;
     g.ym_f = nullptr;

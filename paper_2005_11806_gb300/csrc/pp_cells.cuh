@@ -7,20 +7,22 @@ namespace pp {
 
 struct CellIdx {
   int i, j, k;
-  size_t cim, cip, cjm, cjp;
+  unsigned cim, cip, cjm, cjp;  // grids keep nx ny (nz + 1) below 2^31
 };
 
-__device__ __forceinline__ CellIdx cell_index(const Geo& g, size_t c) {
-  const int nx = g.nx, ny = g.ny;
-  const size_t plane = (size_t)nx * ny;
+// 32-bit divisions: three 64-bit ones cost more than the FP64 work of some of
+// the bodies below.
+__device__ __forceinline__ CellIdx cell_index(const Geo& g, size_t c64) {
+  const unsigned nx = (unsigned)g.nx, ny = (unsigned)g.ny, c = (unsigned)c64;
   CellIdx x;
-  x.i = (int)(c % nx);
-  x.j = (int)((c / nx) % ny);
-  x.k = (int)(c / plane);
-  x.cim = c - x.i + (x.i == 0 ? nx - 1 : x.i - 1);
-  x.cip = c - x.i + (x.i + 1 == nx ? 0 : x.i + 1);
-  x.cjm = c - (size_t)x.j * nx + (size_t)(x.j == 0 ? ny - 1 : x.j - 1) * nx;
-  x.cjp = c - (size_t)x.j * nx + (size_t)(x.j + 1 == ny ? 0 : x.j + 1) * nx;
+  const unsigned row = c / nx, i = c - row * nx, k = row / ny, j = row - k * ny;
+  x.i = (int)i;
+  x.j = (int)j;
+  x.k = (int)k;
+  x.cim = i == 0 ? c + nx - 1 : c - 1;
+  x.cip = i + 1 == nx ? c + 1 - nx : c + 1;
+  x.cjm = j == 0 ? c + (ny - 1) * nx : c - nx;
+  x.cjp = j + 1 == ny ? c - (ny - 1) * nx : c + nx;
   return x;
 }
 
@@ -28,18 +30,24 @@ __device__ __forceinline__ CellIdx cell_index(const Geo& g, size_t c) {
 // z-face "below", x/y coefficients scaled by the layer width dzf_k).  Wall
 // faces get 0: the z walls, and with walls in y the y-face below row 0,
 // which the periodic indexing also reaches as the face above row ny - 1.
+// FP64-pipe bound: five operations a face (512^3: prep_faces and prep_diag
+// together 9.4 -> 5.2 ms, most of it the IEEE divisions and 64-bit index divisions).
 __device__ __forceinline__ void cell_prep_faces(const Geo& g, const double* __restrict__ rho,
                                                 const Faces& fc, size_t c) {
   const CellIdx x = cell_index(g, c);
   const size_t plane = (size_t)g.nx * g.ny;
   const double r = rho[c];
-  const double w = g.dzf[x.k];
-  // stretched y: the row of cell j is scaled by dzf_k s_j; the y face below
-  // it carries t_j = dy / dyc_j
-  const double sj = g.ym ? g.ym[x.j] : 1.0, tj = g.ym ? g.ym[g.ny + x.j] : 1.0;
-  fc.cx[c] = 2.0 / (r + rho[x.cim]) * g.inv_dx2 * w * sj;
-  fc.cy[c] = (g.ywall && x.j == 0) ? 0.0 : 2.0 / (r + rho[x.cjm]) * g.inv_dy2 * w * tj;
-  fc.cz[c] = (x.k == 0) ? 0.0 : 2.0 / (r + rho[c - plane]) * g.inv_dzc[x.k] * sj;
+  // layer factors 2 dzf / dx^2, 2 dzf / dy^2, 2 / dzc (0 on the walls); a product
+  // of uniform factors costs as much of the FP64 pipe as one of the cell's own
+  double fx = g.cw_d[x.k], fy = g.cw_d[g.nz + 1 + x.k], fz = g.cw_d[2 * (g.nz + 1) + x.k];
+  if (g.ym) {  // stretched y: the row of cell j is scaled by dzf_k s_j; the y face below it carries t_j = dy / dyc_j
+    fx *= g.ym[x.j];
+    fy *= g.ym[g.ny + x.j];
+    fz *= g.ym[x.j];
+  }
+  fc.cx[c] = fx * rcp_f64(r + rho[x.cim]);
+  fc.cy[c] = (g.ywall && x.j == 0) ? 0.0 : fy * rcp_f64(r + rho[x.cjm]);
+  fc.cz[c] = (x.k == 0) ? 0.0 : fz * rcp_f64(r + rho[c - plane]);
   if (x.k == g.nz - 1) fc.cz[c + plane] = 0.0;
   fc.rhof[c] = (float)r;
 }
@@ -67,35 +75,41 @@ __device__ __forceinline__ double cell_rhs_b(const Geo& g, const double* __restr
   const double whi = (x.k == g.nz - 1) ? 0.0 : ws[c + plane];
   const double vlo = (g.ywall && x.j == 0) ? 0.0 : vs[c];
   const double vhi = (g.ywall && x.j == g.ny - 1) ? 0.0 : vs[x.cjp];
-  const double sj = g.ym ? g.ym[x.j] : 1.0;
-  double d = (us[x.cip] - us[c]) / g.dx + (vhi - vlo) / (g.dy * sj) + (whi - wlo) * g.inv_dzf[x.k];
+  double dv = vhi - vlo, wd = g.dzf[x.k] * inv_dt;
+  if (g.ym) {
+    dv *= g.ym[2 * g.ny + x.j];
+    wd *= g.ym[x.j];
+  }
+  double d = fma(us[x.cip] - us[c], g.inv_dx, fma(dv, g.inv_dy, (whi - wlo) * g.inv_dzf[x.k]));
   if (S != nullptr) d -= (S[c] - meanS);
-  b[c] = d * g.dzf[x.k] * sj * inv_dt;
+  b[c] = d * wd;
   return d;
 }
 
-// div(k grad T) at cell c: D(k_f G T) with k_f the arithmetic mean of the
+// 2 div(k grad T) at cell c: D(k_f G T) with k_f the arithmetic mean of the
 // two cells of a face, no flux through the z walls, nor through the y walls
 // when y is bounded (Eqs. 30 and 34).
-__device__ __forceinline__ double cell_conduction(const Geo& g, const double* __restrict__ kc,
-                                                  const double* __restrict__ T, size_t c) {
+__device__ __forceinline__ double cell_conduction2(const Geo& g, const double* __restrict__ kc,
+                                                   const double* __restrict__ T, size_t c) {
   const CellIdx x = cell_index(g, c);
   const size_t plane = (size_t)g.nx * g.ny;
   const double k0 = kc[c], t0 = T[c];
-  double sx = 0.5 * (k0 + kc[x.cip]) * (T[x.cip] - t0) + 0.5 * (k0 + kc[x.cim]) * (T[x.cim] - t0);
+  const double sx = fma(k0 + kc[x.cip], T[x.cip] - t0, (k0 + kc[x.cim]) * (T[x.cim] - t0));
   // with walls in y no heat crosses the faces below row 0 and above row ny - 1
   const bool yhi = !(g.ywall && x.j + 1 == g.ny), ylo = !(g.ywall && x.j == 0);
   // stretched y: the face below row j is dyc_j = dy / t_j from the centre
   // below, and the row is dyf_j = s_j dy wide
-  const double thi = (g.ym && yhi) ? g.ym[g.ny + x.j + 1] : 1.0, tlo = g.ym ? g.ym[g.ny + x.j] : 1.0;
-  const double isj = g.ym ? g.ym[2 * g.ny + x.j] : 1.0;
-  double sy = (yhi ? 0.5 * (k0 + kc[x.cjp]) * (T[x.cjp] - t0) * thi : 0.0) +
-              (ylo ? 0.5 * (k0 + kc[x.cjm]) * (T[x.cjm] - t0) * tlo : 0.0);
-  sy *= isj;
+  double fhi = yhi ? T[x.cjp] - t0 : 0.0, flo = ylo ? T[x.cjm] - t0 : 0.0;
+  if (g.ym) {
+    const double isj = g.ym[2 * g.ny + x.j];
+    fhi *= yhi ? g.ym[g.ny + x.j + 1] * isj : 0.0;
+    flo *= g.ym[g.ny + x.j] * isj;
+  }
+  const double sy = fma(k0 + kc[x.cjp], fhi, (k0 + kc[x.cjm]) * flo);
   double sz = 0.0;
-  if (x.k + 1 < g.nz) sz += 0.5 * (k0 + kc[c + plane]) * (T[c + plane] - t0) * g.inv_dzc[x.k + 1];
-  if (x.k > 0) sz += 0.5 * (k0 + kc[c - plane]) * (T[c - plane] - t0) * g.inv_dzc[x.k];
-  return sx * g.inv_dx2 + sy * g.inv_dy2 + sz * g.inv_dzf[x.k];
+  if (x.k + 1 < g.nz) sz = (k0 + kc[c + plane]) * ((T[c + plane] - t0) * g.inv_dzc[x.k + 1]);
+  if (x.k > 0) sz = fma(k0 + kc[c - plane], (T[c - plane] - t0) * g.inv_dzc[x.k], sz);
+  return fma(sx, g.inv_dx2, fma(sy, g.inv_dy2, sz * g.inv_dzf[x.k]));
 }
 
 // u = u* - dt beta G p at the faces of cell c (Eq. corr); w walls = 0, and
@@ -113,11 +127,17 @@ __device__ __forceinline__ void cell_correct(const Geo& g, const Faces& fc,
   // dt beta_x / dx = dt dx cx / dzf_k (cx carries dzf_k); on a stretched y
   // cx and cz also carry s_j, and dt beta_y / dyc_j = dt dy cy / dzf_k
   // (cy carries dzf_k t_j = dzf_k dy / dyc_j)
-  const double is = g.ym ? g.ym[2 * g.ny + x.j] : 1.0;
-  const double ax = dt * g.dx * g.inv_dzf[x.k] * is, ay = dt * g.dy * g.inv_dzf[x.k];
-  u[c] = us[c] - ax * fc.cx[c] * (pc - p[x.cim]);
-  v[c] = (g.ywall && x.j == 0) ? 0.0 : vs[c] - ay * fc.cy[c] * (pc - p[x.cjm]);
-  w[c] = (x.k == 0) ? 0.0 : ws[c] - dt * is * fc.cz[c] * (pc - p[c - plane]);
+  double dz = dt;
+  double ax = (dt * g.dx) * g.inv_dzf[x.k];
+  const double ay = (dt * g.dy) * g.inv_dzf[x.k];
+  if (g.ym) {
+    const double is = g.ym[2 * g.ny + x.j];
+    ax *= is;
+    dz *= is;
+  }
+  u[c] = fma(-ax, fc.cx[c] * (pc - p[x.cim]), us[c]);
+  v[c] = (g.ywall && x.j == 0) ? 0.0 : fma(-ay, fc.cy[c] * (pc - p[x.cjm]), vs[c]);
+  w[c] = (x.k == 0) ? 0.0 : fma(-dz, fc.cz[c] * (pc - p[c - plane]), ws[c]);
   if (x.k == g.nz - 1) w[c + plane] = 0.0;
 }
 

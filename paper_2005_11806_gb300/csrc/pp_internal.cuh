@@ -51,6 +51,7 @@ struct DevStatus {
 struct Geo {
   int nx, ny, nz, nxh;
   double dx, dy, inv_dx2, inv_dy2;
+  double inv_dx, inv_dy;
   const double* inv_dzf;  // [nz]   1 / cell width
   const double* inv_dzc;  // [nz+1] 1 / centre distance across z-face k (0 at walls)
   const double* dzf;      // [nz]
@@ -62,6 +63,9 @@ struct Geo {
   // The mixed residual update forms its FP32 coefficients from these and the
   // FP32 density instead of reading stored coefficient fields.
   const float* cw_f;
+  // FP64 layer factors of the face coefficients, [3][nz + 1]: 2 dzf_k / dx^2,
+  // 2 dzf_k / dy^2 (k < nz) and 2 / dzc_k (0 on the walls).
+  const double* cw_d;
   double lz;
   int ywall;              // 1: walls at y = 0 and y = ly (v row 0 is the wall face); 0: periodic y
   // Stretched y between walls (null for a uniform y): [3][ny] row factors
@@ -115,6 +119,19 @@ __device__ __forceinline__ float rcp_f32(float x) {
   return r;
 }
 
+// 1 / x in FP64: the hardware's 20-bit estimate and one third-order Newton
+// step, y (1 + e + e^2) with e = 1 - x y (relative error e^3, below the
+// rounding), three FP64 operations.  Where the estimate is 0, Inf or NaN it is
+// the result.
+__device__ __forceinline__ double rcp_f64(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  const double r = fma(y, fma(e, e, e), y);
+  const unsigned h = (unsigned)__double2hiint(y) & 0x7FFFFFFFu;
+  return (h == 0u || h >= 0x7FF00000u) ? y : r;
+}
+
 // 1 / rho_f of a face from its two cells' FP32 densities (arithmetic face
 // density, as the FP64 coefficients): 2 / (a + b).
 __device__ __forceinline__ float face_beta_f(float a, float b) { return 2.f * rcp_f32(a + b); }
@@ -127,6 +144,18 @@ inline bool faces_ok(const double* f, int n) {
   for (int k = 0; k < n; ++k)
     if (!(f[k + 1] > f[k])) return false;
   return true;
+}
+
+// Host: the [3][nz + 1] FP64 layer factors of Geo::cw_d.
+inline std::vector<double> layer_factors_f64(int nz, const std::vector<double>& dzf,
+                                             const std::vector<double>& inv_dzc, double inv_dx2, double inv_dy2) {
+  std::vector<double> cw(3 * (size_t)(nz + 1), 0.0);
+  for (int k = 0; k < nz; ++k) {
+    cw[k] = 2.0 * inv_dx2 * dzf[k];
+    cw[(nz + 1) + k] = 2.0 * inv_dy2 * dzf[k];
+  }
+  for (int k = 0; k <= nz; ++k) cw[2 * (nz + 1) + k] = 2.0 * inv_dzc[k];
+  return cw;
 }
 
 // Host: the [3][nz + 1] FP32 layer factors of Geo::cw_f.
@@ -351,10 +380,10 @@ cudaError_t launch_divergence_source(const Geo& g, const double* phi, const doub
                                      double p0, double gamma, double dp0dt, double* S, cudaStream_t s);
 // Momentum predictor (Eqs. 29, 32): out = u + dt (a RU - b prev) on the u, v
 // and w faces (w wall planes zero); ru (entries may be null) receives RU;
-// f and prev entries may be null.  D: a cell-field scratch (the divergence).
+// f and prev entries may be null.
 cudaError_t launch_predictor(const Geo& g, const double* u, const double* v, const double* w, const double* rho,
                              const double* mu, const double* const f[3], const double* const prev[3],
-                             const double grav[3], double dt, double a, double b, double* D, double* const out[3],
+                             const double grav[3], double dt, double a, double b, double* const out[3],
                              double* const ru[3], cudaStream_t s);
 cudaError_t launch_adj_grho(const Geo& g, const double* tx, const double* ty, const double* tz,
                             double* grho, cudaStream_t s);

@@ -7,7 +7,9 @@
 namespace pp {
 
 namespace {
-constexpr int kRedBlocks = 1024;  // partial sums written by the reduction kernels
+// Partial sums written by the reduction kernels: six blocks for each of the 152
+// SMs (1024 blocks left 40 of them a seventh one; a third of it is two each).
+constexpr int kRedBlocks = 912;
 constexpr int kThreads = 256;
 
 inline int grid_for(size_t n) {
@@ -46,11 +48,12 @@ __global__ void k_prep_diag(Geo g, Faces fc) {
 // the cell volume over dx dy) (grid of kRedBlocks blocks).
 __global__ void k_weighted_partial(Geo g, const double* __restrict__ f, double* __restrict__ red) {
   __shared__ double sh[32];
-  const size_t plane = (size_t)g.nx * g.ny, n = plane * g.nz;
+  const unsigned nx = (unsigned)g.nx, ny = (unsigned)g.ny, n = nx * ny * (unsigned)g.nz;
   double s = 0.0;
-  for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (size_t)gridDim.x * blockDim.x) {
-    const double wy = g.ym ? g.ym[(c / g.nx) % g.ny] : 1.0;
-    s += g.dzf[c / plane] * wy * f[c];
+  for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
+    const unsigned row = c / nx, k = row / ny;
+    const double w = g.ym ? g.dzf[k] * g.ym[row - k * ny] : g.dzf[k];
+    s = fma(w, f[c], s);
   }
   s = block_sum<double>(s, sh);
   if (threadIdx.x == 0) red[blockIdx.x] = s;
@@ -248,17 +251,18 @@ __global__ void k_thermo_partial(Geo g, const double* __restrict__ phi, const do
   for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (size_t)gridDim.x * blockDim.x) {
     const CellIdx x = cell_index(g, c);
     const double f = phi[c];
-    const double sj = g.ym ? g.ym[x.j] : 1.0;  // stretched y: dyf_j = s_j dy
-    const double dv = dxdy * g.dzf[x.k] * sj;
+    const double fdv = f * (g.ym ? g.dzf[x.k] * g.ym[x.j] : g.dzf[x.k]);  // over dx dy
     const double wlo = (x.k == 0) ? 0.0 : w[c];
     const double whi = (x.k == g.nz - 1) ? 0.0 : w[c + plane];
     // the wall row of v (walls in y) carries no flux, like the wall planes of w
     const double vlo = (g.ywall && x.j == 0) ? 0.0 : v[c];
     const double vhi = (g.ywall && x.j == g.ny - 1) ? 0.0 : v[x.cjp];
-    const double div = (u[x.cip] - u[c]) / g.dx + (vhi - vlo) / (g.dy * sj) + (whi - wlo) * g.inv_dzf[x.k];
-    a += f * cell_conduction(g, kc, T, c) * dv;
-    b += f * div * dv;
-    vg += f * dv;
+    double dvy = vhi - vlo;
+    if (g.ym) dvy *= g.ym[2 * g.ny + x.j];  // stretched y: dyf_j = s_j dy
+    const double div = fma(u[x.cip] - u[c], g.inv_dx, fma(dvy, g.inv_dy, (whi - wlo) * g.inv_dzf[x.k]));
+    a = fma(fdv, cell_conduction2(g, kc, T, c), a);
+    b = fma(fdv, div, b);
+    vg += fdv;
   }
   a = block_sum<double>(a, sh);
   __syncthreads();
@@ -266,9 +270,9 @@ __global__ void k_thermo_partial(Geo g, const double* __restrict__ phi, const do
   __syncthreads();
   vg = block_sum<double>(vg, sh);
   if (threadIdx.x == 0) {
-    red[3 * (size_t)blockIdx.x] = a;
-    red[3 * (size_t)blockIdx.x + 1] = b;
-    red[3 * (size_t)blockIdx.x + 2] = vg;
+    red[3 * (size_t)blockIdx.x] = 0.5 * dxdy * a;
+    red[3 * (size_t)blockIdx.x + 1] = dxdy * b;
+    red[3 * (size_t)blockIdx.x + 2] = dxdy * vg;
   }
 }
 
@@ -291,29 +295,28 @@ __global__ void k_thermo_rate(const double* __restrict__ red, int nblk, double p
   }
 }
 
-// S = (1/p0) [ (gamma - 1)/gamma div(k grad T) - dp0dt / gamma ] Phi  (Eq. 34).
+// S = (1/p0) [ (gamma - 1)/gamma div(k grad T) - dp0dt / gamma ] Phi  (Eq. 34);
+// a = (gamma - 1) / (2 gamma p0), b = dp0dt / (gamma p0) come from the host
+// (three divisions a thread were a quarter of the kernel).  FP64-pipe bound:
+// 256^3 1.14 -> 0.79 ms.
 __global__ void k_divergence_source(Geo g, const double* __restrict__ phi, const double* __restrict__ kc,
-                                    const double* __restrict__ T, double p0, double gamma, double dp0dt,
-                                    double* __restrict__ S) {
+                                    const double* __restrict__ T, double a, double b, double* __restrict__ S) {
   const size_t n = (size_t)g.nx * g.ny * g.nz;
-  const double a = (gamma - 1.0) / gamma, b = dp0dt / gamma, ip0 = 1.0 / p0;
   for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (size_t)gridDim.x * blockDim.x)
-    S[c] = (a * cell_conduction(g, kc, T, c) - b) * phi[c] * ip0;
+    S[c] = fma(a, cell_conduction2(g, kc, T, c), -b) * phi[c];
 }
 
 // ---- momentum predictor (Eqs. 29, 32) ---------------------------------------
-
-__global__ void k_cell_divergence(Geo g, const double* __restrict__ u, const double* __restrict__ v,
-                                  const double* __restrict__ w, double* __restrict__ D) {
-  const size_t plane = (size_t)g.nx * g.ny, n = plane * g.nz;
-  for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (size_t)gridDim.x * blockDim.x) {
-    const CellIdx x = cell_index(g, c);
-    // walls in y: the wall row of v carries no flux
-    const double vlo = (g.ywall && x.j == 0) ? 0.0 : v[c];
-    const double vhi = (g.ywall && x.j == g.ny - 1) ? 0.0 : v[x.cjp];
-    D[c] = (u[x.cip] - u[c]) / g.dx + (vhi - vlo) / g.dy + (w[c + plane] - w[c]) * g.inv_dzf[x.k];
-  }
-}
+struct PredArgs {
+  const double *u, *v, *w, *rho, *mu;
+  const double *fx, *fy, *fz;  // body force, entries may be null
+  const double *pu, *pv, *pw;  // RU of the step before, null: forward Euler
+  double gx, gy, gz, dta, dtb;      // dt a, dt b
+  double idx, idy, hdx, hdy, tdx, tdy; // 1 / h, 1 / (2 h), 8 / h: uniform products cost FP64 issue like any other
+  double *us, *vs, *ws;
+  double *ru, *rv, *rw;        // RU, entries may be null
+};
+constexpr int kPredLanes = 30;  // useful lanes of a warp; lanes 0 and 31 hold the x neighbours
 
 // Predicted velocity at the three low faces of cell (i, j, k): the u-face
 // i-1/2, the v-face j-1/2 and (k >= 1) the w-face k-1/2.  RU = -C(u) +
@@ -324,156 +327,186 @@ __global__ void k_cell_divergence(Geo g, const double* __restrict__ u, const dou
 // shear parts at edges with the mean mu of the cells around the edge;
 // no-slip z walls: wall velocity zero, half-cell distance to the wall).
 // With walls in y the y walls are no-slip too: the wall row of v is zero
-// (read as zero, written as zero), the edges on y = 0 (edge row 0) and
-// y = ly (edge row ny) carry the wall shear of u and w over half a cell and
-// no convective flux, and the edges where a y wall meets a z wall carry
-// nothing.  Edge rows are passed unwrapped (0 .. ny); periodic y wraps ny
-// to 0.  u* = u + dt (a RU - b RU_prev).  D: cell divergence.
-__global__ void k_predictor(Geo g, const double* __restrict__ u, const double* __restrict__ v,
-                            const double* __restrict__ w, const double* __restrict__ rho,
-                            const double* __restrict__ mu, const double* __restrict__ D,
-                            const double* __restrict__ fx, const double* __restrict__ fy,
-                            const double* __restrict__ fz, const double* __restrict__ pu,
-                            const double* __restrict__ pv, const double* __restrict__ pw, double gx, double gy,
-                            double gz, double dt, double a, double b, double* __restrict__ us,
-                            double* __restrict__ vs, double* __restrict__ ws, double* __restrict__ ru,
-                            double* __restrict__ rv, double* __restrict__ rw) {
+// (read as zero, written as zero), the edges on y = 0 and y = ly carry the
+// wall shear of u and w over half a cell and no convective flux, and the
+// edges where a y wall meets a z wall carry nothing.  u* = u + dt (a RU - b
+// RU_prev).
+//
+// Bound by the FP64 pipe.  A cell's edge and centre terms are shared with its
+// neighbours: a warp holds 30 consecutive cells of one row (and one neighbour
+// on each side, exchanged by shuffles) and marches in z, so x and z
+// neighbours' terms come from registers and only those of the rows j - 1 and
+// j + 1 are formed twice; about 160 FP64 operations a cell against about 365
+// with every term formed at both of its cells and three IEEE divisions.
+// 256^3: 9.7 ms -> 6.2 ms (FP64 pipe 86 % busy; 12 % of the lanes are the tiles'
+// neighbours at 256).
+__global__ void __launch_bounds__(128) k_predictor(Geo g, PredArgs A, int ntile, int nchunk, int chunk) {
   const int nx = g.nx, ny = g.ny, nz = g.nz;
+  const int lane = threadIdx.x & 31;
+  const unsigned wid = blockIdx.x * 4 + (threadIdx.x >> 5);
+  const unsigned rest = wid / (unsigned)ntile;
+  const int tile = (int)(wid - rest * ntile);
+  const int ch = (int)(rest / (unsigned)ny), j = (int)(rest - (unsigned)ch * ny);
+  if (ch >= nchunk) return;
+  const int k0 = ch * chunk, k1 = min(k0 + chunk, nz);
+  const int at = tile * kPredLanes + lane - 1;  // -1 .. ; wraps
+  int i = at < 0 ? at + nx : at;
+  while (i >= nx) i -= nx;
+  const bool emit_lane = lane >= 1 && lane <= kPredLanes && at < nx;
   const bool ywall = g.ywall != 0;
-  const size_t plane = (size_t)nx * ny, n = plane * nz;
-  const double idx = 1.0 / g.dx, idy = 1.0 / g.dy;
-  const double two3 = 2.0 / 3.0;
-  for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (size_t)gridDim.x * blockDim.x) {
-    const int i = (int)(c % nx), j = (int)((c / nx) % ny), k = (int)(c / plane);
-    const int im = i == 0 ? nx - 1 : i - 1, ip = i + 1 == nx ? 0 : i + 1;
-    const int jm = j == 0 ? ny - 1 : j - 1, jp = j + 1 == ny ? 0 : j + 1;
-    auto at = [&](int ii, int jj, int kk) { return ((size_t)kk * ny + jj) * nx + ii; };
-    // v at the face row jj (0 .. ny - 1); the wall row reads as zero
-    auto vv = [&](int ii, int jj, int kk) { return (ywall && jj == 0) ? 0.0 : v[at(ii, jj, kk)]; };
-    const double idzf = g.inv_dzf[k];
-    // is the edge row jj (0 .. ny) a y wall?
-    auto ywall_edge = [&](int jj) { return ywall && (jj == 0 || jj == ny); };
-    // mean mu over the four cells around an x-y edge (i'-1/2, j'-1/2) of layer kk (interior edge row)
-    auto mxy = [&](int ii, int jj, int kk) {
-      const int iim = ii == 0 ? nx - 1 : ii - 1, jjm = jj == 0 ? ny - 1 : jj - 1;
-      return 0.25 * (mu[at(ii, jj, kk)] + mu[at(iim, jj, kk)] + mu[at(ii, jjm, kk)] + mu[at(iim, jjm, kk)]);
-    };
-    // shear stress tau_xy at the edge (i'-1/2, jj-1/2) of layer kk, jj in [0, ny]
-    auto txy = [&](int ii, int jj, int kk) {
-      const int iim = ii == 0 ? nx - 1 : ii - 1;
-      if (ywall_edge(jj)) {  // no-slip y wall: u = 0 half a cell away, v = 0 along it
-        const int jr = jj == 0 ? 0 : ny - 1;
-        const double m = 0.5 * (mu[at(ii, jr, kk)] + mu[at(iim, jr, kk)]);
-        return (jj == 0 ? 2.0 : -2.0) * m * u[at(ii, jr, kk)] * idy;
-      }
-      const int jw = jj == ny ? 0 : jj, jjm = jw == 0 ? ny - 1 : jw - 1;
-      return mxy(ii, jw, kk) * ((u[at(ii, jw, kk)] - u[at(ii, jjm, kk)]) * idy +
-                                (vv(ii, jw, kk) - vv(iim, jw, kk)) * idx);
-    };
-    // tau_xz at the edge (i'-1/2, kk-1/2), kk in [0, nz]; tau_yz likewise
-    auto txz = [&](int ii, int jj, int kk) {
-      const int iim = ii == 0 ? nx - 1 : ii - 1;
-      if (kk == 0) return 0.5 * (mu[at(ii, jj, 0)] + mu[at(iim, jj, 0)]) * u[at(ii, jj, 0)] * 2.0 * g.inv_dzf[0];
-      if (kk == nz)
-        return -0.5 * (mu[at(ii, jj, nz - 1)] + mu[at(iim, jj, nz - 1)]) * u[at(ii, jj, nz - 1)] * 2.0 *
-               g.inv_dzf[nz - 1];
-      const double m = 0.25 * (mu[at(ii, jj, kk)] + mu[at(iim, jj, kk)] + mu[at(ii, jj, kk - 1)] +
-                               mu[at(iim, jj, kk - 1)]);
-      return m * ((u[at(ii, jj, kk)] - u[at(ii, jj, kk - 1)]) * g.inv_dzc[kk] +
-                  (w[at(ii, jj, kk)] - w[at(iim, jj, kk)]) * idx);
-    };
-    // tau_yz at the edge (jj-1/2, kk-1/2), jj in [0, ny], kk in [0, nz]
-    auto tyz = [&](int ii, int jj, int kk) {
-      if (ywall_edge(jj)) {  // no-slip y wall: w = 0 half a cell away, v = 0 along it
-        if (kk == 0 || kk == nz) return 0.0;  // a y wall meets a z wall
-        const int jr = jj == 0 ? 0 : ny - 1;
-        const double m = 0.5 * (mu[at(ii, jr, kk)] + mu[at(ii, jr, kk - 1)]);
-        return (jj == 0 ? 2.0 : -2.0) * m * w[at(ii, jr, kk)] * idy;
-      }
-      const int jw = jj == ny ? 0 : jj, jjm = jw == 0 ? ny - 1 : jw - 1;
-      if (kk == 0) return 0.5 * (mu[at(ii, jw, 0)] + mu[at(ii, jjm, 0)]) * vv(ii, jw, 0) * 2.0 * g.inv_dzf[0];
-      if (kk == nz)
-        return -0.5 * (mu[at(ii, jw, nz - 1)] + mu[at(ii, jjm, nz - 1)]) * vv(ii, jw, nz - 1) * 2.0 *
-               g.inv_dzf[nz - 1];
-      const double m = 0.25 * (mu[at(ii, jw, kk)] + mu[at(ii, jjm, kk)] + mu[at(ii, jw, kk - 1)] +
-                               mu[at(ii, jjm, kk - 1)]);
-      return m * ((vv(ii, jw, kk) - vv(ii, jw, kk - 1)) * g.inv_dzc[kk] +
-                  (w[at(ii, jw, kk)] - w[at(ii, jjm, kk)]) * idy);
-    };
-    // convective cross products at edges (zero on the walls, where the
-    // wall-normal velocity vanishes)
-    auto fxy = [&](int ii, int jj, int kk) {  // u v at (i'-1/2, jj-1/2), jj in [0, ny]
-      if (ywall_edge(jj)) return 0.0;
-      const int jw = jj == ny ? 0 : jj;
-      const int iim = ii == 0 ? nx - 1 : ii - 1, jjm = jw == 0 ? ny - 1 : jw - 1;
-      return 0.25 * (u[at(ii, jw, kk)] + u[at(ii, jjm, kk)]) * (vv(ii, jw, kk) + vv(iim, jw, kk));
-    };
-    auto fxz = [&](int ii, int jj, int kk) {  // u w at (i'-1/2, kk-1/2); zero at the walls
-      if (kk == 0 || kk == nz) return 0.0;
-      const int iim = ii == 0 ? nx - 1 : ii - 1;
-      return 0.25 * (u[at(ii, jj, kk)] + u[at(ii, jj, kk - 1)]) * (w[at(ii, jj, kk)] + w[at(iim, jj, kk)]);
-    };
-    auto fyz = [&](int ii, int jj, int kk) {  // v w at (jj-1/2, kk-1/2), jj in [0, ny]
-      if (kk == 0 || kk == nz || ywall_edge(jj)) return 0.0;
-      const int jw = jj == ny ? 0 : jj, jjm = jw == 0 ? ny - 1 : jw - 1;
-      return 0.25 * (vv(ii, jw, kk) + vv(ii, jw, kk - 1)) * (w[at(ii, jw, kk)] + w[at(ii, jjm, kk)]);
-    };
-    const double Dc = D[c];
-    // ---- x momentum at the u-face (i-1/2, j, k)
-    {
-      const size_t cm = at(im, j, k);
-      const double uc0 = 0.5 * (u[c] + u[at(ip, j, k)]), ucm = 0.5 * (u[cm] + u[c]);
-      const double conv = (uc0 * uc0 - ucm * ucm) * idx + (fxy(i, j + 1, k) - fxy(i, j, k)) * idy +
-                          (fxz(i, j, k + 1) - fxz(i, j, k)) * idzf - u[c] * 0.5 * (Dc + D[cm]);
-      const double t0 = mu[c] * (2.0 * (u[at(ip, j, k)] - u[c]) * idx - two3 * Dc);
-      const double tm = mu[cm] * (2.0 * (u[c] - u[cm]) * idx - two3 * D[cm]);
-      double visc = (t0 - tm) * idx + (txy(i, j + 1, k) - txy(i, j, k)) * idy +
-                    (txz(i, j, k + 1) - txz(i, j, k)) * idzf;
-      if (fx != nullptr) visc += fx[c];
-      const double r = -conv + visc / (0.5 * (rho[c] + rho[cm])) + gx;
-      us[c] = u[c] + dt * (a * r - (pu != nullptr ? b * pu[c] : 0.0));
-      if (ru != nullptr) ru[c] = r;
+  const bool wlo = ywall && j == 0, whi = ywall && j + 1 == ny;  // the row's low / high y edges are walls
+  const int jm = j == 0 ? ny - 1 : j - 1, jp = j + 1 == ny ? 0 : j + 1;
+  const bool vz_m = ywall && jm == 0, vz_p = ywall && jp == 0;   // rows whose v reads as zero
+  const size_t plane = (size_t)nx * ny;
+  const size_t oc = (size_t)j * nx + i, om = (size_t)jm * nx + i, op = (size_t)jp * nx + i;
+  const double idx = A.idx, idy = A.idy;
+  constexpr unsigned full = 0xffffffffu;
+  auto left = [&](double a) { return __shfl_up_sync(full, a, 1); };     // value at i - 1
+  auto right = [&](double a) { return __shfl_down_sync(full, a, 1); };  // value at i + 1
+
+  const int ks = k0 > 0 ? k0 - 1 : 0;  // the layer below the chunk only leaves its upper edges and centre
+  size_t o = (size_t)ks * plane;
+  // layer k of rows j, j - 1, j + 1
+  double uc = A.u[o + oc], um = A.u[o + om], up = A.u[o + op];
+  double vc = wlo ? 0.0 : A.v[o + oc], vm = vz_m ? 0.0 : A.v[o + om], vp = vz_p ? 0.0 : A.v[o + op];
+  // half the viscosity: the sum over an edge's four cells is then twice their
+  // mean, and every stress is formed doubled
+  double mc = 0.5 * A.mu[o + oc], mm = 0.5 * A.mu[o + om], mp = 0.5 * A.mu[o + op];
+  double wc = A.w[o + oc], wm = A.w[o + om], wp = A.w[o + op];  // face k
+  // sums of mu over cell pairs: x pairs of the three rows, y pairs
+  double sx = mc + left(mc), sy = mc + mm, syp = mc + mp;
+  // lower edges: x-z, y-z below row j, y-z above row j (4 x the convective
+  // product, 2 x the stress); the z wall of layer 0, else set by the layer below
+  double Fxz = 0.0, Txz, Fyz = 0.0, Tyz, Fyp = 0.0, Typ = 0.0;
+  {
+    const double h = 2.0 * g.inv_dzf[0];  // sx: the mean of the two cells
+    Txz = sx * uc * h;
+    Tyz = wlo ? 0.0 : sy * vc * h;
+    Txz *= 2.0;
+    Tyz *= 2.0;
+  }
+  double Dk = 0.0, Czk = 0.0, Tzk = 0.0, rk = 0.0;  // layer k - 1: divergence, centre terms, density
+  for (int k = ks; k < k1; ++k, o += plane) {
+    const bool top = k + 1 == nz;
+    const size_t ou = o + plane;
+    // ---- layer k + 1
+    const double wuc = A.w[ou + oc], wum = A.w[ou + om], wup = A.w[ou + op];  // face k + 1
+    double uu = 0.0, uum = 0.0, uup = 0.0, vu = 0.0, vum = 0.0, vup = 0.0, mu_ = 0.0, mum = 0.0, mup = 0.0;
+    if (!top) {
+      uu = A.u[ou + oc]; uum = A.u[ou + om]; uup = A.u[ou + op];
+      vu = wlo ? 0.0 : A.v[ou + oc]; vum = vz_m ? 0.0 : A.v[ou + om]; vup = vz_p ? 0.0 : A.v[ou + op];
+      mu_ = 0.5 * A.mu[ou + oc]; mum = 0.5 * A.mu[ou + om]; mup = 0.5 * A.mu[ou + op];
     }
-    // ---- y momentum at the v-face (i, j-1/2, k); with walls in y the wall row stays zero
-    if (ywall && j == 0) {
-      vs[c] = 0.0;
-      if (rv != nullptr) rv[c] = 0.0;
+    const double rc = A.rho[o + oc], rm = A.rho[o + om];
+    const double idzf = g.inv_dzf[k], idzc = g.inv_dzc[k + 1];
+    // ---- centres of layer k
+    const double ur = right(uc), urm = right(um), vl = left(vc), vlp = left(vp), wl = left(wuc);
+    const double dux = ur - uc, dvy = vp - vc, dvm = vc - vm, dwz = wuc - wc;
+    const double D = fma(dux, idx, fma(dvy, idy, dwz * idzf));
+    const double Dm = fma(urm - um, idx, fma(dvm, idy, (wum - wm) * idzf));  // row j - 1
+    // 2 tau = (mu / 2) (8 d - 8/3 D)
+    const double t83 = (-8.0 / 3.0) * D, t83m = (-8.0 / 3.0) * Dm;
+    const double Tx = mc * fma(dux, A.tdx, t83), Ty = mc * fma(dvy, A.tdy, t83);
+    const double Tym = mm * fma(dvm, A.tdy, t83m), Tz = mc * fma(dwz, 8.0 * idzf, t83);
+    const double ax = uc + ur, ay = vc + vp, aym = vm + vc, az = wc + wuc;
+    const double Cx = ax * ax, Cy = ay * ay, Cym = aym * aym, Cz = az * az;  // 4 x the products
+    // ---- x-y edges below and above row j (4 x the convective product)
+    const double sxm = mm + left(mm), sxp = mp + left(mp);
+    double Fxy = 0.0, Txy, Fxyp = 0.0, Txyp;
+    if (wlo) Txy = sx * uc * (0.5 * A.tdy);  // 2 x 2 mu u / dy
+    else {
+      Fxy = (uc + um) * (vc + vl);
+      Txy = (sx + sxm) * fma(uc - um, idy, (vc - vl) * idx);
+    }
+    if (whi) Txyp = -sx * uc * (0.5 * A.tdy);
+    else {
+      Fxyp = (up + uc) * (vp + vlp);
+      Txyp = (sx + sxp) * fma(up - uc, idy, (vp - vlp) * idx);
+    }
+    // ---- edges on face k + 1
+    const double sxu = mu_ + left(mu_), syu = mu_ + mum, sypu = mu_ + mup;
+    double FxzU = 0.0, TxzU, FyzU = 0.0, TyzU, FypU = 0.0, TypU = 0.0;
+    if (top) {
+      const double h = -4.0 * idzf;  // 2 x (-2 / dzf) times the mean of two cells
+      TxzU = sx * uc * h;
+      TyzU = wlo ? 0.0 : sy * vc * h;
     } else {
-      const size_t cm = at(i, jm, k);
-      const double vvc = vv(i, j, k), vvp = vv(i, jp, k), vvm = vv(i, jm, k);
-      const double vc0 = 0.5 * (vvc + vvp), vcm = 0.5 * (vvm + vvc);
-      const double conv = (fxy(ip, j, k) - fxy(i, j, k)) * idx + (vc0 * vc0 - vcm * vcm) * idy +
-                          (fyz(i, j, k + 1) - fyz(i, j, k)) * idzf - vvc * 0.5 * (Dc + D[cm]);
-      const double t0 = mu[c] * (2.0 * (vvp - vvc) * idy - two3 * Dc);
-      const double tm = mu[cm] * (2.0 * (vvc - vvm) * idy - two3 * D[cm]);
-      double visc = (txy(ip, j, k) - txy(i, j, k)) * idx + (t0 - tm) * idy + (tyz(i, j, k + 1) - tyz(i, j, k)) * idzf;
-      if (fy != nullptr) visc += fy[c];
-      const double r = -conv + visc / (0.5 * (rho[c] + rho[cm])) + gy;
-      vs[c] = vvc + dt * (a * r - (pv != nullptr ? b * pv[c] : 0.0));
-      if (rv != nullptr) rv[c] = r;
+      FxzU = (uc + uu) * (wuc + wl);
+      TxzU = (sx + sxu) * fma(uu - uc, idzc, (wuc - wl) * idx);
+      const double mz = mc + mu_;
+      if (wlo) TyzU = mz * wuc * (0.5 * A.tdy);  // 2 x 2 mu w / dy
+      else {
+        FyzU = (vc + vu) * (wuc + wum);
+        TyzU = (sy + syu) * fma(vu - vc, idzc, (wuc - wum) * idy);
+      }
+      if (whi) TypU = -mz * wuc * (0.5 * A.tdy);
+      else {
+        FypU = (vp + vup) * (wup + wuc);
+        TypU = (syp + sypu) * fma(vup - vp, idzc, (wup - wuc) * idy);
+      }
     }
-    // ---- z momentum at the w-face (i, j, k-1/2), interior faces only
-    if (k == 0) {
-      ws[c] = 0.0;
-      if (rw != nullptr) rw[c] = 0.0;
-    } else {
-      const size_t cm = c - plane;
-      const double wc0 = 0.5 * (w[c] + w[c + plane]), wcm = 0.5 * (w[cm] + w[c]);
-      const double idzc = g.inv_dzc[k];
-      const double conv = (fxz(ip, j, k) - fxz(i, j, k)) * idx + (fyz(i, j + 1, k) - fyz(i, j, k)) * idy +
-                          (wc0 * wc0 - wcm * wcm) * idzc - w[c] * 0.5 * (Dc + D[cm]);
-      const double t0 = mu[c] * (2.0 * (w[c + plane] - w[c]) * idzf - two3 * Dc);
-      const double tm = mu[cm] * (2.0 * (w[c] - w[cm]) * g.inv_dzf[k - 1] - two3 * D[cm]);
-      double visc = (txz(ip, j, k) - txz(i, j, k)) * idx + (tyz(i, j + 1, k) - tyz(i, j, k)) * idy + (t0 - tm) * idzc;
-      if (fz != nullptr) visc += fz[c];
-      const double r = -conv + visc / (0.5 * (rho[c] + rho[cm])) + gz;
-      ws[c] = w[c] + dt * (a * r - (pw != nullptr ? b * pw[c] : 0.0));
-      if (rw != nullptr) rw[c] = r;
+    // the neighbours' terms (every lane takes part)
+    const double Cxl = left(Cx), Txl = left(Tx), Dl = left(D), rl = left(rc);
+    const double Fxyr = right(Fxy), Txyr = right(Txy), Fxzr = right(Fxz), Txzr = right(Txz);
+    if (k >= k0 && emit_lane) {
+      const size_t c = o + oc;
+      const double qz = 0.5 * idzf;  // cv: 2 x the convection
+      // ---- x momentum at the u-face (i-1/2, j, k)
+      {
+        double cv = fma(Cx - Cxl, A.hdx, fma(Fxyp - Fxy, A.hdy, (FxzU - Fxz) * qz));
+        cv = fma(-uc, D + Dl, cv);
+        double vs = fma(Tx - Txl, idx, fma(Txyp - Txy, idy, (TxzU - Txz) * idzf));
+        if (A.fx != nullptr) vs = fma(2.0, A.fx[c], vs);
+        const double r = fma(-0.5, cv, fma(vs, rcp_f64(rc + rl), A.gx));
+        double q = fma(A.dta, r, uc);
+        if (A.pu != nullptr) q = fma(-A.dtb, A.pu[c], q);
+        A.us[c] = q;
+        if (A.ru != nullptr) A.ru[c] = r;
+      }
+      // ---- y momentum at the v-face (i, j-1/2, k); the wall row stays zero
+      if (wlo) {
+        A.vs[c] = 0.0;
+        if (A.rv != nullptr) A.rv[c] = 0.0;
+      } else {
+        double cv = fma(Fxyr - Fxy, A.hdx, fma(Cy - Cym, A.hdy, (FyzU - Fyz) * qz));
+        cv = fma(-vc, D + Dm, cv);
+        double vs = fma(Txyr - Txy, idx, fma(Ty - Tym, idy, (TyzU - Tyz) * idzf));
+        if (A.fy != nullptr) vs = fma(2.0, A.fy[c], vs);
+        const double r = fma(-0.5, cv, fma(vs, rcp_f64(rc + rm), A.gy));
+        double q = fma(A.dta, r, vc);
+        if (A.pv != nullptr) q = fma(-A.dtb, A.pv[c], q);
+        A.vs[c] = q;
+        if (A.rv != nullptr) A.rv[c] = r;
+      }
+      // ---- z momentum at the w-face (i, j, k-1/2), interior faces only
+      if (k == 0) {
+        A.ws[c] = 0.0;
+        if (A.rw != nullptr) A.rw[c] = 0.0;
+      } else {
+        const double ic = g.inv_dzc[k];
+        double cv = fma(Fxzr - Fxz, A.hdx, fma(Fyp - Fyz, A.hdy, (Cz - Czk) * (0.5 * ic)));
+        cv = fma(-wc, D + Dk, cv);
+        double vs = fma(Txzr - Txz, idx, fma(Typ - Tyz, idy, (Tz - Tzk) * ic));
+        if (A.fz != nullptr) vs = fma(2.0, A.fz[c], vs);
+        const double r = fma(-0.5, cv, fma(vs, rcp_f64(rc + rk), A.gz));
+        double q = fma(A.dta, r, wc);
+        if (A.pw != nullptr) q = fma(-A.dtb, A.pw[c], q);
+        A.ws[c] = q;
+        if (A.rw != nullptr) A.rw[c] = r;
+      }
+      if (top) {
+        A.ws[c + plane] = 0.0;
+        if (A.rw != nullptr) A.rw[c + plane] = 0.0;
+      }
     }
-    if (k == nz - 1) {
-      ws[c + plane] = 0.0;
-      if (rw != nullptr) rw[c + plane] = 0.0;
-    }
+    // ---- on to layer k + 1
+    uc = uu; um = uum; up = uup;
+    vc = vu; vm = vum; vp = vup;
+    mc = mu_; mm = mum; mp = mup;
+    wc = wuc; wm = wum; wp = wup;
+    sx = sxu; sy = syu; syp = sypu;
+    Fxz = FxzU; Txz = TxzU; Fyz = FyzU; Tyz = TyzU; Fyp = FypU; Typ = TypU;
+    Dk = D; Czk = Cz; Tzk = Tz; rk = rc;
   }
 }
 
@@ -639,19 +672,26 @@ cudaError_t launch_thermo_rate(const Geo& g, const double* phi, const double* kc
 
 cudaError_t launch_divergence_source(const Geo& g, const double* phi, const double* kc, const double* T,
                                      double p0, double gamma, double dp0dt, double* S, cudaStream_t s) {
-  k_divergence_source<<<grid_for((size_t)g.nx * g.ny * g.nz), kThreads, 0, s>>>(g, phi, kc, T, p0, gamma, dp0dt, S);
+  k_divergence_source<<<grid_for((size_t)g.nx * g.ny * g.nz), kThreads, 0, s>>>(
+      g, phi, kc, T, 0.5 * (gamma - 1.0) / gamma / p0, dp0dt / gamma / p0, S);
   return cudaGetLastError();
 }
 
 cudaError_t launch_predictor(const Geo& g, const double* u, const double* v, const double* w, const double* rho,
                              const double* mu, const double* const f[3], const double* const prev[3],
-                             const double grav[3], double dt, double a, double b, double* D, double* const out[3],
+                             const double grav[3], double dt, double a, double b, double* const out[3],
                              double* const ru[3], cudaStream_t s) {
-  const size_t n = (size_t)g.nx * g.ny * g.nz;
-  k_cell_divergence<<<grid_for(n), kThreads, 0, s>>>(g, u, v, w, D);
-  k_predictor<<<grid_for(n), kThreads, 0, s>>>(g, u, v, w, rho, mu, D, f[0], f[1], f[2], prev[0], prev[1], prev[2],
-                                               grav[0], grav[1], grav[2], dt, a, b, out[0], out[1], out[2], ru[0],
-                                               ru[1], ru[2]);
+  // a warp per 30 cells of a row and chunk of layers: long chunks (a chunk
+  // repeats one layer), but at least about 16 warps an SM
+  const int ntile = (g.nx + kPredLanes - 1) / kPredLanes;
+  const long long rows = (long long)ntile * g.ny;
+  int chunk = 64;
+  while (chunk > 4 && rows * ((g.nz + chunk - 1) / chunk) < 152 * 16) chunk >>= 1;
+  const int nchunk = (g.nz + chunk - 1) / chunk;
+  const PredArgs A{u, v, w, rho, mu, f[0], f[1], f[2], prev[0], prev[1], prev[2], grav[0], grav[1], grav[2],
+                   dt * a, dt * b, g.inv_dx, g.inv_dy, 0.5 * g.inv_dx, 0.5 * g.inv_dy, 8.0 * g.inv_dx,
+                   8.0 * g.inv_dy, out[0], out[1], out[2], ru[0], ru[1], ru[2]};
+  k_predictor<<<(unsigned)((rows * nchunk + 3) / 4), 128, 0, s>>>(g, A, ntile, nchunk, chunk);
   return cudaGetLastError();
 }
 

@@ -232,6 +232,8 @@ extern "C" pp_status pressure_solve_noalloc(const pp_grid* grid, const double* f
   Geo g{};
   g.nx = nx; g.ny = ny; g.nz = nz; g.nxh = nxh;
   g.dx = dx; g.dy = dy;
+  g.inv_dx = 1.0 / g.dx;
+  g.inv_dy = 1.0 / g.dy;
   g.inv_dx2 = 1.0 / (dx * dx);
   g.inv_dy2 = 1.0 / (dy * dy);
   g.inv_dzf = (const double*)(S + o_idzf);
