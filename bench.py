@@ -351,14 +351,14 @@ def run_ours(args, rank, world, local_rank):
         reps = 20
         out["thermo"] = {}
         # FP64 operations per cell (add, multiply and FMA each one FP64-pipe
-        # slot): the conduction stencil 27, Eq. 34's scaling 3; the rate adds
-        # the velocity divergence (8) and three weighted sums (6)
+        # slot): the conduction stencil 23, Eq. 34's scaling 2; the rate adds
+        # the velocity divergence (6) and three weighted sums (4)
         fp64_slots = 152 * 2 * 2.070e9  # FP64 pipe: 2 lanes per clock per SM
         for label, call, nbytes, ops in (
                 ("divergence_source", lambda: pp.pressure_divergence_source(plan.handle, phi, kf, Tf, 1.0, 1.4,
-                                                                             1e-2, Sf), 32 * npts, 30),
+                                                                             1e-2, Sf), 32 * npts, 25),
                 ("p0_rate", lambda: pp.pressure_p0_rate(plan.handle, phi, kf, Tf, us, vs, ws, 1.0, 1.4),
-                 40 * npts + 8 * (w.nz + 1) * w.ny * w.nx, 41)):
+                 40 * npts + 8 * (w.nz + 1) * w.ny * w.nx, 33)):
             for _ in range(3):
                 call()
             torch.cuda.synchronize()
@@ -398,10 +398,9 @@ def run_ours(args, rank, world, local_rank):
         e1.record()
         torch.cuda.synchronize()
         tms = e0.elapsed_time(e1) / reps
-        # bytes: u, v, w, rho, mu, 3 previous RU read; u*, 3 RU written; the
-        # divergence scratch written and read (16 fields of a cell each)
-        nbytes = 16 * 8 * npts
-        ops = 260  # FP64 operations per cell, counted from the stencil (both kernels)
+        # bytes: u, v, w, rho, mu, 3 previous RU read; u*, 3 RU written (14 fields of a cell each)
+        nbytes = 14 * 8 * npts
+        ops = 160  # FP64 operations per cell, counted from the stencil
         rate = ops * npts / (tms / 1e3)
         gbs = nbytes / (tms / 1e3) / 1e9
         out["predictor"] = {"ms": round(tms, 3), "bound": "alu (FP64 pipe)", "fp64_ops_per_cell": ops,

@@ -14,15 +14,15 @@
 using namespace pp;
 
 namespace {
-enum KId { K_RESID, K_CHECK, K_FFTY_F, K_TRI, K_FFTY_I, K_FFTX_I, K_INIT, K_PREP, K_MEANS, K_RHSB,
+enum KId { K_RESID, K_FFTY_F, K_TRI, K_FFTY_I, K_FFTX_I, K_INIT, K_PREP, K_MEANS, K_RHSB,
            K_RMEAN, K_CORR, K_MIX, K_ADJ_RHS, K_ADJ_FIN, K_ADJ_GRHO, K_RHOT, K_FOLD, K_THERMO, K_SOURCE,
            K_PRED, K_ZDCT_F, K_ZDCT_I, K_COUNT };
 const char* const kNames[K_COUNT] = {
-    "resid_fftx", "check", "ffty_fwd", "tridiag_z", "ffty_inv", "fftx_inv_update", "init_status",
+    "resid_fftx", "ffty_fwd", "tridiag_z", "ffty_inv", "fftx_inv_update", "init_status",
     "prep_faces", "mean_S", "rhs_b", "remove_mean", "correct", "mixture_density", "adj_rhs",
     "adj_finish", "adj_grho", "rho_tilde", "fold_pending", "p0_rate", "divergence_source", "predictor",
     "zdct_fwd", "zdct_inv"};
-const int kLaunches[K_COUNT] = {1, 1, 1, 1, 1, 1, 1, 2, 2, 2, 3, 1, 1, 1, 1, 1, 2, 1, 2, 1, 1, 1, 1};
+const int kLaunches[K_COUNT] = {1, 1, 1, 1, 1, 1, 2, 2, 2, 3, 1, 1, 1, 1, 1, 2, 1, 2, 1, 1, 1, 1};
 struct Rec { int kid; cudaEvent_t a, b; };
 struct Prof {
   bool on = false;
@@ -94,6 +94,8 @@ struct pp_plan_s {
   double* d_delta64 = nullptr;
   double* d_thermo = nullptr;  // [4] sums and rate of Eq. 30
   double* d_red = nullptr;
+  unsigned* d_tick = nullptr;  // loop control of the residual kernels (LoopCheck)
+  double* d_gsum = nullptr;
   size_t red_len = 0;
   DevStatus* d_st = nullptr;
   DevStatus* h_st = nullptr;  // pinned, two slots
@@ -376,12 +378,11 @@ pp_status method3_loop(pp_plan_s* P, const double* rho, double* p, int warm, dou
   int polled = 0;
   bool pending[2] = {false, false};
   for (int it = 0; it <= maxit; ++it) {
-    int nblk = 0;
+    const LoopCheck ck{P->d_st, P->d_tick, P->d_gsum, rtol, maxit, kexact};
     PP_K(P, K_RESID, launch_resid_fftx<T>(g, P->faces, P->fx, twx, P->d_b, inv_dt, rho, p,
-                                          (it == 0 && !warm) ? 1 : 0, 1, spec, P->d_red, &nblk,
+                                          (it == 0 && !warm) ? 1 : 0, 1, spec, P->d_red, &ck,
                                           P->d_st, P->stream, upd ? P->d_E : nullptr,
                                           upd ? P->d_delta : nullptr));
-    PP_K(P, K_CHECK, launch_check(P->d_st, P->d_red, nblk, rtol, maxit, kexact, P->stream));
     pp_status s = solve_pass<T>(P, p, 0, dl, upd ? P->d_sdelta : nullptr);
     if (s != PP_OK) return s;
     if ((it + 1) % chunk == 0) {
@@ -443,7 +444,8 @@ void free_plan(pp_plan_s* P) {
   if (!P) return;
   double* dptrs[] = {P->d_inv_dzf, P->d_inv_dzc, P->d_dzf, P->d_za, P->d_zc, P->d_lamx, P->d_lamy,
                      P->d_invd, P->d_mtab, P->d_b, P->d_red, P->faces.cx, P->faces.cy, P->faces.cz,
-                     P->faces.diag, P->d_rho_tilde, P->d_delta64, P->d_thermo, P->d_cw_d};
+                     P->faces.diag, P->d_rho_tilde, P->d_delta64, P->d_thermo, P->d_cw_d, P->d_gsum};
+  if (P->d_tick) cudaFree(P->d_tick);
   if (P->faces.rhof) cudaFree(P->faces.rhof);
   if (P->d_low) cudaFree(P->d_low);
   float* fptrs[] = {P->faces.diagf, P->d_delta, P->d_sdelta, P->d_mtab_f, P->d_invd_f, P->d_zc_f,
@@ -694,6 +696,7 @@ pp_status pressure_plan_create(const pp_grid* grid, pp_precision prec, void* str
   const size_t rpb_min = 2;
   P->red_len = std::max((size_t)2 * ((size_t)G.ny * nz + rpb_min - 1) / rpb_min + 2,
                         (size_t)reduce_blocks());
+  const size_t ngroups = P->red_len / 2 / kCheckGroup + 1;  // of residual blocks
   const bool hybrid = prec == PP_MIXED_FP32;
   if ((hybrid && (st = dalloc(&P->d_invd, nsp * sizeof(double))) != PP_OK) ||
       (hybrid && (st = dalloc(&P->d_mtab, nsp * sizeof(double))) != PP_OK) ||
@@ -703,6 +706,8 @@ pp_status pressure_plan_create(const pp_grid* grid, pp_precision prec, void* str
       (prec != PP_FP64 && (st = dalloc(&P->d_sdelta, nc * sizeof(float))) != PP_OK) ||
       (st = dalloc(&P->d_b, nc * sizeof(double))) != PP_OK ||
       (st = dalloc(&P->d_red, P->red_len * sizeof(double))) != PP_OK ||
+      (st = dalloc(&P->d_tick, (1 + ngroups) * sizeof(unsigned))) != PP_OK ||
+      (st = dalloc(&P->d_gsum, 2 * ngroups * sizeof(double))) != PP_OK ||
       (st = dalloc(&P->faces.cx, nc * sizeof(double))) != PP_OK ||
       (st = dalloc(&P->faces.cy, nc * sizeof(double))) != PP_OK ||
       (st = dalloc(&P->faces.cz, nw * sizeof(double))) != PP_OK ||
@@ -779,6 +784,7 @@ pp_status pressure_plan_create(const pp_grid* grid, pp_precision prec, void* str
   if ((hybrid &&
        launch_setup_pivots(g, P->d_lamx, P->d_lamy, P->d_invd, P->stream, P->d_mtab) != cudaSuccess) ||
       launch_init_status(P->d_st, P->stream) != cudaSuccess ||
+      cudaMemsetAsync(P->d_tick, 0, (1 + ngroups) * sizeof(unsigned), P->stream) != cudaSuccess ||
       cudaStreamSynchronize(P->stream) != cudaSuccess) {
     free_plan(P);
     return PP_ERR_CUDA;

@@ -14,7 +14,7 @@ __global__ void __launch_bounds__(kBatchWThreads, 5) kb_resid_w(const GridDev* G
 #define PP_X(N)                                                                                               \
   case N:                                                                                                     \
     resid_w_body<float, false, N>(d.g, d.fc, d.twx, d.b, d.rho, d.p, 1, 0, 1, d.spec, d.red, exact, d.E, d.delta, \
-                                  w.y, smem_raw);                                                             \
+                                  w.y, smem_raw, LoopCheck{}, 0u);                                            \
     break;
     PP_WFFT_LENGTHS(PP_X)
 #undef PP_X
@@ -34,7 +34,7 @@ static void shape_x(long long nrows, BatchWShape* out) {
   out->smem_x = (size_t)(N + wpb * W::LW * W::LS) * sizeof(float2);
   static_assert((N + wpb * W::LW * W::LS) * sizeof(float2) <= 48 * 1024, "fits without the opt-in attribute");
   out->nblk_x = (int)((warps + wpb - 1) / wpb);
-  out->nred = (int)warps;
+  out->nred = out->nblk_x;
 }
 
 void batch_wfft_x(int nx, long long nrows, BatchWShape* out) {

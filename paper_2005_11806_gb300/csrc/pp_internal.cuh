@@ -6,6 +6,7 @@
 #include <cstddef>
 #include <vector>
 
+#include "pp_launch.cuh"
 #include "pressure_projection.h"
 
 namespace pp {
@@ -184,9 +185,24 @@ __device__ __forceinline__ float narrow_f64(double d) {
 
 // ---- launchers (pp_kernels_*.cu) -------------------------------------
 
+// Loop control of Algorithm 1, run by the residual kernel itself once its last
+// partial sums are in (resid_ticket): st null: none.  kexact: recompute the
+// residual exactly every kexact passes (<= 1: every pass); convergence is only
+// accepted on an exact residual.  tick (1 + groups of kCheckGroup blocks, zero
+// between launches) counts the blocks, gsum holds the groups' sums.
+constexpr int kCheckGroup = 128;
+struct LoopCheck {
+  DevStatus* st;
+  unsigned* tick;
+  double* gsum;
+  double rtol;
+  int maxit, kexact;
+};
+
 // Residual e = b/dt - D(beta G p) (or e = f when f_only), r = rho * e
 // (or r = e), forward real x-transform of r into spec; block partial sums
-// of e^2 and |e| into red[2*block + {0,1}].  Rows are (k, j) pairs.
+// of e^2 and |e| into red[2*block + {0,1}], then the loop control ck (may be
+// null).  Rows are (k, j) pairs.
 //
 // Mixed path with E != null: E = dzf (D u^s - S_c)/dt is kept in FP32.  When
 // st->need_exact is set it is recomputed from p in FP64 (and stored
@@ -195,14 +211,14 @@ __device__ __forceinline__ float narrow_f64(double d) {
 template <typename T>
 cudaError_t launch_resid_fftx(const Geo& g, const Faces& fc, const FftDesc& fx, const C2<T>* twx,
                               const double* b, double inv_dt, const double* rho, const double* p,
-                              int p_zero, int scale_rho, C2<T>* spec, double* red, int* nblk_out,
+                              int p_zero, int scale_rho, C2<T>* spec, double* red, const LoopCheck* ck,
                               const DevStatus* st, cudaStream_t s, float* E = nullptr,
                               const float* delta = nullptr);
 // The same steps for the lengths of PP_WFFT_LENGTHS (pp_wfft.cuh); the
 // launchers route such plans to them.
 template <typename T>
 cudaError_t launch_resid_w(const Geo& g, const Faces& fc, const C2<T>* twx, const double* b, const double* rho,
-                           const double* p, int p_zero, int scale_rho, C2<T>* spec, double* red, int* nblk_out,
+                           const double* p, int p_zero, int scale_rho, C2<T>* spec, double* red, const LoopCheck* ck,
                            const DevStatus* st, cudaStream_t s, float* E, const float* delta);
 template <typename T>
 cudaError_t launch_ffty_w(const Geo& g, const C2<T>* twy, C2<T>* spec, int inverse, const DevStatus* st,
@@ -211,12 +227,12 @@ template <typename T>
 cudaError_t launch_fftx_inv_w(const Geo& g, const C2<T>* twx, const C2<T>* spec, double scale, double* p, int p_zero,
                               const DevStatus* st, cudaStream_t s, T* delta, float* sdelta);
 template <> cudaError_t launch_resid_w<float>(const Geo&, const Faces&, const C2<float>*, const double*, const double*,
-                                            const double*, int, int, C2<float>*, double*, int*, const DevStatus*,
+                                            const double*, int, int, C2<float>*, double*, const LoopCheck*, const DevStatus*,
                                             cudaStream_t, float*, const float*);
 template <> cudaError_t launch_ffty_w<float>(const Geo&, const C2<float>*, C2<float>*, int, const DevStatus*, cudaStream_t,
                                            const C2<float>*);
 template <> cudaError_t launch_resid_w<double>(const Geo&, const Faces&, const C2<double>*, const double*, const double*,
-                                            const double*, int, int, C2<double>*, double*, int*, const DevStatus*,
+                                            const double*, int, int, C2<double>*, double*, const LoopCheck*, const DevStatus*,
                                             cudaStream_t, float*, const float*);
 template <> cudaError_t launch_ffty_w<double>(const Geo&, const C2<double>*, C2<double>*, int, const DevStatus*, cudaStream_t,
                                            const C2<double>*);
@@ -346,11 +362,6 @@ cudaError_t launch_weighted_mean(const Geo& g, const double* f, double* red, dou
 cudaError_t launch_rhs_b(const Geo& g, const double* us, const double* vs, const double* ws,
                          const double* S, double* b, double* red, DevStatus* st, double inv_dt,
                          cudaStream_t s);
-// Loop control of Algorithm 1 (one block).  kexact: recompute the residual
-// exactly every kexact passes (<= 1: every pass); convergence is only
-// accepted on an exact residual.
-cudaError_t launch_check(DevStatus* st, const double* red, int nblk, double rtol, int maxit,
-                         int kexact, cudaStream_t s);
 cudaError_t launch_init_status(DevStatus* st, cudaStream_t s);
 // u = us - dt beta G p on all faces (w walls = 0).
 cudaError_t launch_correct(const Geo& g, const Faces& fc, const double* us, const double* vs,
@@ -358,7 +369,6 @@ cudaError_t launch_correct(const Geo& g, const Faces& fc, const double* us, cons
                            double* w, cudaStream_t s);
 // p -= <p>_V
 cudaError_t launch_remove_mean(const Geo& g, double* p, double* red, DevStatus* st, cudaStream_t s);
-cudaError_t launch_copy_resid_sums(DevStatus* st, const double* red, int nblk, cudaStream_t s);
 
 // Adjoint helpers.
 // y = -dt * beta * W_f^{-1} g on the faces (wall z-faces zero).

@@ -16,14 +16,14 @@ __global__ void __launch_bounds__(256, 4) k_resid_fftx(Geo g, Faces fc, FftDesc 
                                                     const double* __restrict__ p, int mode, int p_zero,
                                                     int scale_rho, C2<T>* __restrict__ spec,
                                                     double* __restrict__ red, int rpb,
-                                                    const DevStatus* __restrict__ st,
+                                                    const DevStatus* st,
                                                     float* __restrict__ E,
-                                                    const float* __restrict__ delta) {
+                                                    const float* __restrict__ delta, LoopCheck ck) {
   if (stopped(st)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const bool need_exact = (st == nullptr) || st->need_exact;
   stage_resid_fftx<T, YS>(g, fc, fx, twx, b, rho, p, mode, p_zero, scale_rho, spec, red, rpb, blockIdx.x,
-                      need_exact, E, delta, smem_raw);
+                      need_exact, E, delta, smem_raw, ck, gridDim.x);
 }
 
 // DCT: the cosine transform of walls in y instead of the periodic DFT.
@@ -144,10 +144,10 @@ __global__ void __launch_bounds__(256) k_fftx_inv(Geo g, FftDesc fx, const C2<T>
 template <typename T>
 cudaError_t launch_resid_fftx(const Geo& g, const Faces& fc, const FftDesc& fx, const C2<T>* twx,
                               const double* b, double inv_dt, const double* rho, const double* p,
-                              int p_zero, int scale_rho, C2<T>* spec, double* red, int* nblk_out,
+                              int p_zero, int scale_rho, C2<T>* spec, double* red, const LoopCheck* ck,
                               const DevStatus* st, cudaStream_t s, float* E, const float* delta) {
-  if (wfft_length(g.nx))
-    return launch_resid_w<T>(g, fc, twx, b, rho, p, p_zero, scale_rho, spec, red, nblk_out, st, s, E, delta);
+  if (wfft_length(g.nx) || (g.nx == 512 && std::is_same<T, float>::value))
+    return launch_resid_w<T>(g, fc, twx, b, rho, p, p_zero, scale_rho, spec, red, ck, st, s, E, delta);
   const int rpb = rows_per_block(g.nx, kEpt);
   const long nrows = (long)g.nz * g.ny;
   const int nblk = (int)((nrows + rpb - 1) / rpb);
@@ -163,8 +163,7 @@ cudaError_t launch_resid_fftx(const Geo& g, const Faces& fc, const FftDesc& fx, 
   const int mode = (red == nullptr) ? 0 : 1;
   (void)inv_dt;
   kern<<<nblk, kThreads, smem, s>>>(g, fc, fx, twx, b, rho, p, mode, p_zero, scale_rho, spec, red, rpb, st, E,
-                                    delta);
-  if (nblk_out) *nblk_out = nblk;
+                                    delta, ck ? *ck : LoopCheck{});
   return cudaGetLastError();
 }
 
@@ -184,19 +183,17 @@ cudaError_t launch_ffty(const Geo& g, const FftDesc& fy, const C2<T>* twy, C2<T>
   const long long ntiles = (long long)((g.nxh + tx - 1) / tx) * g.nz;
   // persistent grid: exactly the blocks that are resident at once (shared
   // memory and registers both counted), so no block waits for a second wave
-  auto kern = dct ? (inverse ? k_ffty<T, 1, true> : k_ffty<T, -1, true>)
-                  : (inverse ? k_ffty<T, 1, false> : k_ffty<T, -1, false>);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  int per_sm = 0, dev = 0, nsm = 0;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem)) != cudaSuccess) return e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if (per_sm < 1) per_sm = 1;
-  long long nblk = (long long)nsm * per_sm;
-  if (nblk > ntiles) nblk = ntiles;
-  kern<<<(int)nblk, kThreads, smem, s>>>(g, fy, twy, spec, tx, ntiles, st, dct);
-  return cudaGetLastError();
+  auto go = [&](auto resident, auto kern) {
+    long long nblk = 0;
+    const cudaError_t e = resident(&nblk);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)(nblk < ntiles ? nblk : ntiles), kThreads, smem, s>>>(g, fy, twy, spec, tx, ntiles, st, dct);
+    return cudaGetLastError();
+  };
+#define PP_GO(...) go([&](long long* n) { return resident_blocks<__VA_ARGS__>(kThreads, smem, n); }, __VA_ARGS__)
+  if (dct) return inverse ? PP_GO(k_ffty<T, 1, true>) : PP_GO(k_ffty<T, -1, true>);
+  return inverse ? PP_GO(k_ffty<T, 1, false>) : PP_GO(k_ffty<T, -1, false>);
+#undef PP_GO
 }
 
 template <typename T>
@@ -327,7 +324,7 @@ cudaError_t launch_fftx_inv(const Geo& g, const FftDesc& fx, const C2<T>* twx, c
 #define PP_INST(T)                                                                                   \
   template cudaError_t launch_resid_fftx<T>(const Geo&, const Faces&, const FftDesc&, const C2<T>*,  \
                                             const double*, double, const double*, const double*,     \
-                                            int, int, C2<T>*, double*, int*, const DevStatus*,       \
+                                            int, int, C2<T>*, double*, const LoopCheck*, const DevStatus*, \
                                             cudaStream_t, float*, const float*);                    \
   template cudaError_t launch_ffty<T>(const Geo&, const FftDesc&, const C2<T>*, C2<T>*, int,         \
                                       const DevStatus*, cudaStream_t, const C2<T>*);                 \

@@ -145,19 +145,13 @@ cudaError_t launch_fftx512_inv(const Geo& g, const float2* twx, const float2* sp
                                int p_zero, const DevStatus* st, cudaStream_t s, float* delta, float* sdelta) {
   if (g.nxh != kXNh) return cudaErrorInvalidValue;
   const size_t smem = R512<kXLines>::smem_bytes() + (size_t)2 * kXLines * kXStageRow * sizeof(float2);
-  cudaError_t e = cudaFuncSetAttribute(k_fftx512_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   const long long nrows = (long long)g.nz * g.ny;
   const long long ngroups = (nrows + 2 * kXLines - 1) / (2 * kXLines);
-  int per_sm = 0, dev = 0, nsm = 0;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fftx512_inv, 64 * kXLines, smem)) != cudaSuccess)
-    return e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if (per_sm < 1) per_sm = 1;
-  long long nblk = (long long)nsm * per_sm;
-  if (nblk > ngroups) nblk = ngroups;
-  k_fftx512_inv<<<(int)nblk, 64 * kXLines, smem, s>>>(g, twx, spec, scale, p, p_zero, ngroups, st, delta, sdelta);
+  long long nblk = 0;
+  const cudaError_t e = resident_blocks<k_fftx512_inv>(64 * kXLines, smem, &nblk);
+  if (e != cudaSuccess) return e;
+  k_fftx512_inv<<<(unsigned)(nblk < ngroups ? nblk : ngroups), 64 * kXLines, smem, s>>>(
+      g, twx, spec, scale, p, p_zero, ngroups, st, delta, sdelta);
   return cudaGetLastError();
 }
 

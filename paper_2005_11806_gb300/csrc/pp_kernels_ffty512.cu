@@ -63,18 +63,13 @@ cudaError_t launch_ffty512(const Geo& g, const float2* twy, float2* spec, int in
                            cudaStream_t s) {
   constexpr int TX = kFfty512Tx;
   const size_t smem = R512<TX>::smem_bytes();
-  auto kern = inverse ? k_ffty512<1, TX> : k_ffty512<-1, TX>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   const long long ntiles = (long long)((g.nxh + TX - 1) / TX) * g.nz;
-  int per_sm = 0, dev = 0, nsm = 0;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 64 * TX, smem)) != cudaSuccess) return e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if (per_sm < 1) per_sm = 1;
-  long long nblk = (long long)nsm * per_sm;
-  if (nblk > ntiles) nblk = ntiles;
-  kern<<<(int)nblk, 64 * TX, smem, s>>>(g, twy, spec, ntiles, st);
+  long long nblk = 0;
+  const cudaError_t e = inverse ? resident_blocks<k_ffty512<1, TX>>(64 * TX, smem, &nblk)
+                                : resident_blocks<k_ffty512<-1, TX>>(64 * TX, smem, &nblk);
+  if (e != cudaSuccess) return e;
+  auto kern = inverse ? k_ffty512<1, TX> : k_ffty512<-1, TX>;
+  kern<<<(unsigned)(nblk < ntiles ? nblk : ntiles), 64 * TX, smem, s>>>(g, twy, spec, ntiles, st);
   return cudaGetLastError();
 }
 

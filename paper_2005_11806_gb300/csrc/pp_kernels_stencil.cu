@@ -89,22 +89,6 @@ __global__ void k_rhs_b(Geo g, const double* __restrict__ us, const double* __re
 
 __global__ void k_init_status(DevStatus* st) { status_init(st); }
 
-// Loop control of Algorithm 1: reduce the residual partial sums, decide.
-__global__ void k_check(DevStatus* st, const double* __restrict__ red, int nblk, double rtol, int maxit,
-                        int kexact) {
-  __shared__ double sh[32];
-  if (st->done) return;
-  double s2 = 0.0, s1 = 0.0;
-  for (int b = threadIdx.x; b < nblk; b += blockDim.x) {
-    s2 += red[2 * (size_t)b];
-    s1 += red[2 * (size_t)b + 1];
-  }
-  s2 = block_sum<double>(s2, sh);
-  s1 = block_sum<double>(s1, sh);
-  if (threadIdx.x != 0) return;
-  status_update(st, s2, s1, rtol, maxit, kexact);
-}
-
 // u = u* - dt beta G p  (Eq. corr); w wall planes are written as zero.
 __global__ void k_correct(Geo g, Faces fc, const double* __restrict__ us, const double* __restrict__ vs,
                           const double* __restrict__ ws, const double* __restrict__ p, double dt,
@@ -620,12 +604,6 @@ cudaError_t launch_rhs_b(const Geo& g, const double* us, const double* vs, const
   return cudaGetLastError();
 }
 
-cudaError_t launch_check(DevStatus* st, const double* red, int nblk, double rtol, int maxit,
-                         int kexact, cudaStream_t s) {
-  k_check<<<1, 1024, 0, s>>>(st, red, nblk, rtol, maxit, kexact);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_init_status(DevStatus* st, cudaStream_t s) {
   k_init_status<<<1, 1, 0, s>>>(st);
   return cudaGetLastError();
@@ -743,7 +721,5 @@ cudaError_t launch_adj_grho(const Geo& g, const double* tx, const double* ty, co
   k_adj_grho<<<grid_for((size_t)g.nx * g.ny * g.nz), kThreads, 0, s>>>(g, tx, ty, tz, grho);
   return cudaGetLastError();
 }
-
-cudaError_t launch_copy_resid_sums(DevStatus*, const double*, int, cudaStream_t) { return cudaSuccess; }
 
 }  // namespace pp

@@ -8,6 +8,7 @@
 #pragma once
 #include <type_traits>
 
+#include "pp_cells.cuh"
 #include "pp_fft.cuh"
 #include "pp_zsweep.cuh"
 
@@ -134,7 +135,7 @@ __device__ __forceinline__ void load_twiddles_smem(const float2* __restrict__ tw
 //   A delta = 2 [w_x (G_x+ - G_x-) + w_y+ G_y+ - w_y- G_y- + w_z+ G_z+ - w_z- G_z-]
 // with the layer (and row) factors w.  Coefficients formed per cell and face
 // took 131 instructions a cell, 35 of them range checks and selects of the
-// division; this form takes about 80.
+// division; this form takes 89 with the transform.
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ float half_flux(float da, float db, float ha, float hb) {
   return (db - da) * rcp_f32(ha + hb);
@@ -151,21 +152,44 @@ struct RowW {
   float x, yl, yh, zd, zu, iv;
 };
 
-// The four cells of a row at offset c: their E updated in place, their
-// scaled residuals returned, e^2 and |e| added to s2 and s1.  Gl, Gh: the
-// half fluxes of the y faces below and above.
-__device__ __forceinline__ float4 resid_row4(const RowW& w, float* __restrict__ E, const float* __restrict__ delta,
-                                             const float* __restrict__ rhof, unsigned c, unsigned il, unsigned ir,
-                                             unsigned plane, bool up, bool dn, float4 d, float4 h, float4 Gl,
-                                             float4 Gh, bool scale, bool own, float rt_f, float& s2, float& s1) {
-  const float dl = delta[il], dr = delta[ir], hl = rhof[il], hr = rhof[ir];
-  float4 du = d, dd = d, hu = h, hd = h;
-  if (up) { du = ld4(delta + c + plane); hu = ld4(rhof + c + plane); }
-  if (dn) { dd = ld4(delta + c - plane); hd = ld4(rhof + c - plane); }
-  float4 e = ld4(E + c);
-  const float x0 = half_flux(dl, d.x, hl, h.x), x1 = half_flux(d.x, d.y, h.x, h.y), x2 = half_flux(d.y, d.z, h.y, h.z),
-              x3 = half_flux(d.z, d.w, h.z, h.w), x4 = half_flux(d.w, dr, h.w, hr);
-  const float4 Gu = half_flux4(d, du, h, hu), Gd = half_flux4(dd, d, hd, h);
+// What the four cells of a row at offset c need beside their own delta and
+// density: the x neighbours (il, ir), the layers above and below, E.
+struct RowIn {
+  float4 du, hu, dd, hd, e;
+  float dl, dr, hl, hr;
+};
+__device__ __forceinline__ RowIn load_row(const float* __restrict__ E, const float* __restrict__ delta,
+                                          const float* __restrict__ rhof, unsigned c, unsigned il, unsigned ir,
+                                          unsigned plane, bool up, bool dn) {
+  RowIn x;
+  const unsigned cu = up ? c + plane : c, cd = dn ? c - plane : c;  // at a wall: the cell itself, no flux
+  x.e = ld4(E + c);
+  x.du = ld4(delta + cu);
+  x.dd = ld4(delta + cd);
+  x.hu = ld4(rhof + cu);
+  x.hd = ld4(rhof + cd);
+  x.dl = delta[il];
+  x.dr = delta[ir];
+  x.hl = rhof[il];
+  x.hr = rhof[ir];
+  return x;
+}
+// Keeps every load before it in flight together: left to itself the compiler
+// sinks them to their uses, and a thread waits for memory several times in a
+// step (residual 256^3 0.104 -> 0.094 ms, 512^3 0.672 -> 0.644 ms).
+__device__ __forceinline__ void loads_issued() { asm volatile("" ::: "memory"); }
+
+// The four cells of a row: their E updated in place, their scaled residuals
+// returned, e^2 and |e| added to s2 and s1.  Gl, Gh: the half fluxes of the y
+// faces below and above.
+__device__ __forceinline__ float4 resid_row4(const RowW& w, const RowIn& x, float* __restrict__ E, unsigned c, float4 d,
+                                             float4 h, float4 Gl, float4 Gh, bool scale, bool own, float rt_f,
+                                             float& s2, float& s1) {
+  float4 e = x.e;
+  const float x0 = half_flux(x.dl, d.x, x.hl, h.x), x1 = half_flux(d.x, d.y, h.x, h.y),
+              x2 = half_flux(d.y, d.z, h.y, h.z), x3 = half_flux(d.z, d.w, h.z, h.w),
+              x4 = half_flux(d.w, x.dr, h.w, x.hr);
+  const float4 Gu = half_flux4(d, x.du, h, x.hu), Gd = half_flux4(x.dd, d, x.hd, h);
   auto cell = [&](float xm, float xp, float gl, float gh, float gd, float gu, float& ev, float hv) -> float {
     float t = w.x * (xp - xm);
     t = fmaf(w.yh, gh, t);
@@ -244,11 +268,12 @@ __device__ __forceinline__ void resid_update_vec4(const Geo& g, const Faces& fc,
         const unsigned rowoff = (unsigned)row * nx, kp = (unsigned)k * plane, c = rowoff + i;
         const unsigned cyp = kp + (unsigned)jp * nx + i, cym = kp + (unsigned)jm * nx + i;
         const float4 d = ld4(delta + c), hc = ld4(fc.rhof + c);
-        const float4 Gl = half_flux4(ld4(delta + cym), d, ld4(fc.rhof + cym), hc);
-        const float4 Gh = half_flux4(d, ld4(delta + cyp), hc, ld4(fc.rhof + cyp));
-        rr[h] = resid_row4(row_factors<YS>(g, k, j), E, delta, fc.rhof, c, rowoff + (i == 0 ? nx - 1 : i - 1),
-                           rowoff + (i + 4 == nx ? 0 : i + 4), plane, k + 1 < nz, k > 0, d, hc, Gl, Gh, scale, own,
-                           rt_f, s2, s1);
+        const float4 dm = ld4(delta + cym), hm = ld4(fc.rhof + cym), dp = ld4(delta + cyp), hp = ld4(fc.rhof + cyp);
+        const RowIn in = load_row(E, delta, fc.rhof, c, rowoff + (i == 0 ? nx - 1 : i - 1),
+                                  rowoff + (i + 4 == nx ? 0 : i + 4), plane, k + 1 < nz, k > 0);
+        loads_issued();
+        rr[h] = resid_row4(row_factors<YS>(g, k, j), in, E, c, d, hc, half_flux4(dm, d, hm, hc),
+                           half_flux4(d, dp, hc, hp), scale, own, rt_f, s2, s1);
       }
     }
     float4* dst = reinterpret_cast<float4*>(bufA + qp * seq_stride + i);
@@ -291,18 +316,18 @@ __device__ __forceinline__ void resid_update_pair4(const Geo& g, const Faces& fc
       const unsigned cm = kp + (unsigned)jm * nx + i, cp = kp + (unsigned)jpp * nx + i;
       const int il = (i == 0) ? nx - 1 : i - 1, ir = (i + 4 == nx) ? 0 : i + 4;
       const bool up = k + 1 < nz, dn = k > 0;
+      const float4 dA = ld4(delta + ca), dB = ld4(delta + cb);
+      const float4 hA = ld4(fc.rhof + ca), hB = ld4(fc.rhof + cb);
+      const float4 dM = ld4(delta + cm), hM = ld4(fc.rhof + cm), dP = ld4(delta + cp), hP = ld4(fc.rhof + cp);
+      const RowIn inA = load_row(E, delta, fc.rhof, ca, oa + il, oa + ir, plane, up, dn);
+      const RowIn inB = load_row(E, delta, fc.rhof, cb, ob + il, ob + ir, plane, up, dn);
       RowW wa = row_factors<YS>(g, k, j), wb = wa;
       if constexpr (YS) wb = row_factors<YS>(g, k, j + 1);
       else { wb.yl = wa.yh; wb.yh = (g.ywall && j + 2 == ny) ? 0.f : wa.yh; }
-      const float4 dA = ld4(delta + ca), dB = ld4(delta + cb);
-      const float4 hA = ld4(fc.rhof + ca), hB = ld4(fc.rhof + cb);
+      loads_issued();
       const float4 Gm = half_flux4(dA, dB, hA, hB);
-      const float4 Gl = half_flux4(ld4(delta + cm), dA, ld4(fc.rhof + cm), hA);
-      ra = resid_row4(wa, E, delta, fc.rhof, ca, oa + il, oa + ir, plane, up, dn, dA, hA, Gl, Gm, scale, own, rt_f,
-                      s2, s1);
-      const float4 Gh = half_flux4(dB, ld4(delta + cp), hB, ld4(fc.rhof + cp));
-      rb = resid_row4(wb, E, delta, fc.rhof, cb, ob + il, ob + ir, plane, up, dn, dB, hB, Gm, Gh, scale, own, rt_f,
-                      s2, s1);
+      ra = resid_row4(wa, inA, E, ca, dA, hA, half_flux4(dM, dA, hM, hA), Gm, scale, own, rt_f, s2, s1);
+      rb = resid_row4(wb, inB, E, cb, dB, hB, Gm, half_flux4(dB, dP, hB, hP), scale, own, rt_f, s2, s1);
     }
     float4* dst = reinterpret_cast<float4*>(bufA + qp * seq_stride + i);
     dst[0] = make_float4(ra.x, rb.x, ra.y, rb.y);
@@ -509,6 +534,56 @@ __device__ __forceinline__ void resid_rows(const Geo& g, const Faces& fc, const 
   }
 }
 
+// The last steps of a residual kernel, by one warp of each block after its
+// block's partial sums are in red[2 blk + {0, 1}] (written by lane 0): the last
+// block of each group adds the group's pairs, the last group adds the groups'
+// and runs the loop control.  Every sum runs in a fixed order.  No block waits
+// for another.  (A kernel of one block reduced the sums before: 0.004 to
+// 0.028 ms and a launch a pass.)
+__device__ __forceinline__ void resid_ticket(const LoopCheck& ck, const double* red, unsigned blk, unsigned nblk) {
+  constexpr unsigned full = 0xffffffffu;
+  const unsigned lane = threadIdx.x & 31u;
+  const unsigned ngrp = (nblk + kCheckGroup - 1) / kCheckGroup, grp = blk / kCheckGroup;
+  const unsigned first = grp * kCheckGroup, n = min((unsigned)kCheckGroup, nblk - first);
+  auto last_of = [&](unsigned* t, unsigned count) {  // lane 0's earlier writes are visible to the last one
+    unsigned last = 0u;
+    if (lane == 0u) {
+      unsigned before;
+      asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(before) : "l"(t) : "memory");
+      last = before == count - 1u ? 1u : 0u;
+      if (last) *t = 0u;  // nobody else arrives in this launch
+    }
+    last = __shfl_sync(full, last, 0);
+    __syncwarp();
+    return last != 0u;
+  };
+  auto sum2 = [&](const double* src, unsigned count, double& a, double& b) {
+    a = b = 0.0;
+    for (unsigned i = lane; i < count; i += 32u) {
+      a += __ldcg(src + 2 * (size_t)i);
+      b += __ldcg(src + 2 * (size_t)i + 1);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      a += __shfl_xor_sync(full, a, o);
+      b += __shfl_xor_sync(full, b, o);
+    }
+  };
+  if (!last_of(ck.tick + 1 + grp, n)) return;
+  double a, b;
+  sum2(red + 2 * (size_t)first, n, a, b);
+  if (ngrp == 1u) {
+    if (lane == 0u) status_update(ck.st, a, b, ck.rtol, ck.maxit, ck.kexact);
+    return;
+  }
+  if (lane == 0u) {
+    ck.gsum[2 * (size_t)grp] = a;
+    ck.gsum[2 * (size_t)grp + 1] = b;
+  }
+  if (!last_of(ck.tick, ngrp)) return;
+  sum2(ck.gsum, ngrp, a, b);
+  if (lane == 0u) status_update(ck.st, a, b, ck.rtol, ck.maxit, ck.kexact);
+}
+
 template <typename T, bool YS = false>
 __device__ __forceinline__ void stage_resid_fftx(const Geo& g, const Faces& fc, const FftDesc& fx,
                                                  const C2<T>* __restrict__ twx,
@@ -519,7 +594,8 @@ __device__ __forceinline__ void stage_resid_fftx(const Geo& g, const Faces& fc, 
                                                  double* __restrict__ red, int rpb, int blk,
                                                  bool need_exact, float* __restrict__ E,
                                                  const float* __restrict__ delta,
-                                                 unsigned char* smem_raw) {
+                                                 unsigned char* smem_raw, LoopCheck ck = LoopCheck{},
+                                                 unsigned nblk = 0) {
   __shared__ double shred[64];
   const int nx = g.nx, ny = g.ny, nz = g.nz, nxh = g.nxh;
   const int nseq = rpb >> 1;
@@ -548,6 +624,7 @@ __device__ __forceinline__ void stage_resid_fftx(const Geo& g, const Faces& fc, 
     }
   }
   __syncthreads();
+  if (mode != 0 && ck.st != nullptr && threadIdx.x < 32) resid_ticket(ck, red, (unsigned)blk, nblk);
   const C2<T>* res = nullptr;
   if constexpr (F32) {
     if (fast)

@@ -120,6 +120,7 @@ struct WSplit {
   static constexpr int U1 = (R2 + L - 1) / L, U2 = (R1 + L - 1) / L;
   static constexpr int S = (R2 & 1) ? R2 : R2 + 1;  // odd row stride of E: no bank conflicts on the columns
   static constexpr int LW = 32 / L;                 // lines a warp
+  static constexpr int TW = N;                      // twiddle entries
   // Elements between the lines of a warp.  With 8 threads a line, two lines
   // share a half warp's access and start 8 entries apart modulo 16.
   static constexpr int raw = R1 * S > N ? R1 * S : N;
@@ -153,6 +154,12 @@ PP_WPLAN(192, 16, 12, 16)
 PP_WPLAN(240, 16, 15, 16)
 PP_WPLAN(256, 16, 16, 16)
 #undef PP_WPLAN
+// 512 = 8 x 8 x 8 with 32 threads a line, 16 values each (the x transform of
+// the FP32 residual, wfft512_line): rows of the two exchanges 72 and 73
+// entries apart, twiddle tables as R512.
+template <> struct WPlan<512> {
+  static constexpr int N = 512, L = 32, LW = 1, LS = 8 * 73, TW = 8 * 64 + 64;
+};
 #define PP_WFFT_LENGTHS(X) \
   X(32) X(36) X(40) X(48) X(50) X(54) X(60) X(64) X(72) X(80) X(90) X(96) X(100) X(108) X(120) X(128) X(144) X(150) \
   X(160) X(180) X(192) X(240) X(256)

@@ -1,58 +1,16 @@
 // The x and y kernels of a pass for the lengths of PP_WFFT_LENGTHS
 // (pp_wfft.cuh); the launchers choose them by length.
 #pragma once
+#include "pp_r512.cuh"
 #include "pp_stages.cuh"
 #include "pp_wfft.cuh"
 
 namespace pp {
 
-// ---------------------------------------------------------------------------
-// Residual and forward real x transform (stage_resid_fftx), a warp at a time:
-// a warp computes the rows of its own LW sequences (2 LW rows) into its own
-// shared buffer, transforms and separates them, with warp barriers only, so
-// the stencil's loads of one warp overlap the transforms of the others.  The
-// block kernel (stage_resid_fftx) meets a block barrier after each of its
-// steps, and its smallest unit (2048 values) leaves most SMs without work on
-// small grids.  FP32: bound by the latency of its global loads (40 % of the
-// stalls, issue 56 % busy) and by the instructions of the stencil; FP64: by
-// the FP64 pipe.  Block kernel -> this, ms: mixed 256^3 0.106 -> 0.095,
-// mixed 192 x 160 x 144 0.040 -> 0.025, FP64 128^3 0.138 -> 0.105, FP64 32^3
-// 0.019 -> 0.011.  Measured and dropped: prefetching a later block's rows
-// into L2 (256^3: 0.106), six blocks an SM (256^3 0.092, 192 x 160 x 144
-// 0.027).
-// red: one pair of partial sums per warp.
-template <typename T, bool YS, int N>
-__device__ __forceinline__ void resid_w_body(const Geo& g, const Faces& fc, const C2<T>* __restrict__ twx,
-                                             const double* __restrict__ b, const double* __restrict__ rho,
-                                             const double* __restrict__ p, int mode, int p_zero, int scale_rho,
-                                             C2<T>* __restrict__ spec, double* __restrict__ red, bool need_exact,
-                                             float* __restrict__ E, const float* __restrict__ delta, unsigned blk,
-                                             unsigned char* smem_raw) {
-  using W = WPlan<N>;
-  C2<T>* tw = reinterpret_cast<C2<T>*>(smem_raw);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  C2<T>* buf = tw + N + (size_t)warp * W::LW * W::LS;
-  wfft_load_twiddles<W, T>(tw, twx);
-  const unsigned gw = blk * (blockDim.x >> 5) + warp;
-  const int nrows = g.nz * g.ny;
-  const int nxh = N / 2 + 1;
-  const long row0 = (long)gw * (2 * W::LW);
-  T s2 = (T)0, s1 = (T)0;
-  if (row0 < nrows)
-    resid_rows<T, YS>(g, fc, b, rho, p, mode, p_zero, scale_rho, row0, 2 * W::LW, need_exact, E, delta, buf, W::LS,
-                      s2, s1, lane, 32);
-  __syncthreads();  // twiddles; the warp's rows
-  if (row0 >= nrows) return;
-  if (mode != 0) {
-    for (int o = 16; o > 0; o >>= 1) {
-      s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-    }
-    if (lane == 0) {
-      red[2 * (size_t)gw] = (double)s2;
-      red[2 * (size_t)gw + 1] = (double)s1;
-    }
-  }
+// Forward transform of a warp's lines in place, natural order in and out
+// (buf: LW lines LS entries apart).
+template <class W, typename T>
+__device__ __forceinline__ void wfft_lines(C2<T>* buf, const C2<T>* tw, int lane) {
   const int l = lane & (W::L - 1);
   C2<T>* line = buf + (lane / W::L) * W::LS;
   {
@@ -99,6 +57,122 @@ __device__ __forceinline__ void resid_w_body(const Geo& g, const Faces& fc, cons
     }
   }
   __syncwarp();
+}
+
+// The same for one line of 512 entries: three 8-point stages, two transforms
+// a thread (thread j of pp_r512.cuh is (lane, u): j = lane + 32 u).
+template <int DIR>
+__device__ __forceinline__ void wfft512_line(float2* line, const float2* tw, int lane) {
+  float2 v[2][8];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int j = lane + 32 * u;
+#pragma unroll
+    for (int a = 0; a < 8; ++a) v[u][a] = line[64 * a + j];
+    Dft<float, DIR, 8>::run(v[u]);
+    r512_twiddle8<DIR>(v[u], tw, 64, j);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+#pragma unroll
+    for (int c = 0; c < 8; ++c) line[c * 72 + lane + 32 * u] = v[u][c];
+  __syncwarp();
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int j = lane + 32 * u, c = j >> 3, f = j & 7;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[u][e] = line[c * 72 + 8 * e + f];
+    Dft<float, DIR, 8>::run(v[u]);
+    r512_twiddle8<DIR>(v[u], tw + 512, 8, f);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int j = lane + 32 * u, c = j >> 3, f = j & 7;
+#pragma unroll
+    for (int gg = 0; gg < 8; ++gg) line[c * 73 + gg * 8 + f] = v[u][gg];
+  }
+  __syncwarp();
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int j = lane + 32 * u, c = j & 7, gg = j >> 3;
+#pragma unroll
+    for (int f = 0; f < 8; ++f) v[u][f] = line[c * 73 + gg * 8 + f];
+    Dft<float, DIR, 8>::run(v[u]);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+#pragma unroll
+    for (int h = 0; h < 8; ++h) line[lane + 32 * u + 64 * h] = v[u][h];
+  __syncwarp();
+}
+
+// ---------------------------------------------------------------------------
+// Residual and forward real x transform (stage_resid_fftx), a warp at a time:
+// a warp computes the rows of its own LW sequences (2 LW rows) into its own
+// shared buffer, transforms and separates them, with warp barriers only, so
+// the stencil's loads of one warp overlap the transforms of the others.  The
+// block kernel (stage_resid_fftx) meets a block barrier after each of its
+// steps, and its smallest unit (2048 values) leaves most SMs without work on
+// small grids.  FP32: bound by the latency of its global loads (half of the
+// stalls, issue 45 % busy, DRAM 39 % at 256^3); FP64: by the FP64 pipe.  Block
+// kernel and loop-control kernel -> this, ms: mixed 256^3 0.114 -> 0.094, mixed
+// 512^3 0.805 -> 0.644, mixed 192 x 160 x 144 0.046 -> 0.029, FP64 128^3 0.142
+// -> 0.106, FP64 32^3 0.023 -> 0.016.  Measured and dropped: prefetching a later
+// block's rows into L2 (256^3: 0.106); four and three blocks an SM (192 x 160 x
+// 144 0.034, 0.038), six (256^3 gains 3 %, 192 x 160 x 144 loses 8 %).
+// red: one pair of partial sums per block.
+template <typename T, bool YS, int N>
+__device__ __forceinline__ void resid_w_body(const Geo& g, const Faces& fc, const C2<T>* __restrict__ twx,
+                                             const double* __restrict__ b, const double* __restrict__ rho,
+                                             const double* __restrict__ p, int mode, int p_zero, int scale_rho,
+                                             C2<T>* __restrict__ spec, double* __restrict__ red, bool need_exact,
+                                             float* __restrict__ E, const float* __restrict__ delta, unsigned blk,
+                                             unsigned char* smem_raw, const LoopCheck& ck, unsigned nblk) {
+  using W = WPlan<N>;
+  __shared__ T shs[16];  // the warps' sums
+  C2<T>* tw = reinterpret_cast<C2<T>*>(smem_raw);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  C2<T>* buf = tw + W::TW + (size_t)warp * W::LW * W::LS;
+  if constexpr (N == 512) r512_load_twiddles(tw, twx);
+  else wfft_load_twiddles<W, T>(tw, twx);
+  const unsigned gw = blk * (blockDim.x >> 5) + warp;
+  const int nrows = g.nz * g.ny;
+  const int nxh = N / 2 + 1;
+  const long row0 = (long)gw * (2 * W::LW);
+  T s2 = (T)0, s1 = (T)0;
+  if (row0 < nrows)
+    resid_rows<T, YS>(g, fc, b, rho, p, mode, p_zero, scale_rho, row0, 2 * W::LW, need_exact, E, delta, buf, W::LS,
+                      s2, s1, lane, 32);
+  if (mode != 0) {
+    for (int o = 16; o > 0; o >>= 1) {
+      s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+    }
+    if (lane == 0) {
+      shs[warp] = s2;
+      shs[8 + warp] = s1;
+    }
+  }
+  __syncthreads();  // twiddles, the warps' sums
+  if (mode != 0 && warp == 0) {
+    if (lane == 0) {
+      T a = (T)0, c = (T)0;
+      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+        a += shs[w];
+        c += shs[8 + w];
+      }
+      red[2 * (size_t)blk] = (double)a;
+      red[2 * (size_t)blk + 1] = (double)c;
+    }
+    // (at the end of the block instead: the same time)
+    if (ck.st != nullptr) resid_ticket(ck, red, blk, nblk);
+  }
+  if (row0 >= nrows) return;
+  if constexpr (N == 512) wfft512_line<-1>(buf, tw, lane);
+  else wfft_lines<W, T>(buf, tw, lane);
   // 2 A = Z + conj W, 2 B = (Z - conj W)/i of the two rows of each line (kSpecScale)
 #pragma unroll
   for (int q = 0; q < W::LW; ++q) {
@@ -118,12 +192,12 @@ template <typename T, bool YS, int N>
 __global__ void __launch_bounds__(128, sizeof(T) == sizeof(float) ? 5 : 3) k_resid_w(
     Geo g, Faces fc, const C2<T>* __restrict__ twx, const double* __restrict__ b, const double* __restrict__ rho,
     const double* __restrict__ p, int mode, int p_zero, int scale_rho, C2<T>* __restrict__ spec,
-    double* __restrict__ red, const DevStatus* __restrict__ st, float* __restrict__ E,
-    const float* __restrict__ delta) {
+    double* __restrict__ red, const DevStatus* st, float* __restrict__ E, const float* __restrict__ delta,
+    LoopCheck ck) {
   if (stopped(st)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   resid_w_body<T, YS, N>(g, fc, twx, b, rho, p, mode, p_zero, scale_rho, spec, red,
-                         (st == nullptr) || st->need_exact, E, delta, blockIdx.x, smem_raw);
+                         (st == nullptr) || st->need_exact, E, delta, blockIdx.x, smem_raw, ck, gridDim.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -446,21 +520,18 @@ inline int wfft_warps_per_block(long long warps) {
 
 template <typename T, int N>
 cudaError_t launch_resid_w_n(const Geo& g, const Faces& fc, const C2<T>* twx, const double* b, const double* rho,
-                             const double* p, int p_zero, int scale_rho, C2<T>* spec, double* red, int* nblk_out,
-                             const DevStatus* st, cudaStream_t s, float* E, const float* delta) {
+                             const double* p, int p_zero, int scale_rho, C2<T>* spec, double* red,
+                             const LoopCheck* ck, const DevStatus* st, cudaStream_t s, float* E, const float* delta) {
   using W = WPlan<N>;
   const long long nrows = (long long)g.nz * g.ny;
   const long long warps = (nrows + 2 * W::LW - 1) / (2 * W::LW);
   const int wpb = wfft_warps_per_block(warps);
-  const size_t smem = (size_t)(N + wpb * W::LW * W::LS) * sizeof(C2<T>);
+  const size_t smem = (size_t)(W::TW + wpb * W::LW * W::LS) * sizeof(C2<T>);
   auto kern = (g.ym != nullptr) ? k_resid_w<T, true, N> : k_resid_w<T, false, N>;
-  if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  static_assert((W::TW + 4 * W::LW * W::LS) * sizeof(C2<T>) <= 48 * 1024, "fits without the opt-in attribute");
   kern<<<(unsigned)((warps + wpb - 1) / wpb), 32 * wpb, smem, s>>>(g, fc, twx, b, rho, p, red == nullptr ? 0 : 1,
-                                                                  p_zero, scale_rho, spec, red, st, E, delta);
-  if (nblk_out) *nblk_out = (int)warps;
+                                                                  p_zero, scale_rho, spec, red, st, E, delta,
+                                                                  ck ? *ck : LoopCheck{});
   return cudaGetLastError();
 }
 
@@ -472,33 +543,32 @@ cudaError_t launch_fftx_inv_w_n(const Geo& g, const C2<T>* twx, const C2<T>* spe
   const long long warps = (nrows + 2 * W::LW - 1) / (2 * W::LW);
   const int wpb = wfft_warps_per_block(warps);
   const size_t smem = (size_t)(N + wpb * W::LW * W::LS) * sizeof(C2<T>);
-  if (smem > 48 * 1024) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(k_fftx_inv_w<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  static_assert((N + 4 * W::LW * W::LS) * sizeof(C2<T>) <= 48 * 1024, "fits without the opt-in attribute");
   k_fftx_inv_w<T, N><<<(unsigned)((warps + wpb - 1) / wpb), 32 * wpb, smem, s>>>(g, twx, spec, scale, p, p_zero, st,
                                                                                 delta, sdelta);
+  return cudaGetLastError();
+}
+
+template <auto K, typename T, int N>
+cudaError_t launch_ffty_w_k(const Geo& g, const C2<T>* twy, C2<T>* spec, const DevStatus* st, cudaStream_t s,
+                            const C2<T>* dct) {
+  using Y = WyShape<T, N>;
+  const long long ntiles = (long long)((g.nxh + kWyTx - 1) / kWyTx) * g.nz;
+  long long nblk = 0;
+  const cudaError_t e = resident_blocks<K>(Y::threads, Y::smem, &nblk);
+  if (e != cudaSuccess) return e;
+  K<<<(unsigned)(nblk < ntiles ? nblk : ntiles), Y::threads, Y::smem, s>>>(g, twy, spec, ntiles, st, dct);
   return cudaGetLastError();
 }
 
 template <typename T, int N>
 cudaError_t launch_ffty_w_n(const Geo& g, const C2<T>* twy, C2<T>* spec, int inverse, const DevStatus* st,
                             cudaStream_t s, const C2<T>* dct) {
-  using Y = WyShape<T, N>;
-  const long long ntiles = (long long)((g.nxh + kWyTx - 1) / kWyTx) * g.nz;
-  auto kern = dct ? (inverse ? k_ffty_w<T, 1, true, N> : k_ffty_w<T, -1, true, N>)
-                  : (inverse ? k_ffty_w<T, 1, false, N> : k_ffty_w<T, -1, false, N>);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Y::smem);
-  if (e != cudaSuccess) return e;
-  int per_sm = 0, dev = 0, nsm = 0;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, Y::threads, Y::smem)) != cudaSuccess) return e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  long long nblk = (long long)nsm * (per_sm < 1 ? 1 : per_sm);
-  if (nblk > ntiles) nblk = ntiles;
-  kern<<<(unsigned)nblk, Y::threads, Y::smem, s>>>(g, twy, spec, ntiles, st, dct);
-  return cudaGetLastError();
+  if (dct)
+    return inverse ? launch_ffty_w_k<k_ffty_w<T, 1, true, N>, T, N>(g, twy, spec, st, s, dct)
+                   : launch_ffty_w_k<k_ffty_w<T, -1, true, N>, T, N>(g, twy, spec, st, s, dct);
+  return inverse ? launch_ffty_w_k<k_ffty_w<T, 1, false, N>, T, N>(g, twy, spec, st, s, dct)
+                 : launch_ffty_w_k<k_ffty_w<T, -1, false, N>, T, N>(g, twy, spec, st, s, dct);
 }
 
 }  // namespace pp
