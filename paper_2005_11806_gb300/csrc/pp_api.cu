@@ -101,8 +101,9 @@ struct pp_plan_s {
   DevStatus* h_st = nullptr;  // pinned, two slots
   cudaEvent_t ev[2] = {nullptr, nullptr};
   // kGraphPasses passes of the loop as one graph launch (method3_loop): the
-  // capture stream, the executable graph and its kernel launches
-  cudaStream_t cap = nullptr;
+  // executable graph, its kernel launches, and the chain that the launches of
+  // a pass go to while it is built
+  GraphChain* chain = nullptr;
   cudaGraphExec_t gexec = nullptr;
   long long gexec_launches = 0;
   // lazily allocated: host staging (10 face-sized buffers), adjoint scratch
@@ -115,6 +116,8 @@ struct pp_plan_s {
   float* d_mu = nullptr;
   unsigned char* d_za1 = nullptr;
   unsigned char* d_za2 = nullptr;
+
+  Queue queue() const { return Queue(stream, chain); }
 };
 
 namespace {
@@ -301,11 +304,11 @@ pp_status solve_pass(pp_plan_s* P, double* p, int p_zero, T* delta = nullptr, fl
     a.ld = 2LL * P->nxh;
     return a;
   };
-  if (ytc) PP_K(P, K_FFTY_F, launch_dense_tc(ytc_args(spec, zs, P->d_ytc_f), P->d_st, P->stream));
+  if (ytc) PP_K(P, K_FFTY_F, launch_dense_tc(ytc_args(spec, zs, P->d_ytc_f), P->d_st, P->queue()));
   else if (P->ystretch) {
     if constexpr (std::is_same<T, double>::value)
-      PP_K(P, K_FFTY_F, launch_ydense(g, (const double*)P->d_ymt_f, spec, P->d_st, P->stream));
-  } else PP_K(P, K_FFTY_F, launch_ffty<T>(g, P->fy, twy, spec, 0, P->d_st, P->stream, dct));
+      PP_K(P, K_FFTY_F, launch_ydense(g, (const double*)P->d_ymt_f, spec, P->d_st, P->queue()));
+  } else PP_K(P, K_FFTY_F, launch_ffty<T>(g, P->fy, twy, spec, 0, P->d_st, P->queue(), dct));
   if (P->z_tc) {
     // z expansion on the tensor cores: zs -> the other spectrum buffer with
     // the eigenvalue divide, then back
@@ -326,32 +329,32 @@ pp_status solve_pass(pp_plan_s* P, double* p, int p_zero, T* delta = nullptr, fl
     a.lamy = P->d_lamy;
     a.nxh = P->nxh;
     a.zero_mode = P->ze.zero_mode;
-    PP_K(P, K_TRI, launch_dense_tc(a, P->d_st, P->stream));
+    PP_K(P, K_TRI, launch_dense_tc(a, P->d_st, P->queue()));
     a.x = other;
     a.y = (float*)zs;
     a.mat = P->ze.a2;
     a.mu = nullptr;
-    PP_K(P, K_TRI, launch_dense_tc(a, P->d_st, P->stream));
+    PP_K(P, K_TRI, launch_dense_tc(a, P->d_st, P->queue()));
   } else if (P->zsolve == PP_ZSOLVE_COSINE) {
     if constexpr (std::is_same<T, double>::value) {
       const ZDivide zd{P->d_lamx, P->d_lamy, P->d_lamz};
-      PP_K(P, K_ZDCT_F, launch_zdct<double>(g, P->fz, P->d_twz, zs, 0, P->d_st, P->stream, P->d_dctz, zd));
-      PP_K(P, K_ZDCT_I, launch_zdct<double>(g, P->fz, P->d_twz, zs, 1, P->d_st, P->stream, P->d_dctz, zd));
+      PP_K(P, K_ZDCT_F, launch_zdct<double>(g, P->fz, P->d_twz, zs, 0, P->d_st, P->queue(), P->d_dctz, zd));
+      PP_K(P, K_ZDCT_I, launch_zdct<double>(g, P->fz, P->d_twz, zs, 1, P->d_st, P->queue(), P->d_dctz, zd));
     } else {
       return PP_ERR_UNSUPPORTED;
     }
   } else if (P->use_z) {
     const TriZ<T> tz{P->d_zm, P->d_ze, (const T*)P->d_zd, P->z_nyt, P->z_ysym};
-    PP_K(P, K_TRI, launch_zsolve<T>(g, tz, zs, P->d_st, P->stream));
+    PP_K(P, K_TRI, launch_zsolve<T>(g, tz, zs, P->d_st, P->queue()));
   } else {
-    PP_K(P, K_TRI, launch_tridiag<T>(g, P->d_invd, zs, nullptr, P->d_st, P->stream, P->d_mtab, &P->tri32));
+    PP_K(P, K_TRI, launch_tridiag<T>(g, P->d_invd, zs, nullptr, P->d_st, P->queue(), P->d_mtab, &P->tri32));
   }
-  if (ytc) PP_K(P, K_FFTY_I, launch_dense_tc(ytc_args(zs, spec, P->d_ytc_i), P->d_st, P->stream));
+  if (ytc) PP_K(P, K_FFTY_I, launch_dense_tc(ytc_args(zs, spec, P->d_ytc_i), P->d_st, P->queue()));
   else if (P->ystretch) {
     if constexpr (std::is_same<T, double>::value)
-      PP_K(P, K_FFTY_I, launch_ydense(g, (const double*)P->d_ymt_i, spec, P->d_st, P->stream));
-  } else PP_K(P, K_FFTY_I, launch_ffty<T>(g, P->fy, twy, spec, 1, P->d_st, P->stream, dct));
-  PP_K(P, K_FFTX_I, launch_fftx_inv<T>(g, P->fx, twx, spec, scale, p, p_zero, P->d_st, P->stream, delta,
+      PP_K(P, K_FFTY_I, launch_ydense(g, (const double*)P->d_ymt_i, spec, P->d_st, P->queue()));
+  } else PP_K(P, K_FFTY_I, launch_ffty<T>(g, P->fy, twy, spec, 1, P->d_st, P->queue(), dct));
+  PP_K(P, K_FFTX_I, launch_fftx_inv<T>(g, P->fx, twx, spec, scale, p, p_zero, P->d_st, P->queue(), delta,
                                        sdelta));
   return PP_OK;
 }
@@ -369,39 +372,32 @@ template <> double* increment_buffer<double>(pp_plan_s* P, bool) {
 constexpr int kGraphPasses = 4;  // passes of one graph launch, and between polls
 constexpr int kGraphAfter = 8;   // passes launched one by one first
 
-// The passes body() issues on P->stream, captured on the plan's own stream and
-// put into P->gexec (updated in place when only arguments changed).  False:
-// no graph (nothing was launched).
+// The launches of kGraphPasses calls of body() as the nodes of P->gexec
+// (updated in place when only arguments changed).  False: no graph (nothing
+// was launched).
 template <class F>
-bool capture_passes(pp_plan_s* P, F&& body) {
-  if (P->cap == nullptr && cudaStreamCreateWithFlags(&P->cap, cudaStreamNonBlocking) != cudaSuccess) {
-    P->cap = nullptr;
-    (void)cudaGetLastError();
-    return false;
-  }
+bool build_passes(pp_plan_s* P, F&& body) {
   const long long before = P->prof.launches;
-  cudaStream_t own = P->stream;
-  cudaGraph_t graph = nullptr;
-  bool ok = cudaStreamBeginCapture(P->cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+  GraphChain chain{nullptr, nullptr};
+  bool ok = cudaGraphCreate(&chain.graph, 0) == cudaSuccess;
   if (ok) {
-    P->stream = P->cap;
+    P->chain = &chain;
     for (int q = 0; q < kGraphPasses && ok; ++q) ok = body() == PP_OK;
-    P->stream = own;
-    ok = cudaStreamEndCapture(P->cap, &graph) == cudaSuccess && ok && graph != nullptr;
+    P->chain = nullptr;
   }
   P->gexec_launches = P->prof.launches - before;
   P->prof.launches = before;
   if (ok && P->gexec != nullptr) {
     cudaGraphExecUpdateResultInfo info;
-    if (cudaGraphExecUpdate(P->gexec, graph, &info) != cudaSuccess) {
+    if (cudaGraphExecUpdate(P->gexec, chain.graph, &info) != cudaSuccess) {
       (void)cudaGetLastError();
-      cudaStreamSynchronize(own);  // earlier launches of the old one
+      cudaStreamSynchronize(P->stream);  // earlier launches of the old one
       cudaGraphExecDestroy(P->gexec);
       P->gexec = nullptr;
     }
   }
-  if (ok && P->gexec == nullptr) ok = cudaGraphInstantiate(&P->gexec, graph, 0) == cudaSuccess;
-  if (graph != nullptr) cudaGraphDestroy(graph);
+  if (ok && P->gexec == nullptr) ok = cudaGraphInstantiate(&P->gexec, chain.graph, 0) == cudaSuccess;
+  if (chain.graph != nullptr) cudaGraphDestroy(chain.graph);
   if (!ok) {
     if (P->gexec != nullptr) cudaGraphExecDestroy(P->gexec);
     P->gexec = nullptr;
@@ -414,7 +410,7 @@ bool capture_passes(pp_plan_s* P, F&& body) {
 // hold beta of rho.  p is the iterate (zeroed by the caller unless warm).
 // With P->method = I or II the same loop runs with the constant scaling.
 // After kGraphAfter passes the passes are launched kGraphPasses at a time as
-// one graph, captured while those first passes run: a launch costs the host
+// one graph, built while those first passes run: a launch costs the host
 // more than a small grid's kernel takes.  Single launches -> graphs, ms a pass:
 // FP64 32^3 0.056 -> 0.045, mixed 192 x 160 x 144 0.102 -> 0.090, mixed 256^3
 // 0.300 -> 0.287.
@@ -432,19 +428,19 @@ pp_status method3_loop(pp_plan_s* P, const double* rho, double* p, int warm, dou
   auto one_pass = [&](int p_zero) -> pp_status {
     const LoopCheck ck{P->d_st, P->d_tick, P->d_gsum, rtol, maxit, kexact};
     PP_K(P, K_RESID, launch_resid_fftx<T>(g, P->faces, P->fx, twx, P->d_b, inv_dt, rho, p, p_zero, 1, spec, P->d_red,
-                                          &ck, P->d_st, P->stream, upd ? P->d_E : nullptr,
+                                          &ck, P->d_st, P->queue(), upd ? P->d_E : nullptr,
                                           upd ? P->d_delta : nullptr));
     return solve_pass<T>(P, p, 0, dl, upd ? P->d_sdelta : nullptr);
   };
   int polled = 0;
   bool pending[2] = {false, false};
-  bool graph = !P->prof.on, captured = false;
+  bool graph = !P->prof.on, built = false;
   for (int it = 0; it <= maxit;) {
-    if (graph && it >= kGraphAfter && !captured) {
-      captured = capture_passes(P, [&]() { return one_pass(0); });
-      graph = captured;
+    if (graph && it >= kGraphAfter && !built) {
+      built = build_passes(P, [&]() { return one_pass(0); });
+      graph = built;
     }
-    if (captured) {
+    if (built) {
       PP_CK(cudaGraphLaunch(P->gexec, P->stream));
       P->prof.launches += P->gexec_launches;
       it += kGraphPasses;  // passes past maxit find the loop stopped
@@ -546,7 +542,6 @@ void free_plan(pp_plan_s* P) {
   if (P->h_st) cudaFreeHost(P->h_st);
   for (auto& e : P->ev) if (e) cudaEventDestroy(e);
   if (P->gexec) cudaGraphExecDestroy(P->gexec);
-  if (P->cap) cudaStreamDestroy(P->cap);
   for (double* d : P->d_stage) if (d) cudaFree(d);
   for (double* d : P->d_adj) if (d) cudaFree(d);
   for (auto& r : P->prof.rec) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }

@@ -418,17 +418,16 @@ bool encode_view_map(const DenseTcArgs& a, CUtensorMap* map) {
 
 template <bool TMA>
 cudaError_t launch_dense_tc_t(const DenseTcArgs& a, const CUtensorMap& map, int grid, DevStatus* st,
-                              cudaStream_t s) {
+                              Queue s) {
   cudaError_t e = cudaFuncSetAttribute(k_dense_tc<TMA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)Cfg<TMA>::smem);
   if (e != cudaSuccess) return e;
-  k_dense_tc<TMA><<<grid, kThreadsTC, Cfg<TMA>::smem, s>>>(a, map, st);
-  return cudaGetLastError();
+  return enqueue(s, k_dense_tc<TMA>, grid, kThreadsTC, Cfg<TMA>::smem, a, map, st);
 }
 
 }  // namespace
 
-cudaError_t launch_dense_tc(const DenseTcArgs& a, DevStatus* st, cudaStream_t s) {
+cudaError_t launch_dense_tc(const DenseTcArgs& a, DevStatus* st, Queue s) {
   int dev = 0, nsm = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

@@ -212,29 +212,29 @@ template <typename T>
 cudaError_t launch_resid_fftx(const Geo& g, const Faces& fc, const FftDesc& fx, const C2<T>* twx,
                               const double* b, double inv_dt, const double* rho, const double* p,
                               int p_zero, int scale_rho, C2<T>* spec, double* red, const LoopCheck* ck,
-                              const DevStatus* st, cudaStream_t s, float* E = nullptr,
+                              const DevStatus* st, Queue s, float* E = nullptr,
                               const float* delta = nullptr);
 // The same steps for the lengths of PP_WFFT_LENGTHS (pp_wfft.cuh); the
 // launchers route such plans to them.
 template <typename T>
 cudaError_t launch_resid_w(const Geo& g, const Faces& fc, const C2<T>* twx, const double* b, const double* rho,
                            const double* p, int p_zero, int scale_rho, C2<T>* spec, double* red, const LoopCheck* ck,
-                           const DevStatus* st, cudaStream_t s, float* E, const float* delta);
+                           const DevStatus* st, Queue s, float* E, const float* delta);
 template <typename T>
 cudaError_t launch_ffty_w(const Geo& g, const C2<T>* twy, C2<T>* spec, int inverse, const DevStatus* st,
-                          cudaStream_t s, const C2<T>* dct);
+                          Queue s, const C2<T>* dct);
 template <typename T>
 cudaError_t launch_fftx_inv_w(const Geo& g, const C2<T>* twx, const C2<T>* spec, double scale, double* p, int p_zero,
-                              const DevStatus* st, cudaStream_t s, T* delta, float* sdelta);
+                              const DevStatus* st, Queue s, T* delta, float* sdelta);
 template <> cudaError_t launch_resid_w<float>(const Geo&, const Faces&, const C2<float>*, const double*, const double*,
                                             const double*, int, int, C2<float>*, double*, const LoopCheck*, const DevStatus*,
-                                            cudaStream_t, float*, const float*);
-template <> cudaError_t launch_ffty_w<float>(const Geo&, const C2<float>*, C2<float>*, int, const DevStatus*, cudaStream_t,
+                                            Queue, float*, const float*);
+template <> cudaError_t launch_ffty_w<float>(const Geo&, const C2<float>*, C2<float>*, int, const DevStatus*, Queue,
                                            const C2<float>*);
 template <> cudaError_t launch_resid_w<double>(const Geo&, const Faces&, const C2<double>*, const double*, const double*,
                                             const double*, int, int, C2<double>*, double*, const LoopCheck*, const DevStatus*,
-                                            cudaStream_t, float*, const float*);
-template <> cudaError_t launch_ffty_w<double>(const Geo&, const C2<double>*, C2<double>*, int, const DevStatus*, cudaStream_t,
+                                            Queue, float*, const float*);
+template <> cudaError_t launch_ffty_w<double>(const Geo&, const C2<double>*, C2<double>*, int, const DevStatus*, Queue,
                                            const C2<double>*);
 // z solve of a uniform walled z by the cosine basis (FP64 plans): forward
 // transform with the eigenvalue divide (inverse = 0), then the inverse
@@ -246,17 +246,17 @@ struct ZDivide {
 };
 template <typename T>
 cudaError_t launch_zdct(const Geo& g, const FftDesc& fz, const C2<T>* twz, C2<T>* spec, int inverse,
-                        const DevStatus* st, cudaStream_t s, const C2<T>* dct, const ZDivide& zd);
+                        const DevStatus* st, Queue s, const C2<T>* dct, const ZDivide& zd);
 
 // dct: the cosine-transform twiddles exp(-i pi m / (2 ny)) for walls in y,
 // or null for the periodic DFT.
 template <typename T>
 cudaError_t launch_ffty(const Geo& g, const FftDesc& fy, const C2<T>* twy, C2<T>* spec, int inverse,
-                        const DevStatus* st, cudaStream_t s, const C2<T>* dct = nullptr);
+                        const DevStatus* st, Queue s, const C2<T>* dct = nullptr);
 // FP32 y transform of length 512 (periodic y) with the data in registers
 // (pp_kernels_ffty512.cu); launch_ffty routes such plans to it.
 cudaError_t launch_ffty512(const Geo& g, const float2* twy, float2* spec, int inverse, const DevStatus* st,
-                           cudaStream_t s);
+                           Queue s);
 // FP32 Thomas tables for the well-conditioned z columns of mixed plans.  A
 // column (kx, ky) has the shift lambda = lambda_x(kx) + lambda_y(ky) <= 0;
 // the eigenvalues of its system lie in [lambda - 2 Dmax, lambda] with
@@ -286,7 +286,7 @@ int tri_mixed_blocks(size_t ncol, int nlow);
 // values; may alias spec).
 template <typename T>
 cudaError_t launch_tridiag(const Geo& g, const double* invd, C2<T>* spec, double2* ybuf,
-                           const DevStatus* st, cudaStream_t s, const double* mtab = nullptr,
+                           const DevStatus* st, Queue s, const double* mtab = nullptr,
                            const TriF32* f32 = nullptr);
 // z solve of FP64 and PP_MIXED_Z64 plans: FP64 recurrences in every (kx, ky)
 // column, values stored in the spectrum's precision T.  Thomas elimination
@@ -313,7 +313,7 @@ template <typename T>
 cudaError_t launch_setup_z(const Geo& g, const double* lamx, const double* lamy, int nyt, double* m, double* e,
                            T* d, cudaStream_t s);
 template <typename T>
-cudaError_t launch_zsolve(const Geo& g, const TriZ<T>& t, C2<T>* spec, const DevStatus* st, cudaStream_t s);
+cudaError_t launch_zsolve(const Geo& g, const TriZ<T>& t, C2<T>* spec, const DevStatus* st, Queue s);
 // dst[i] = (float) src[i], i < n.
 cudaError_t launch_narrow(const double* src, float* dst, size_t n, cudaStream_t s);
 // Inverse x-transform; p = scale * z (p_zero) or p += scale * z; when delta
@@ -324,12 +324,12 @@ cudaError_t launch_narrow(const double* src, float* dst, size_t n, cudaStream_t 
 // loop has stopped.
 template <typename T>
 cudaError_t launch_fftx_inv(const Geo& g, const FftDesc& fx, const C2<T>* twx, const C2<T>* spec,
-                            double scale, double* p, int p_zero, const DevStatus* st, cudaStream_t s,
+                            double scale, double* p, int p_zero, const DevStatus* st, Queue s,
                             T* delta = nullptr, float* sdelta = nullptr);
 // The same for FP32 spectra of length nx = 512, with the transform in
 // registers (pp_kernels_fftx512.cu); launch_fftx_inv routes such plans to it.
 cudaError_t launch_fftx512_inv(const Geo& g, const float2* twx, const float2* spec, double scale, double* p,
-                               int p_zero, const DevStatus* st, cudaStream_t s, float* delta, float* sdelta);
+                               int p_zero, const DevStatus* st, Queue s, float* delta, float* sdelta);
 cudaError_t launch_fold_pending(const Geo& g, double* p, const float* sdelta, const DevStatus* st,
                                 cudaStream_t s);
 
@@ -406,7 +406,7 @@ int reduce_blocks();  // number of partial sums the reduction kernels write
 // (back); mt holds M transposed, mt[j * ny + m] = M[m][j]
 // (pp_kernels_ydense.cu).  ny <= 1024.  Mixed plans take the tensor-core
 // dense transform (launch_dense_tc) instead.
-cudaError_t launch_ydense(const Geo& g, const double* mt, double2* spec, const DevStatus* st, cudaStream_t s);
+cudaError_t launch_ydense(const Geo& g, const double* mt, double2* spec, const DevStatus* st, Queue s);
 
 // Host: eigenpairs of a symmetric tridiagonal S (diagonal d, off-diagonal e)
 // by Sturm-sequence bisection and inverse iteration with Gram-Schmidt,
@@ -443,7 +443,7 @@ struct DenseTcArgs {
 int dense_tc_out_tiles(int n);
 int dense_tc_k_chunks(int n);
 void dense_tc_tiles(const std::vector<double>& M, int n, std::vector<uint16_t>& out);
-cudaError_t launch_dense_tc(const DenseTcArgs& a, DevStatus* st, cudaStream_t s);
+cudaError_t launch_dense_tc(const DenseTcArgs& a, DevStatus* st, Queue s);
 
 // Tables of the tensor-core z expansion (PP_MIXED_TC): two launches of the
 // dense transform, V^T W with the eigenvalue divide into the second

@@ -145,7 +145,7 @@ template <typename T>
 cudaError_t launch_resid_fftx(const Geo& g, const Faces& fc, const FftDesc& fx, const C2<T>* twx,
                               const double* b, double inv_dt, const double* rho, const double* p,
                               int p_zero, int scale_rho, C2<T>* spec, double* red, const LoopCheck* ck,
-                              const DevStatus* st, cudaStream_t s, float* E, const float* delta) {
+                              const DevStatus* st, Queue s, float* E, const float* delta) {
   if (wfft_length(g.nx) || (g.nx == 512 && std::is_same<T, float>::value))
     return launch_resid_w<T>(g, fc, twx, b, rho, p, p_zero, scale_rho, spec, red, ck, st, s, E, delta);
   const int rpb = rows_per_block(g.nx, kEpt);
@@ -162,14 +162,13 @@ cudaError_t launch_resid_fftx(const Geo& g, const Faces& fc, const FftDesc& fx, 
   if (e != cudaSuccess) return e;
   const int mode = (red == nullptr) ? 0 : 1;
   (void)inv_dt;
-  kern<<<nblk, kThreads, smem, s>>>(g, fc, fx, twx, b, rho, p, mode, p_zero, scale_rho, spec, red, rpb, st, E,
-                                    delta, ck ? *ck : LoopCheck{});
-  return cudaGetLastError();
+  return enqueue(s, kern, nblk, kThreads, smem, g, fc, fx, twx, b, rho, p, mode, p_zero, scale_rho, spec, red, rpb,
+                 st, E, delta, ck ? *ck : LoopCheck{});
 }
 
 template <typename T>
 cudaError_t launch_ffty(const Geo& g, const FftDesc& fy, const C2<T>* twy, C2<T>* spec, int inverse,
-                        const DevStatus* st, cudaStream_t s, const C2<T>* dct) {
+                        const DevStatus* st, Queue s, const C2<T>* dct) {
   if constexpr (std::is_same<T, float>::value) {
     if (g.ny == 512 && dct == nullptr)
       return launch_ffty512(g, reinterpret_cast<const float2*>(twy), reinterpret_cast<float2*>(spec), inverse, st, s);
@@ -187,8 +186,8 @@ cudaError_t launch_ffty(const Geo& g, const FftDesc& fy, const C2<T>* twy, C2<T>
     long long nblk = 0;
     const cudaError_t e = resident(&nblk);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)(nblk < ntiles ? nblk : ntiles), kThreads, smem, s>>>(g, fy, twy, spec, tx, ntiles, st, dct);
-    return cudaGetLastError();
+    return enqueue(s, kern, (unsigned)(nblk < ntiles ? nblk : ntiles), kThreads, smem, g, fy, twy, spec, tx, ntiles,
+                   st, dct);
   };
 #define PP_GO(...) go([&](long long* n) { return resident_blocks<__VA_ARGS__>(kThreads, smem, n); }, __VA_ARGS__)
   if (dct) return inverse ? PP_GO(k_ffty<T, 1, true>) : PP_GO(k_ffty<T, -1, true>);
@@ -198,7 +197,7 @@ cudaError_t launch_ffty(const Geo& g, const FftDesc& fy, const C2<T>* twy, C2<T>
 
 template <typename T>
 cudaError_t launch_zdct(const Geo& g, const FftDesc& fz, const C2<T>* twz, C2<T>* spec, int inverse,
-                        const DevStatus* st, cudaStream_t s, const C2<T>* dct, const ZDivide& zd) {
+                        const DevStatus* st, Queue s, const C2<T>* dct, const ZDivide& zd) {
   const int tx = ffty_tile(g.nz, sizeof(C2<T>), kEpt);
   const int tsz = g.nz * tx;
   const size_t smem = (sizeof(T) == sizeof(float))
@@ -215,11 +214,10 @@ cudaError_t launch_zdct(const Geo& g, const FftDesc& fz, const C2<T>* twz, C2<T>
   if (per_sm < 1) per_sm = 1;
   long long nblk = (long long)nsm * per_sm;
   if (nblk > ntiles) nblk = ntiles;
-  kern<<<(int)nblk, kThreads, smem, s>>>(g, fz, twz, spec, tx, ntiles, st, dct, zd);
-  return cudaGetLastError();
+  return enqueue(s, kern, (int)nblk, kThreads, smem, g, fz, twz, spec, tx, ntiles, st, dct, zd);
 }
 template cudaError_t launch_zdct<double>(const Geo&, const FftDesc&, const double2*, double2*, int,
-                                         const DevStatus*, cudaStream_t, const double2*, const ZDivide&);
+                                         const DevStatus*, Queue, const double2*, const ZDivide&);
 
 int tri_mixed_blocks(size_t ncol, int nlow) {
   constexpr int kWarps = kZThreads / 32;
@@ -228,25 +226,21 @@ int tri_mixed_blocks(size_t ncol, int nlow) {
 
 template <typename T>
 cudaError_t launch_tridiag(const Geo& g, const double* invd, C2<T>* spec, double2* ybuf,
-                           const DevStatus* st, cudaStream_t s, const double* mtab, const TriF32* f32) {
+                           const DevStatus* st, Queue s, const double* mtab, const TriF32* f32) {
   const size_t ncol = (size_t)g.ny * g.nxh;
   if (f32 != nullptr && sizeof(T) == sizeof(float)) {
-    k_tridiag_mixed<<<tri_mixed_blocks(ncol, f32->nlow), kZThreads, zsweep_smem<ZForm32, 1>(), s>>>(
-        g, mtab, invd, *f32, reinterpret_cast<float2*>(spec), st);
-  } else {
-    const int nblk = (int)((ncol + 127) / 128);
-    k_tridiag<T><<<nblk, 128, 0, s>>>(g, invd, spec, ybuf, st);
+    return enqueue(s, k_tridiag_mixed, tri_mixed_blocks(ncol, f32->nlow), kZThreads, zsweep_smem<ZForm32, 1>(), g,
+                   mtab, invd, *f32, reinterpret_cast<float2*>(spec), st);
   }
-  return cudaGetLastError();
+  return enqueue(s, k_tridiag<T>, (int)((ncol + 127) / 128), 128, 0, g, invd, spec, ybuf, st);
 }
 
 template <class F, int P>
 static cudaError_t launch_zsolve_p(const Geo& g, const F& form, int nyt, int ysym, size_t work, typename F::Val* spec,
-                                   const DevStatus* st, cudaStream_t s) {
+                                   const DevStatus* st, Queue s) {
   static_assert(zsweep_smem<F, P>() <= 48 * 1024, "fits without the opt-in attribute");
-  k_zsolve<F, P><<<(unsigned)((work + kZThreads - 1) / kZThreads), kZThreads, zsweep_smem<F, P>(), s>>>(
-      g, form, nyt, ysym, spec, st);
-  return cudaGetLastError();
+  return enqueue(s, k_zsolve<F, P>, (unsigned)((work + kZThreads - 1) / kZThreads), kZThreads, zsweep_smem<F, P>(), g,
+                 form, nyt, ysym, spec, st);
 }
 
 // Two columns a thread halve the table traffic and leave half the warps: it
@@ -254,7 +248,7 @@ static cudaError_t launch_zsolve_p(const Geo& g, const F& form, int nyt, int ysy
 // 512^3, 3.4 warps, 0.533 / 0.512 ms; 384^3, 1.9 warps, 0.235 / 0.214 ms;
 // 256^3, 0.85 warps, 0.088 / 0.115 ms).
 template <typename T>
-cudaError_t launch_zsolve(const Geo& g, const TriZ<T>& t, C2<T>* spec, const DevStatus* st, cudaStream_t s) {
+cudaError_t launch_zsolve(const Geo& g, const TriZ<T>& t, C2<T>* spec, const DevStatus* st, Queue s) {
   const size_t ncol = (size_t)g.ny * g.nxh;
   if constexpr (std::is_same<T, float>::value) {
     const ZForm64 form{t.m, t.d, t.e};
@@ -267,8 +261,8 @@ cudaError_t launch_zsolve(const Geo& g, const TriZ<T>& t, C2<T>* spec, const Dev
     return launch_zsolve_p<ZFormD, 1>(g, form, t.nyt, t.ysym, 2 * ncol, reinterpret_cast<double*>(spec), st, s);
   }
 }
-template cudaError_t launch_zsolve<float>(const Geo&, const TriZ<float>&, float2*, const DevStatus*, cudaStream_t);
-template cudaError_t launch_zsolve<double>(const Geo&, const TriZ<double>&, double2*, const DevStatus*, cudaStream_t);
+template cudaError_t launch_zsolve<float>(const Geo&, const TriZ<float>&, float2*, const DevStatus*, Queue);
+template cudaError_t launch_zsolve<double>(const Geo&, const TriZ<double>&, double2*, const DevStatus*, Queue);
 
 std::vector<int> tri_low_columns(const std::vector<double>& lamx, const std::vector<double>& lamy,
                                  double thr) {
@@ -298,7 +292,7 @@ cudaError_t launch_narrow(const double* src, float* dst, size_t n, cudaStream_t 
 
 template <typename T>
 cudaError_t launch_fftx_inv(const Geo& g, const FftDesc& fx, const C2<T>* twx, const C2<T>* spec,
-                            double scale, double* p, int p_zero, const DevStatus* st, cudaStream_t s,
+                            double scale, double* p, int p_zero, const DevStatus* st, Queue s,
                             T* delta, float* sdelta) {
   if constexpr (std::is_same<T, float>::value) {
     if (g.nx == 512)
@@ -317,22 +311,21 @@ cudaError_t launch_fftx_inv(const Geo& g, const FftDesc& fx, const C2<T>* twx, c
                           : 2 * nbuf * sizeof(C2<T>);
   cudaError_t e = cudaFuncSetAttribute(k_fftx_inv<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_fftx_inv<T><<<nblk, kThreads, smem, s>>>(g, fx, twx, spec, scale, p, p_zero, rpb, st, delta, sdelta);
-  return cudaGetLastError();
+  return enqueue(s, k_fftx_inv<T>, nblk, kThreads, smem, g, fx, twx, spec, scale, p, p_zero, rpb, st, delta, sdelta);
 }
 
 #define PP_INST(T)                                                                                   \
   template cudaError_t launch_resid_fftx<T>(const Geo&, const Faces&, const FftDesc&, const C2<T>*,  \
                                             const double*, double, const double*, const double*,     \
                                             int, int, C2<T>*, double*, const LoopCheck*, const DevStatus*, \
-                                            cudaStream_t, float*, const float*);                    \
+                                            Queue, float*, const float*);                    \
   template cudaError_t launch_ffty<T>(const Geo&, const FftDesc&, const C2<T>*, C2<T>*, int,         \
-                                      const DevStatus*, cudaStream_t, const C2<T>*);                 \
+                                      const DevStatus*, Queue, const C2<T>*);                 \
   template cudaError_t launch_tridiag<T>(const Geo&, const double*, C2<T>*, double2*,                \
-                                         const DevStatus*, cudaStream_t, const double*,              \
+                                         const DevStatus*, Queue, const double*,              \
                                          const TriF32*);                                             \
   template cudaError_t launch_fftx_inv<T>(const Geo&, const FftDesc&, const C2<T>*, const C2<T>*,    \
-                                          double, double*, int, const DevStatus*, cudaStream_t,      \
+                                          double, double*, int, const DevStatus*, Queue,      \
                                           T*, float*);
 PP_INST(double)
 PP_INST(float)

@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(64 * kXLines, 4) k_fftx512_inv(Geo g, const fl
 }
 
 cudaError_t launch_fftx512_inv(const Geo& g, const float2* twx, const float2* spec, double scale, double* p,
-                               int p_zero, const DevStatus* st, cudaStream_t s, float* delta, float* sdelta) {
+                               int p_zero, const DevStatus* st, Queue s, float* delta, float* sdelta) {
   if (g.nxh != kXNh) return cudaErrorInvalidValue;
   const size_t smem = R512<kXLines>::smem_bytes() + (size_t)2 * kXLines * kXStageRow * sizeof(float2);
   const long long nrows = (long long)g.nz * g.ny;
@@ -150,9 +150,8 @@ cudaError_t launch_fftx512_inv(const Geo& g, const float2* twx, const float2* sp
   long long nblk = 0;
   const cudaError_t e = resident_blocks<k_fftx512_inv>(64 * kXLines, smem, &nblk);
   if (e != cudaSuccess) return e;
-  k_fftx512_inv<<<(unsigned)(nblk < ngroups ? nblk : ngroups), 64 * kXLines, smem, s>>>(
-      g, twx, spec, scale, p, p_zero, ngroups, st, delta, sdelta);
-  return cudaGetLastError();
+  return enqueue(s, k_fftx512_inv, (unsigned)(nblk < ngroups ? nblk : ngroups), 64 * kXLines, smem, g, twx, spec,
+                 scale, p, p_zero, ngroups, st, delta, sdelta);
 }
 
 }  // namespace pp

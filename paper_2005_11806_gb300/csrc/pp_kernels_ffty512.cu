@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(64 * TX) k_ffty512(Geo g, const float2* __rest
 constexpr int kFfty512Tx = 8;
 
 cudaError_t launch_ffty512(const Geo& g, const float2* twy, float2* spec, int inverse, const DevStatus* st,
-                           cudaStream_t s) {
+                           Queue s) {
   constexpr int TX = kFfty512Tx;
   const size_t smem = R512<TX>::smem_bytes();
   const long long ntiles = (long long)((g.nxh + TX - 1) / TX) * g.nz;
@@ -69,8 +69,7 @@ cudaError_t launch_ffty512(const Geo& g, const float2* twy, float2* spec, int in
                                 : resident_blocks<k_ffty512<-1, TX>>(64 * TX, smem, &nblk);
   if (e != cudaSuccess) return e;
   auto kern = inverse ? k_ffty512<1, TX> : k_ffty512<-1, TX>;
-  kern<<<(unsigned)(nblk < ntiles ? nblk : ntiles), 64 * TX, smem, s>>>(g, twy, spec, ntiles, st);
-  return cudaGetLastError();
+  return enqueue(s, kern, (unsigned)(nblk < ntiles ? nblk : ntiles), 64 * TX, smem, g, twy, spec, ntiles, st);
 }
 
 }  // namespace pp

@@ -76,17 +76,16 @@ __global__ void __launch_bounds__(256) k_ydense(Geo g, const T* __restrict__ mt,
 }
 
 template <typename T, int TX, int R>
-static cudaError_t launch_ydense_r(const Geo& g, const T* mt, C2<T>* spec, const DevStatus* st, cudaStream_t s) {
+static cudaError_t launch_ydense_r(const Geo& g, const T* mt, C2<T>* spec, const DevStatus* st, Queue s) {
   const size_t smem = (size_t)g.ny * TX * sizeof(C2<T>);
   cudaError_t e = cudaFuncSetAttribute(k_ydense<T, TX, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const long long nblk = (long long)((g.nxh + TX - 1) / TX) * g.nz;
-  k_ydense<T, TX, R><<<(unsigned)nblk, 256, smem, s>>>(g, mt, spec, st);
-  return cudaGetLastError();
+  return enqueue(s, k_ydense<T, TX, R>, (unsigned)nblk, 256, smem, g, mt, spec, st);
 }
 
 // Columns per block: 4 complex FP64 values of a row, 64 bytes.
-cudaError_t launch_ydense(const Geo& g, const double* mt, double2* spec, const DevStatus* st, cudaStream_t s) {
+cudaError_t launch_ydense(const Geo& g, const double* mt, double2* spec, const DevStatus* st, Queue s) {
   constexpr int TX = 4;
   switch ((g.ny + 255) / 256) {
     case 1: return launch_ydense_r<double, TX, 1>(g, mt, spec, st, s);

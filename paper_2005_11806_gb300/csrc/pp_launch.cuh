@@ -4,8 +4,54 @@
 
 #include <atomic>
 #include <cstdint>
+#include <tuple>
 
 namespace pp {
+
+// Kernel nodes strung one after the other in a graph under construction.
+struct GraphChain {
+  cudaGraph_t graph;
+  cudaGraphNode_t last;
+};
+
+// Where a launch goes: to a stream, or with a chain to the chain's end.  The
+// nodes are added one by one, not captured from a stream: while any stream of
+// a device is being captured, another host thread may not wait for the device
+// (cudaErrorStreamCaptureUnsupported), and a projection must not forbid that.
+struct Queue {
+  cudaStream_t stream;
+  GraphChain* chain;
+  Queue(cudaStream_t s, GraphChain* c = nullptr) : stream(s), chain(c) {}
+};
+
+template <class... P, class... A>
+inline cudaError_t enqueue(Queue q, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, A&&... args) {
+  static_assert(sizeof...(P) == sizeof...(A), "");
+  std::tuple<P...> value(static_cast<P>(args)...);
+  void* at[sizeof...(P)];
+  std::apply([&](P&... v) {
+    void* a[] = {(void*)&v...};
+    for (size_t i = 0; i < sizeof...(P); ++i) at[i] = a[i];
+  }, value);
+  cudaError_t e;
+  if (q.chain == nullptr) {
+    e = cudaLaunchKernel((const void*)kernel, grid, block, at, smem, q.stream);
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e;
+  }
+  cudaKernelNodeParams kp{};
+  kp.func = (void*)kernel;
+  kp.gridDim = grid;
+  kp.blockDim = block;
+  kp.sharedMemBytes = (unsigned)smem;
+  kp.kernelParams = at;
+  GraphChain* c = q.chain;
+  cudaGraphNode_t node = nullptr;
+  e = cudaGraphAddKernelNode(&node, c->graph, c->last ? &c->last : nullptr, c->last ? 1 : 0, &kp);
+  if (e == cudaSuccess) c->last = node;
+  else (void)cudaGetLastError();
+  return e;
+}
 
 // Blocks of K resident at once on the current device (at least one an SM),
 // with smem bytes of dynamic shared memory allowed for it: the grid of a

@@ -5,7 +5,7 @@ namespace pp {
 
 template <typename T>
 cudaError_t launch_fftx_inv_w(const Geo& g, const C2<T>* twx, const C2<T>* spec, double scale, double* p, int p_zero,
-                              const DevStatus* st, cudaStream_t s, T* delta, float* sdelta) {
+                              const DevStatus* st, Queue s, T* delta, float* sdelta) {
   switch (g.nx) {
 #define PP_X(N) case N: return launch_fftx_inv_w_n<T, N>(g, twx, spec, scale, p, p_zero, st, s, delta, sdelta);
     PP_WFFT_LENGTHS(PP_X)
@@ -14,8 +14,8 @@ cudaError_t launch_fftx_inv_w(const Geo& g, const C2<T>* twx, const C2<T>* spec,
   return cudaErrorInvalidValue;
 }
 template cudaError_t launch_fftx_inv_w<float>(const Geo&, const float2*, const float2*, double, double*, int,
-                                              const DevStatus*, cudaStream_t, float*, float*);
+                                              const DevStatus*, Queue, float*, float*);
 template cudaError_t launch_fftx_inv_w<double>(const Geo&, const double2*, const double2*, double, double*, int,
-                                               const DevStatus*, cudaStream_t, double*, float*);
+                                               const DevStatus*, Queue, double*, float*);
 
 }  // namespace pp

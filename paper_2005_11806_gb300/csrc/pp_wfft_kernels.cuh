@@ -521,7 +521,7 @@ inline int wfft_warps_per_block(long long warps) {
 template <typename T, int N>
 cudaError_t launch_resid_w_n(const Geo& g, const Faces& fc, const C2<T>* twx, const double* b, const double* rho,
                              const double* p, int p_zero, int scale_rho, C2<T>* spec, double* red,
-                             const LoopCheck* ck, const DevStatus* st, cudaStream_t s, float* E, const float* delta) {
+                             const LoopCheck* ck, const DevStatus* st, Queue s, float* E, const float* delta) {
   using W = WPlan<N>;
   const long long nrows = (long long)g.nz * g.ny;
   const long long warps = (nrows + 2 * W::LW - 1) / (2 * W::LW);
@@ -529,41 +529,37 @@ cudaError_t launch_resid_w_n(const Geo& g, const Faces& fc, const C2<T>* twx, co
   const size_t smem = (size_t)(W::TW + wpb * W::LW * W::LS) * sizeof(C2<T>);
   auto kern = (g.ym != nullptr) ? k_resid_w<T, true, N> : k_resid_w<T, false, N>;
   static_assert((W::TW + 4 * W::LW * W::LS) * sizeof(C2<T>) <= 48 * 1024, "fits without the opt-in attribute");
-  kern<<<(unsigned)((warps + wpb - 1) / wpb), 32 * wpb, smem, s>>>(g, fc, twx, b, rho, p, red == nullptr ? 0 : 1,
-                                                                  p_zero, scale_rho, spec, red, st, E, delta,
-                                                                  ck ? *ck : LoopCheck{});
-  return cudaGetLastError();
+  return enqueue(s, kern, (unsigned)((warps + wpb - 1) / wpb), 32 * wpb, smem, g, fc, twx, b, rho, p,
+                 red == nullptr ? 0 : 1, p_zero, scale_rho, spec, red, st, E, delta, ck ? *ck : LoopCheck{});
 }
 
 template <typename T, int N>
 cudaError_t launch_fftx_inv_w_n(const Geo& g, const C2<T>* twx, const C2<T>* spec, double scale, double* p,
-                                int p_zero, const DevStatus* st, cudaStream_t s, T* delta, float* sdelta) {
+                                int p_zero, const DevStatus* st, Queue s, T* delta, float* sdelta) {
   using W = WPlan<N>;
   const long long nrows = (long long)g.nz * g.ny;
   const long long warps = (nrows + 2 * W::LW - 1) / (2 * W::LW);
   const int wpb = wfft_warps_per_block(warps);
   const size_t smem = (size_t)(N + wpb * W::LW * W::LS) * sizeof(C2<T>);
   static_assert((N + 4 * W::LW * W::LS) * sizeof(C2<T>) <= 48 * 1024, "fits without the opt-in attribute");
-  k_fftx_inv_w<T, N><<<(unsigned)((warps + wpb - 1) / wpb), 32 * wpb, smem, s>>>(g, twx, spec, scale, p, p_zero, st,
-                                                                                delta, sdelta);
-  return cudaGetLastError();
+  return enqueue(s, k_fftx_inv_w<T, N>, (unsigned)((warps + wpb - 1) / wpb), 32 * wpb, smem, g, twx, spec, scale, p,
+                 p_zero, st, delta, sdelta);
 }
 
 template <auto K, typename T, int N>
-cudaError_t launch_ffty_w_k(const Geo& g, const C2<T>* twy, C2<T>* spec, const DevStatus* st, cudaStream_t s,
+cudaError_t launch_ffty_w_k(const Geo& g, const C2<T>* twy, C2<T>* spec, const DevStatus* st, Queue s,
                             const C2<T>* dct) {
   using Y = WyShape<T, N>;
   const long long ntiles = (long long)((g.nxh + kWyTx - 1) / kWyTx) * g.nz;
   long long nblk = 0;
   const cudaError_t e = resident_blocks<K>(Y::threads, Y::smem, &nblk);
   if (e != cudaSuccess) return e;
-  K<<<(unsigned)(nblk < ntiles ? nblk : ntiles), Y::threads, Y::smem, s>>>(g, twy, spec, ntiles, st, dct);
-  return cudaGetLastError();
+  return enqueue(s, K, (unsigned)(nblk < ntiles ? nblk : ntiles), Y::threads, Y::smem, g, twy, spec, ntiles, st, dct);
 }
 
 template <typename T, int N>
 cudaError_t launch_ffty_w_n(const Geo& g, const C2<T>* twy, C2<T>* spec, int inverse, const DevStatus* st,
-                            cudaStream_t s, const C2<T>* dct) {
+                            Queue s, const C2<T>* dct) {
   if (dct)
     return inverse ? launch_ffty_w_k<k_ffty_w<T, 1, true, N>, T, N>(g, twy, spec, st, s, dct)
                    : launch_ffty_w_k<k_ffty_w<T, -1, true, N>, T, N>(g, twy, spec, st, s, dct);

@@ -6,7 +6,7 @@ namespace pp {
 template <>
 cudaError_t launch_resid_w<float>(const Geo& g, const Faces& fc, const C2<float>* twx, const double* b, const double* rho,
                                 const double* p, int p_zero, int scale_rho, C2<float>* spec, double* red,
-                                const LoopCheck* ck, const DevStatus* st, cudaStream_t s, float* E, const float* delta) {
+                                const LoopCheck* ck, const DevStatus* st, Queue s, float* E, const float* delta) {
   switch (g.nx) {
 #define PP_X(N) \
   case N: return launch_resid_w_n<float, N>(g, fc, twx, b, rho, p, p_zero, scale_rho, spec, red, ck, st, s, E, delta);

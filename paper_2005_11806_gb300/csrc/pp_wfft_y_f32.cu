@@ -5,7 +5,7 @@ namespace pp {
 
 template <>
 cudaError_t launch_ffty_w<float>(const Geo& g, const C2<float>* twy, C2<float>* spec, int inverse, const DevStatus* st,
-                               cudaStream_t s, const C2<float>* dct) {
+                               Queue s, const C2<float>* dct) {
   switch (g.ny) {
 #define PP_X(N) case N: return launch_ffty_w_n<float, N>(g, twy, spec, inverse, st, s, dct);
     PP_WFFT_LENGTHS(PP_X)
