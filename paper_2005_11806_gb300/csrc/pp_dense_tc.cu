@@ -419,8 +419,7 @@ bool encode_view_map(const DenseTcArgs& a, CUtensorMap* map) {
 template <bool TMA>
 cudaError_t launch_dense_tc_t(const DenseTcArgs& a, const CUtensorMap& map, int grid, DevStatus* st,
                               Queue s) {
-  cudaError_t e = cudaFuncSetAttribute(k_dense_tc<TMA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)Cfg<TMA>::smem);
+  const cudaError_t e = allow_smem<k_dense_tc<TMA>>();
   if (e != cudaSuccess) return e;
   return enqueue(s, k_dense_tc<TMA>, grid, kThreadsTC, Cfg<TMA>::smem, a, map, st);
 }

@@ -158,7 +158,7 @@ cudaError_t launch_resid_fftx(const Geo& g, const Faces& fc, const FftDesc& fx, 
                           ? (nbuf + fft_pad_elems((int)nbuf) + g.nx) * sizeof(float2)
                           : 2 * nbuf * sizeof(C2<T>);
   auto kern = (g.ym != nullptr) ? k_resid_fftx<T, true> : k_resid_fftx<T, false>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = (g.ym != nullptr) ? allow_smem<k_resid_fftx<T, true>>() : allow_smem<k_resid_fftx<T, false>>();
   if (e != cudaSuccess) return e;
   const int mode = (red == nullptr) ? 0 : 1;
   (void)inv_dt;
@@ -205,7 +205,7 @@ cudaError_t launch_zdct(const Geo& g, const FftDesc& fz, const C2<T>* twz, C2<T>
                           : (size_t)3 * tsz * sizeof(C2<T>);
   const long long ntiles = (long long)((g.nxh + tx - 1) / tx) * g.ny;
   auto kern = inverse ? k_fftz<T, 1> : k_fftz<T, -1>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = inverse ? allow_smem<k_fftz<T, 1>>() : allow_smem<k_fftz<T, -1>>();
   if (e != cudaSuccess) return e;
   int per_sm = 0, dev = 0, nsm = 0;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem)) != cudaSuccess) return e;
@@ -309,7 +309,7 @@ cudaError_t launch_fftx_inv(const Geo& g, const FftDesc& fx, const C2<T>* twx, c
   const size_t smem = (sizeof(T) == sizeof(float))
                           ? (nbuf + fft_pad_elems((int)nbuf) + g.nx) * sizeof(float2)
                           : 2 * nbuf * sizeof(C2<T>);
-  cudaError_t e = cudaFuncSetAttribute(k_fftx_inv<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem<k_fftx_inv<T>>();
   if (e != cudaSuccess) return e;
   return enqueue(s, k_fftx_inv<T>, nblk, kThreads, smem, g, fx, twx, spec, scale, p, p_zero, rpb, st, delta, sdelta);
 }

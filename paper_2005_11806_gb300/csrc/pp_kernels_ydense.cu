@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(256) k_ydense(Geo g, const T* __restrict__ mt,
 template <typename T, int TX, int R>
 static cudaError_t launch_ydense_r(const Geo& g, const T* mt, C2<T>* spec, const DevStatus* st, Queue s) {
   const size_t smem = (size_t)g.ny * TX * sizeof(C2<T>);
-  cudaError_t e = cudaFuncSetAttribute(k_ydense<T, TX, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem<k_ydense<T, TX, R>>();
   if (e != cudaSuccess) return e;
   const long long nblk = (long long)((g.nxh + TX - 1) / TX) * g.nz;
   return enqueue(s, k_ydense<T, TX, R>, (unsigned)nblk, 256, smem, g, mt, spec, st);

@@ -53,11 +53,30 @@ inline cudaError_t enqueue(Queue q, void (*kernel)(P...), dim3 grid, dim3 block,
   return e;
 }
 
+// Lets K be launched with any dynamic shared memory that the current device
+// has.  The limit belongs to the function and the process, so it is set once,
+// to its largest value, and never lowered: plans of other lengths may be
+// launching K from other threads.
+template <auto K>
+inline cudaError_t allow_smem() {
+  static std::atomic<uint64_t> done;  // a bit per device
+  int dev = 0, most = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = dev >= 0 && dev < 64 ? (uint64_t)1 << dev : 0;
+  if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  cudaFuncAttributes a;
+  if ((e = cudaFuncGetAttributes(&a, K)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)a.sharedSizeBytes);
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+  return e;
+}
+
 // Blocks of K resident at once on the current device (at least one an SM),
-// with smem bytes of dynamic shared memory allowed for it: the grid of a
-// persistent kernel.  One entry per kernel and device, remembered for the last
-// smem asked for (three runtime calls a launch before: 1 to 2 % of a pass up
-// to 256^3).
+// with smem bytes of dynamic shared memory: the grid of a persistent kernel.
+// One entry per kernel and device, remembered for the last smem asked for
+// (three runtime calls a launch before: 1 to 2 % of a pass up to 256^3).
 //
 // Measured and dropped: programmatic stream serialization of the pass kernels
 // (blocks placed early, waiting for the kernel before): 32^3 0.0567 ms a pass
@@ -70,17 +89,17 @@ inline cudaError_t resident_blocks(int threads, size_t smem, long long* out) {
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   const bool slot = dev >= 0 && dev < 64;
-  const uint64_t seen = slot ? known[dev].load(std::memory_order_relaxed) : 0;
+  const uint64_t seen = slot ? known[dev].load(std::memory_order_acquire) : 0;
   if (seen != 0 && (seen >> 32) == (uint64_t)smem) {
     *out = (long long)(seen & 0xFFFFFFFFu);
     return cudaSuccess;
   }
   int per_sm = 0, nsm = 0;
-  if ((e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+  if ((e = allow_smem<K>()) != cudaSuccess) return e;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, K, threads, smem)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   *out = (long long)nsm * (per_sm < 1 ? 1 : per_sm);
-  if (slot) known[dev].store(((uint64_t)smem << 32) | (uint64_t)*out, std::memory_order_relaxed);
+  if (slot) known[dev].store(((uint64_t)smem << 32) | (uint64_t)*out, std::memory_order_release);
   return cudaSuccess;
 }
 

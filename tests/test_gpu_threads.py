@@ -110,3 +110,13 @@ def test_graph_equals_single_launches(dims, kw):
         plan.close()
     assert torch.equal(found[0], found[1])
     assert torch.isfinite(found[0]).all() and found[0].abs().max() > 0
+
+
+def test_two_plans_with_other_shared_memory():
+    """Two threads whose plans take the same y kernel with 76.8 and 96 KB of shared memory."""
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    cases = [_case((16, ny, 8), s.cuda_stream, precision="fp64") for ny, s in zip((200, 250), streams)]
+    errors, counts = _together([lambda c=c: c[1](3) for c in cases], 4.0)
+    assert not errors and min(counts) > 100
+    for plan, _, _ in cases:
+        plan.close()
