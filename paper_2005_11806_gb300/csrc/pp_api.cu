@@ -43,7 +43,8 @@ struct pp_plan_s {
   FftDesc fx, fy;
   Geo geo;
   Faces faces;
-  // device tables
+  // device tables; the FP64 ones of the metrics lie in one allocation
+  double* d_metrics = nullptr;
   double *d_inv_dzf = nullptr, *d_inv_dzc = nullptr, *d_dzf = nullptr, *d_za = nullptr, *d_zc = nullptr;
   double *d_lamx = nullptr, *d_lamy = nullptr, *d_invd = nullptr, *d_mtab = nullptr;
   float* d_inv_dzf_f = nullptr;
@@ -85,7 +86,8 @@ struct pp_plan_s {
   float *d_mtab_f = nullptr, *d_invd_f = nullptr, *d_zc_f = nullptr;
   int* d_low = nullptr;
   TriF32 tri32{};
-  // FP64 and PP_MIXED_Z64: tables of the FP64-recurrence z solve (TriZ)
+  // FP64 and PP_MIXED_Z64: tables of the FP64-recurrence z solve (TriZ), in one
+  // allocation that starts at d_zm
   double *d_zm = nullptr, *d_ze = nullptr;
   void* d_zd = nullptr;  // 1 / d_k in the spectrum's precision
   int z_nyt = 0, z_ysym = 0;
@@ -506,16 +508,13 @@ pp_status check_plan(pp_plan P) {
 
 void free_plan(pp_plan_s* P) {
   if (!P) return;
-  double* dptrs[] = {P->d_inv_dzf, P->d_inv_dzc, P->d_dzf, P->d_za, P->d_zc, P->d_lamx, P->d_lamy,
-                     P->d_invd, P->d_mtab, P->d_b, P->d_red, P->faces.cx, P->faces.cy, P->faces.cz,
-                     P->faces.diag, P->d_rho_tilde, P->d_delta64, P->d_thermo, P->d_cw_d};
+  double* dptrs[] = {P->d_metrics, P->d_invd, P->d_mtab, P->d_b, P->d_red, P->faces.cx, P->faces.cy, P->faces.cz,
+                     P->faces.diag, P->d_rho_tilde, P->d_delta64, P->d_thermo};
   if (P->faces.rhof) cudaFree(P->faces.rhof);
   if (P->d_low) cudaFree(P->d_low);
   float* fptrs[] = {P->faces.diagf, P->d_delta, P->d_sdelta, P->d_mtab_f, P->d_invd_f, P->d_zc_f,
                     P->d_cw_f};
   if (P->d_zm) cudaFree(P->d_zm);
-  if (P->d_ze) cudaFree(P->d_ze);
-  if (P->d_zd) cudaFree(P->d_zd);
   for (float* f : fptrs) if (f) cudaFree(f);
   if (P->d_E) cudaFree(P->d_E);
   if (P->d_mu) cudaFree(P->d_mu);
@@ -672,17 +671,23 @@ pp_status pressure_plan_create(const pp_grid* grid, pp_precision prec, void* str
     return cudaMemcpy(*d, h.data(), h.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess
                ? PP_OK : PP_ERR_CUDA;
   };
-  if ((st = up(&P->d_inv_dzf, inv_dzf)) != PP_OK || (st = up(&P->d_inv_dzc, inv_dzc)) != PP_OK ||
-      (st = up(&P->d_dzf, dzf)) != PP_OK || (st = up(&P->d_za, za)) != PP_OK ||
-      (st = up(&P->d_zc, zc)) != PP_OK || (st = up(&P->d_lamx, lamx)) != PP_OK ||
-      (st = up(&P->d_lamy, lamy)) != PP_OK) {
+  // one allocation and one copy: each costs the host more than the bytes do
+  const std::vector<double> cwd = layer_factors_f64(nz, dzf, inv_dzc, 1.0 / (P->dx * P->dx), 1.0 / (P->dy * P->dy));
+  const struct { double** at; const std::vector<double>* v; } metrics[] = {
+      {&P->d_inv_dzf, &inv_dzf}, {&P->d_inv_dzc, &inv_dzc}, {&P->d_dzf, &dzf}, {&P->d_za, &za}, {&P->d_zc, &zc},
+      {&P->d_lamx, &lamx}, {&P->d_lamy, &lamy}, {&P->d_cw_d, &cwd}};
+  std::vector<double> packed;
+  for (const auto& m : metrics) packed.insert(packed.end(), m.v->begin(), m.v->end());
+  if ((st = up(&P->d_metrics, packed)) != PP_OK) {
     free_plan(P);
     return st;
   }
-  if ((st = up(&P->d_cw_d, layer_factors_f64(nz, dzf, inv_dzc, 1.0 / (P->dx * P->dx), 1.0 / (P->dy * P->dy)))) !=
-      PP_OK) {
-    free_plan(P);
-    return st;
+  {
+    double* at = P->d_metrics;
+    for (const auto& m : metrics) {
+      *m.at = at;
+      at += m.v->size();
+    }
   }
   if (ystretch) {
     std::vector<float> ymf(ymet.begin(), ymet.end());
@@ -774,7 +779,7 @@ pp_status pressure_plan_create(const pp_grid* grid, pp_precision prec, void* str
       (st = dalloc(&P->faces.cy, nc * sizeof(double))) != PP_OK ||
       (st = dalloc(&P->faces.cz, nw * sizeof(double))) != PP_OK ||
       (st = dalloc(&P->faces.diag, nc * sizeof(double))) != PP_OK ||
-      (st = dalloc(&P->faces.rhof, nc * sizeof(float))) != PP_OK ||
+      (prec != PP_FP64 && (st = dalloc(&P->faces.rhof, nc * sizeof(float))) != PP_OK) ||
       (st = dalloc(&P->d_inv_dzf_f, (size_t)nz * sizeof(float))) != PP_OK ||
       (st = dalloc(&P->d_cw_f, 3 * (size_t)(nz + 1) * sizeof(float))) != PP_OK ||
       (st = dalloc(&P->d_st, sizeof(DevStatus))) != PP_OK ||
@@ -845,6 +850,26 @@ pp_status pressure_plan_create(const pp_grid* grid, pp_precision prec, void* str
     P->ze.a1 = P->d_za1;
     P->ze.a2 = P->d_za2;
   }
+  if (prec == PP_MIXED_Z64 || prec == PP_FP64) {
+    // periodic y: lambda_y(ky) = lambda_y(ny - ky), one table column for both
+    P->z_ysym = ywall ? 0 : 1;
+    P->z_nyt = ywall ? G.ny : G.ny / 2 + 1;
+    const size_t ntab = (size_t)nz * P->z_nyt * P->nxh;
+    if ((st = dalloc(&P->d_zm, ntab * (2 * sizeof(double) + csz / 2))) != PP_OK) {
+      free_plan(P);
+      return st;
+    }
+    P->d_ze = P->d_zm + ntab;
+    P->d_zd = P->d_ze + ntab;
+    if ((prec == PP_FP64 ? launch_setup_z<double>(g, P->d_lamx, P->d_lamy, P->z_nyt, P->d_zm, P->d_ze,
+                                                  (double*)P->d_zd, P->stream)
+                         : launch_setup_z<float>(g, P->d_lamx, P->d_lamy, P->z_nyt, P->d_zm, P->d_ze,
+                                                 (float*)P->d_zd, P->stream)) != cudaSuccess) {
+      free_plan(P);
+      return PP_ERR_CUDA;
+    }
+    P->use_z = true;
+  }
   if ((hybrid &&
        launch_setup_pivots(g, P->d_lamx, P->d_lamy, P->d_invd, P->stream, P->d_mtab) != cudaSuccess) ||
       launch_init_status(P->d_st, P->stream) != cudaSuccess ||
@@ -880,25 +905,6 @@ pp_status pressure_plan_create(const pp_grid* grid, pp_precision prec, void* str
     P->tri32.thr = thr;
     P->tri32.low = P->d_low;
     P->tri32.nlow = (int)low.size();
-  }
-  if (prec == PP_MIXED_Z64 || prec == PP_FP64) {
-    // periodic y: lambda_y(ky) = lambda_y(ny - ky), one table column for both
-    P->z_ysym = ywall ? 0 : 1;
-    P->z_nyt = ywall ? G.ny : G.ny / 2 + 1;
-    const size_t ntab = (size_t)nz * P->z_nyt * P->nxh;
-    const size_t tsz = (prec == PP_FP64) ? sizeof(double) : sizeof(float);
-    if ((st = dalloc(&P->d_zm, ntab * sizeof(double))) != PP_OK ||
-        (st = dalloc(&P->d_ze, ntab * sizeof(double))) != PP_OK ||
-        (st = dalloc((unsigned char**)&P->d_zd, ntab * tsz)) != PP_OK ||
-        (prec == PP_FP64 ? launch_setup_z<double>(g, P->d_lamx, P->d_lamy, P->z_nyt, P->d_zm, P->d_ze,
-                                                  (double*)P->d_zd, P->stream)
-                         : launch_setup_z<float>(g, P->d_lamx, P->d_lamy, P->z_nyt, P->d_zm, P->d_ze,
-                                                 (float*)P->d_zd, P->stream)) != cudaSuccess ||
-        cudaStreamSynchronize(P->stream) != cudaSuccess) {
-      free_plan(P);
-      return st != PP_OK ? st : PP_ERR_CUDA;
-    }
-    P->use_z = true;
   }
   *out = P;
   return PP_OK;

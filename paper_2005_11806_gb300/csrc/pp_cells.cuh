@@ -49,7 +49,7 @@ __device__ __forceinline__ void cell_prep_faces(const Geo& g, const double* __re
   fc.cy[c] = (g.ywall && x.j == 0) ? 0.0 : fy * rcp_f64(r + rho[x.cjm]);
   fc.cz[c] = (x.k == 0) ? 0.0 : fz * rcp_f64(r + rho[c - plane]);
   if (x.k == g.nz - 1) fc.cz[c + plane] = 0.0;
-  fc.rhof[c] = (float)r;
+  if (fc.rhof != nullptr) fc.rhof[c] = (float)r;
 }
 
 // diag = sum of the six (row-scaled) coefficients of cell c.

@@ -96,7 +96,7 @@ struct Faces {
   double* cy;    // [nz][ny][nx]
   double* cz;    // [nz+1][ny][nx]
   double* diag;  // [nz][ny][nx]
-  float* rhof;   // [nz][ny][nx]
+  float* rhof;   // [nz][ny][nx]; null on FP64 plans, which do not read it
   float* diagf;
   const double* rho_tilde;
 };
