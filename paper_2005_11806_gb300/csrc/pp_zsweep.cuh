@@ -47,7 +47,12 @@ template <int N> __device__ __forceinline__ void zs_wait() { asm volatile("cp.as
 // one unchanged (127 - 1023 = -896), so widening takes three integer
 // instructions instead of nine, zero and subnormals included, and narrowing
 // seven.  The recurrences are linear, so nothing else changes; a result at
-// or above 2^128 (Inf and NaN inputs stay there) narrows to Inf.
+// or above 2^128 narrows to Inf.  Inf and NaN widen to finite values from
+// 2^128 up, and a sweep may damp these below 2^128 again, so a bad row does
+// not make its whole column Inf.  It reaches the caller all the same: a
+// projection stops on the residual's norm before the sweep, and in a plain
+// solve the mean of column (0, 0), taken in plain FP64, makes that column and
+// with it every value of p non-finite.
 __device__ __forceinline__ double zs_widen(float f) {
   const int b = __float_as_int(f);
   return __hiloint2double((b >> 3) & (int)0x8FFFFFFF, b << 29);
