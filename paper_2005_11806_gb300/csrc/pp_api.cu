@@ -349,7 +349,10 @@ pp_status solve_pass(pp_plan_s* P, double* p, int p_zero, T* delta = nullptr, fl
     const TriZ<T> tz{P->d_zm, P->d_ze, (const T*)P->d_zd, P->z_nyt, P->z_ysym};
     PP_K(P, K_TRI, launch_zsolve<T>(g, tz, zs, P->d_st, P->queue()));
   } else {
-    PP_K(P, K_TRI, launch_tridiag<T>(g, P->d_invd, zs, nullptr, P->d_st, P->queue(), P->d_mtab, &P->tri32));
+    if constexpr (std::is_same<T, float>::value)
+      PP_K(P, K_TRI, launch_tridiag_mixed(g, P->d_invd, P->d_mtab, P->tri32, zs, P->d_st, P->queue()));
+    else
+      return PP_ERR_UNSUPPORTED;
   }
   if (ytc) PP_K(P, K_FFTY_I, launch_dense_tc(ytc_args(zs, spec, P->d_ytc_i), P->d_st, P->queue()));
   else if (P->ystretch) {

@@ -287,7 +287,7 @@ pp_status build_fft_lists(pp_batch_s* B, int ept_x, int ept_y) {
     if (wfft_length(d.g.nx)) {
       batch_wfft_x(d.g.nx, nrows, &sh);
       d.rpb = 0;
-      d.nblk_x = sh.nred;
+      d.nblk_x = sh.nblk_x;
       for (int b = 0; b < sh.nblk_x; ++b) wxw.push_back(make_int2(i, b));
       B->smem_xw = std::max(B->smem_xw, sh.smem_x);
     } else {

@@ -42,7 +42,7 @@ cudaError_t launch_batch_ffty_w(const GridDev* G, const int2* work, int n, size_
 // the partial-sum pairs of the residual) and y kernels (groups of tiles).
 struct BatchWShape {
   size_t smem_x = 0, smem_y = 0;
-  int nblk_x = 0, nred = 0, ngroups_y = 0;
+  int nblk_x = 0, ngroups_y = 0;
 };
 void batch_wfft_x(int nx, long long nrows, BatchWShape* out);
 void batch_wfft_y(int ny, int nxh, int nz, BatchWShape* out);

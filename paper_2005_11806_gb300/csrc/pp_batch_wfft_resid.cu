@@ -34,7 +34,6 @@ static void shape_x(long long nrows, BatchWShape* out) {
   out->smem_x = (size_t)(N + wpb * W::LW * W::LS) * sizeof(float2);
   static_assert((N + wpb * W::LW * W::LS) * sizeof(float2) <= 48 * 1024, "fits without the opt-in attribute");
   out->nblk_x = (int)((warps + wpb - 1) / wpb);
-  out->nred = out->nblk_x;
 }
 
 void batch_wfft_x(int nx, long long nrows, BatchWShape* out) {

@@ -284,14 +284,14 @@ std::vector<int> tri_low_columns(const std::vector<double>& lamx, const std::vec
 // column, then a thread per column).
 int tri_mixed_blocks(size_t ncol, int nlow);
 
-// With f32 (PP_MIXED_FP32 plans) the well-conditioned columns run in FP32 and
-// the others in FP64 with the multipliers mtab; without it one thread solves
-// a whole column in FP64 from the inverse pivots alone (ybuf: its forward
-// values; may alias spec).
-template <typename T>
-cudaError_t launch_tridiag(const Geo& g, const double* invd, C2<T>* spec, double2* ybuf,
-                           const DevStatus* st, Queue s, const double* mtab = nullptr,
-                           const TriF32* f32 = nullptr);
+// FP64 z solve from the inverse pivots alone, one thread a column (the
+// allocation-free solve); ybuf takes the forward values and may alias spec.
+cudaError_t launch_tridiag(const Geo& g, const double* invd, double2* spec, double2* ybuf, const DevStatus* st,
+                           Queue s);
+// z solve of PP_MIXED_FP32 plans: the well-conditioned columns in FP32, the
+// others in FP64 with the multipliers mtab.
+cudaError_t launch_tridiag_mixed(const Geo& g, const double* invd, const double* mtab, const TriF32& f32, float2* spec,
+                                 const DevStatus* st, Queue s);
 // z solve of FP64 and PP_MIXED_Z64 plans: FP64 recurrences in every (kx, ky)
 // column, values stored in the spectrum's precision T.  Thomas elimination
 // in the form

@@ -51,16 +51,15 @@ __global__ void __launch_bounds__(256, 2) k_fftz(Geo g, FftDesc fz, const C2<T>*
   stage_ffty_persistent<T, DIR, true, 1>(g, fz, twz, spec, tx, ntiles, blockIdx.x, gridDim.x, smem_raw, dct, zd);
 }
 
-template <typename T>
 __global__ void __launch_bounds__(128) k_tridiag(Geo g, const double* __restrict__ invd,
-                                                 C2<T>* spec, double2* ybuf,  // ybuf may alias spec
+                                                 double2* spec, double2* ybuf,  // ybuf may alias spec
                                                  const DevStatus* __restrict__ st) {
   if (stopped(st)) return;
   const size_t ncol = (size_t)g.ny * g.nxh;
   const size_t col = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (col >= ncol) return;
-  if (col == 0) thomas_column<T, true>(g, invd, spec, ybuf, col, ncol);
-  else thomas_column<T, false>(g, invd, spec, ybuf, col, ncol);
+  if (col == 0) thomas_column<true>(g, invd, spec, ybuf, col, ncol);
+  else thomas_column<false>(g, invd, spec, ybuf, col, ncol);
 }
 
 // z solve of FP64 and PP_MIXED_Z64 plans: one thread per column of `spec`
@@ -224,15 +223,17 @@ int tri_mixed_blocks(size_t ncol, int nlow) {
   return (nlow + kWarps - 1) / kWarps + (int)((ncol + kZThreads - 1) / kZThreads);
 }
 
-template <typename T>
-cudaError_t launch_tridiag(const Geo& g, const double* invd, C2<T>* spec, double2* ybuf,
-                           const DevStatus* st, Queue s, const double* mtab, const TriF32* f32) {
+cudaError_t launch_tridiag(const Geo& g, const double* invd, double2* spec, double2* ybuf, const DevStatus* st,
+                           Queue s) {
   const size_t ncol = (size_t)g.ny * g.nxh;
-  if (f32 != nullptr && sizeof(T) == sizeof(float)) {
-    return enqueue(s, k_tridiag_mixed, tri_mixed_blocks(ncol, f32->nlow), kZThreads, zsweep_smem<ZForm32, 1>(), g,
-                   mtab, invd, *f32, reinterpret_cast<float2*>(spec), st);
-  }
-  return enqueue(s, k_tridiag<T>, (int)((ncol + 127) / 128), 128, 0, g, invd, spec, ybuf, st);
+  return enqueue(s, k_tridiag, (int)((ncol + 127) / 128), 128, 0, g, invd, spec, ybuf, st);
+}
+
+cudaError_t launch_tridiag_mixed(const Geo& g, const double* invd, const double* mtab, const TriF32& f32, float2* spec,
+                                 const DevStatus* st, Queue s) {
+  const size_t ncol = (size_t)g.ny * g.nxh;
+  return enqueue(s, k_tridiag_mixed, tri_mixed_blocks(ncol, f32.nlow), kZThreads, zsweep_smem<ZForm32, 1>(), g, mtab,
+                 invd, f32, spec, st);
 }
 
 template <class F, int P>
@@ -321,9 +322,6 @@ cudaError_t launch_fftx_inv(const Geo& g, const FftDesc& fx, const C2<T>* twx, c
                                             Queue, float*, const float*);                    \
   template cudaError_t launch_ffty<T>(const Geo&, const FftDesc&, const C2<T>*, C2<T>*, int,         \
                                       const DevStatus*, Queue, const C2<T>*);                 \
-  template cudaError_t launch_tridiag<T>(const Geo&, const double*, C2<T>*, double2*,                \
-                                         const DevStatus*, Queue, const double*,              \
-                                         const TriF32*);                                             \
   template cudaError_t launch_fftx_inv<T>(const Geo&, const FftDesc&, const C2<T>*, const C2<T>*,    \
                                           double, double*, int, const DevStatus*, Queue,      \
                                           T*, float*);

@@ -258,7 +258,7 @@ extern "C" pp_status pressure_solve_noalloc(const pp_grid* grid, const double* f
       launch_setup_pivots(g, (const double*)(S + o_lamx), (const double*)(S + o_lamy), invd, s) != cudaSuccess ||
       launch_resid_fftx<double>(g, none, fx, dtwx, f, 1.0, nullptr, nullptr, 1, 0, spec, nullptr, nullptr, st, s) != cudaSuccess ||
       launch_ffty<double>(g, fy, dtwy, spec, 0, st, s, dct) != cudaSuccess ||
-      launch_tridiag<double>(g, invd, spec, spec, st, s) != cudaSuccess ||
+      launch_tridiag(g, invd, spec, spec, st, s) != cudaSuccess ||
       launch_ffty<double>(g, fy, dtwy, spec, 1, st, s, dct) != cudaSuccess ||
       launch_fftx_inv<double>(g, fx, dtwx, spec, scale, p, 1, st, s) != cudaSuccess ||
       launch_remove_mean(g, p, red, st, s) != cudaSuccess)

@@ -39,9 +39,11 @@ inline int ffty_tile(int ny, size_t csize, int ept) {
 
 __device__ __forceinline__ bool stopped(const DevStatus* st) { return st != nullptr && st->done; }
 
-// Transform dispatch: compile-time passes for the power-of-two lengths and
-// batch shapes the default block sizes produce, the generic mixed-radix
-// passes otherwise (same passes in the same order, so the same results).
+// Transform dispatch: compile-time passes for FP64 lines of 512 (x, y and z) and
+// of 256, 128 and 64 along z (cosine plans), the generic mixed-radix passes
+// otherwise (same passes in the same order, so the same results).  FP32 lines
+// of 512 take fft_dispatch_smem; x and y lines of the other powers of two the
+// register transforms of pp_wfft.cuh.
 #define PP_TRY_FIXED(NN, NBB)                                                                       \
   if (n == NN && nbatch == NBB) {                                                                   \
     if (BATCH_FAST) return fft_block_fixed<T, DIR, true, NN, NBB, NBB, 1>(a, b, tw, tid, nth);      \
@@ -53,66 +55,28 @@ __device__ __forceinline__ C2<T>* fft_dispatch(C2<T>* a, C2<T>* b, const FftDesc
                                                const C2<T>* __restrict__ tw, int tid, int nth) {
   const int n = d.n;
   const bool shape_ok = BATCH_FAST ? (es == nbatch && bs == 1) : (es == 1 && bs == n);
-  if (shape_ok) {
-    if (BATCH_FAST) {
+  if constexpr (std::is_same<T, double>::value) {
+    if (shape_ok) {
       PP_TRY_FIXED(512, 4)
-      PP_TRY_FIXED(256, 8)
-      PP_TRY_FIXED(128, 16)
-      PP_TRY_FIXED(128, 8)
-      PP_TRY_FIXED(64, 16)
-      PP_TRY_FIXED(64, 8)
-    } else {
-      PP_TRY_FIXED(512, 4)
-      PP_TRY_FIXED(256, 8)
-      PP_TRY_FIXED(128, 16)
-      PP_TRY_FIXED(64, 32)
-      PP_TRY_FIXED(32, 32)
+      if constexpr (BATCH_FAST) {
+        PP_TRY_FIXED(256, 8)
+        PP_TRY_FIXED(128, 8)
+        PP_TRY_FIXED(64, 8)
+      }
     }
   }
   return fft_block<T, DIR, BATCH_FAST>(a, b, d, nbatch, es, bs, tw, tid, nth);
 }
 #undef PP_TRY_FIXED
 
-// FP32 fast path (fft_block_smem) for the same shapes; returns the element
-// offset of the result buffer, or -1 when the shape has no fast path (the
-// caller then runs fft_dispatch).  twb: offset of the N-entry twiddle table.
-#define PP_TRY_SMEM(NN, NBB)                                                                        \
-  if (n == NN && nbatch == NBB) {                                                                   \
-    if (BATCH_FAST) return fft_block_smem<DIR, true, NN, NBB, NBB, 1>(a, b, twb, tid, nth);         \
-    return fft_block_smem<DIR, false, NN, NBB, 1, NN>(a, b, twb, tid, nth);                         \
-  }
+// Whether the FP32 fast path (fft_dispatch_smem) takes this shape.
+__host__ __device__ inline bool fft_smem_shape(int n, int nbatch) { return n == 512 && nbatch == 4; }
 
+// FP32 fast path (fft_block_smem) of that shape; returns the element offset of
+// the result buffer.  twb: offset of the N-entry twiddle table.
 template <int DIR, bool BATCH_FAST>
-__device__ __forceinline__ int fft_dispatch_smem(int a, int b, int twb, const FftDesc& d, int nbatch, int es,
-                                                 int bs, int tid, int nth) {
-  const int n = d.n;
-  const bool shape_ok = BATCH_FAST ? (es == nbatch && bs == 1) : (es == 1 && bs == n);
-  if (!shape_ok) return -1;
-  if (BATCH_FAST) {
-    PP_TRY_SMEM(512, 4)
-    PP_TRY_SMEM(256, 8)
-    PP_TRY_SMEM(128, 16)
-    PP_TRY_SMEM(128, 8)
-    PP_TRY_SMEM(64, 16)
-    PP_TRY_SMEM(64, 8)
-  } else {
-    PP_TRY_SMEM(512, 4)
-    PP_TRY_SMEM(256, 8)
-    PP_TRY_SMEM(128, 16)
-    PP_TRY_SMEM(64, 32)
-    PP_TRY_SMEM(32, 32)
-  }
-  return -1;
-}
-#undef PP_TRY_SMEM
-
-// Whether fft_dispatch_smem has a fast path for this shape (host and device).
-__host__ __device__ inline bool fft_smem_shape(int n, int nbatch, bool batch_fast) {
-  if (batch_fast)
-    return (n == 512 && nbatch == 4) || (n == 256 && nbatch == 8) || (n == 128 && (nbatch == 16 || nbatch == 8)) ||
-           (n == 64 && (nbatch == 16 || nbatch == 8));
-  return (n == 512 && nbatch == 4) || (n == 256 && nbatch == 8) || (n == 128 && nbatch == 16) ||
-         (n == 64 && nbatch == 32) || (n == 32 && nbatch == 32);
+__device__ __forceinline__ int fft_dispatch_smem(int a, int b, int twb, int tid, int nth) {
+  return fft_block_smem<DIR, BATCH_FAST, 512, 4, BATCH_FAST ? 4 : 1, BATCH_FAST ? 1 : 512>(a, b, twb, tid, nth);
 }
 
 // Copies the N-entry twiddle table into shared memory at element offset twb.
@@ -608,7 +572,7 @@ __device__ __forceinline__ void stage_resid_fftx(const Geo& g, const Faces& fc, 
   // pass: fft_pad_elems), then the twiddle table
   constexpr bool F32 = std::is_same<T, float>::value;
   const int twb = nseq * nx + fft_pad_elems(nseq * nx);
-  const bool fast = F32 && fft_smem_shape(nx, nseq, false);
+  const bool fast = F32 && fft_smem_shape(nx, nseq);
   if constexpr (F32) {
     if (fast) load_twiddles_smem(twx, nx, twb);
   }
@@ -628,7 +592,7 @@ __device__ __forceinline__ void stage_resid_fftx(const Geo& g, const Faces& fc, 
   const C2<T>* res = nullptr;
   if constexpr (F32) {
     if (fast)
-      res = smem_f2() + fft_dispatch_smem<-1, false>(0, nseq * nx, twb, fx, nseq, 1, nx, threadIdx.x, blockDim.x);
+      res = smem_f2() + fft_dispatch_smem<-1, false>(0, nseq * nx, twb, threadIdx.x, blockDim.x);
   }
   if (!fast) res = fft_dispatch<T, -1, false>(bufA, bufB, fx, nseq, 1, nx, twx, threadIdx.x, blockDim.x);
   // (q, kx) walked incrementally: no division by the odd nxh per element
@@ -681,7 +645,7 @@ __device__ __forceinline__ void stage_ffty(const Geo& g, const FftDesc& fy, cons
   const int lg_tx = 31 - __clz(tx);  // tx is a power of two (ffty_tile)
   constexpr bool F32 = std::is_same<T, float>::value;
   const int twb = ny * tx + fft_pad_elems(ny * tx);  // buffer B is written padded
-  const bool fast = F32 && fft_smem_shape(ny, tx, true);
+  const bool fast = F32 && fft_smem_shape(ny, tx);
   if constexpr (F32) {
     if (fast) load_twiddles_smem(twy, ny, twb);
   }
@@ -710,7 +674,7 @@ __device__ __forceinline__ void stage_ffty(const Geo& g, const FftDesc& fy, cons
   }
   const C2<T>* res = nullptr;
   if constexpr (F32) {
-    if (fast) res = smem_f2() + fft_dispatch_smem<DIR, true>(0, ny * tx, twb, fy, tx, tx, 1, threadIdx.x, blockDim.x);
+    if (fast) res = smem_f2() + fft_dispatch_smem<DIR, true>(0, ny * tx, twb, threadIdx.x, blockDim.x);
   }
   if (!fast) res = fft_dispatch<T, DIR, true>(bufA, bufB, fy, tx, tx, 1, twy, threadIdx.x, blockDim.x);
   for (int t = threadIdx.x; t < ny * tx; t += blockDim.x) {
@@ -828,7 +792,7 @@ __device__ __forceinline__ void stage_ffty_persistent(const Geo& g, const FftDes
   const int qsz = F32 ? fft_pad_elems(tsz) : tsz;
   int L = 0, Q = tsz, F = tsz + qsz;
   const int twb = 2 * tsz + qsz;
-  const bool fast = F32 && fft_smem_shape(ny, tx, true);
+  const bool fast = F32 && fft_smem_shape(ny, tx);
   if constexpr (F32) {
     if (fast) load_twiddles_smem(twy, ny, twb);
   }
@@ -860,7 +824,7 @@ __device__ __forceinline__ void stage_ffty_persistent(const Geo& g, const FftDes
     }
     const C2<T>* res = nullptr;
     if constexpr (F32) {
-      if (fast) res = smem_f2() + fft_dispatch_smem<DIR, true>(L, Q, twb, fy, tx, tx, 1, threadIdx.x, blockDim.x);
+      if (fast) res = smem_f2() + fft_dispatch_smem<DIR, true>(L, Q, twb, threadIdx.x, blockDim.x);
     }
     if (!fast) res = fft_dispatch<T, DIR, true>(X0 + L, X0 + Q, fy, tx, tx, 1, twy, threadIdx.x, blockDim.x);
     const int bz = (int)(tile / ntx), bx = (int)(tile - (long long)bz * ntx);
@@ -901,28 +865,16 @@ __device__ __forceinline__ void stage_ffty_persistent(const Geo& g, const FftDes
 // inverse pivots precomputed at plan time.  Column (0, 0) is singular: its
 // right-hand side loses its dzf-weighted mean (compatibility) and its last
 // unknown is pinned (inverse pivot 0); the pressure gauge is fixed later.
-// Loads run PF levels ahead of the recurrence; FP32 spectra are widened and
-// narrowed on the integer pipe.
-template <typename T> __device__ __forceinline__ double2 to_d2(C2<T> v);
-template <> __device__ __forceinline__ double2 to_d2<double>(double2 v) { return v; }
-template <> __device__ __forceinline__ double2 to_d2<float>(float2 v) {
-  return make_double2(widen_f32(v.x), widen_f32(v.y));
-}
-template <typename T> __device__ __forceinline__ C2<T> from_d(double x, double y);
-template <> __device__ __forceinline__ double2 from_d<double>(double x, double y) { return make_double2(x, y); }
-template <> __device__ __forceinline__ float2 from_d<float>(double x, double y) {
-  return make_float2(narrow_f64(x), narrow_f64(y));
-}
-
-template <typename T, bool ZERO_MODE>
+// Loads run PF levels ahead of the recurrence.
+template <bool ZERO_MODE>
 __device__ __forceinline__ void thomas_column(const Geo& g, const double* __restrict__ invd,
-                                              C2<T>* spec, double2* ybuf, size_t col, size_t stride) {
+                                              double2* spec, double2* ybuf, size_t col, size_t stride) {
   constexpr int PF = 4;
   const int nz = g.nz;
   double mr = 0.0, mi = 0.0;
   if (ZERO_MODE) {
     for (int k = 0; k < nz; ++k) {
-      const double2 f = to_d2<T>(spec[(size_t)k * stride + col]);
+      const double2 f = spec[(size_t)k * stride + col];
       mr += g.dzf[k] * f.x;
       mi += g.dzf[k] * f.y;
     }
@@ -930,7 +882,7 @@ __device__ __forceinline__ void thomas_column(const Geo& g, const double* __rest
     mi /= g.lz;
   }
   // forward sweep: y_k = f_k - (a_k / d_{k-1}) y_{k-1}
-  C2<T> fq[PF];
+  double2 fq[PF];
   double dq[PF];
 #pragma unroll
   for (int u = 0; u < PF; ++u) {
@@ -944,7 +896,7 @@ __device__ __forceinline__ void thomas_column(const Geo& g, const double* __rest
     for (int u = 0; u < PF; ++u) {
       const int k = k0 + u;
       if (k < nz) {
-        const double2 f = to_d2<T>(fq[u]);
+        const double2 f = fq[u];
         const double d = dq[u];
         const int kn = k + PF < nz ? k + PF : nz - 1;
         fq[u] = spec[(size_t)kn * stride + col];
@@ -959,7 +911,7 @@ __device__ __forceinline__ void thomas_column(const Geo& g, const double* __rest
   }
   // back substitution: x_k = (y_k - c_k x_{k+1}) / d_k
   double xr = yr * dprev, xi = yi * dprev;
-  spec[(size_t)(nz - 1) * stride + col] = from_d<T>(xr, xi);
+  spec[(size_t)(nz - 1) * stride + col] = make_double2(xr, xi);
   double2 yq[PF];
 #pragma unroll
   for (int u = 0; u < PF; ++u) {
@@ -980,7 +932,7 @@ __device__ __forceinline__ void thomas_column(const Geo& g, const double* __rest
         const double c = g.zc[k];
         xr = (y.x - c * xr) * d;
         xi = (y.y - c * xi) * d;
-        spec[(size_t)k * stride + col] = from_d<T>(xr, xi);
+        spec[(size_t)k * stride + col] = make_double2(xr, xi);
       }
     }
   }
@@ -1161,7 +1113,7 @@ __device__ __forceinline__ void stage_fftx_inv_m(const Geo& g, const FftDesc& fx
   const bool pre_p = need_p && MODE == kInvPlain && sizeof(T) == sizeof(double);
   constexpr bool F32 = std::is_same<T, float>::value;
   const int twb = nseq * nx + fft_pad_elems(nseq * nx);  // buffer B is written padded
-  const bool fast = F32 && fft_smem_shape(nx, nseq, false);
+  const bool fast = F32 && fft_smem_shape(nx, nseq);
   if constexpr (F32) {
     if (fast) load_twiddles_smem(twx, nx, twb);
   }
@@ -1229,7 +1181,7 @@ __device__ __forceinline__ void stage_fftx_inv_m(const Geo& g, const FftDesc& fx
   __syncthreads();
   const C2<T>* res = nullptr;
   if constexpr (F32) {
-    if (fast) res = smem_f2() + fft_dispatch_smem<1, false>(0, nseq * nx, twb, fx, nseq, 1, nx, threadIdx.x, blockDim.x);
+    if (fast) res = smem_f2() + fft_dispatch_smem<1, false>(0, nseq * nx, twb, threadIdx.x, blockDim.x);
   }
   if (!fast) res = fft_dispatch<T, 1, false>(bufA, bufB, fx, nseq, 1, nx, twx, threadIdx.x, blockDim.x);
 #pragma unroll
