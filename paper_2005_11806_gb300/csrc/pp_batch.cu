@@ -327,7 +327,7 @@ cudaError_t launch_pass(pp_batch_s* B, cudaStream_t s) {
   kb_check<<<B->n, 1024, 0, s>>>(B->d_dev, B->d_ctl, kExactEveryBatch);
   if (B->n_y) kb_ffty<-1><<<B->n_y, kThreads, B->smem_y, s>>>(B->d_dev, B->w_y);
   if (B->n_yw && (e = launch_batch_ffty_w(B->d_dev, B->w_yw, B->n_yw, B->smem_yw, 0, s)) != cudaSuccess) return e;
-  kb_tridiag<<<B->n_z, kZThreads, zsweep_smem<ZForm32, 1>(), s>>>(B->d_dev, B->w_z);
+  kb_tridiag<<<B->n_z, kZThreads, zsweep_smem<ZForm32>(), s>>>(B->d_dev, B->w_z);
   if (B->n_y) kb_ffty<1><<<B->n_y, kThreads, B->smem_y, s>>>(B->d_dev, B->w_y);
   if (B->n_yw && (e = launch_batch_ffty_w(B->d_dev, B->w_yw, B->n_yw, B->smem_yw, 1, s)) != cudaSuccess) return e;
   if (B->n_x) kb_fftx_inv<<<B->n_x, kThreads, B->smem_x, s>>>(B->d_dev, B->w_x);

@@ -64,20 +64,21 @@ __global__ void __launch_bounds__(128) k_tridiag(Geo g, const double* __restrict
 
 // z solve of FP64 and PP_MIXED_Z64 plans: one thread per column of `spec`
 // (ZForm64: complex entries; ZFormD: scalars, the components apart, which
-// gives small grids twice the chains).  P = 2 (periodic y): a thread takes
-// the columns ky and ny - ky, which share their table column; the columns
-// that are their own mirror are done twice by the same thread.  The warp that
-// holds column 0 first takes its dzf-weighted mean and subtracts it on the
-// way (all its lanes run the ZERO variant, the others with mean 0), so no
-// warp runs two variants.
-template <class F, int P>
+// gives small grids twice the chains).  The warp that holds column 0 first
+// takes its dzf-weighted mean and subtracts it on the way (all its lanes run
+// the ZERO variant, the others with mean 0), so no warp runs two variants.
+//
+// Dropped: a thread taking both columns ky and ny - ky of a shared table
+// column.  It halves the table traffic and leaves half the warps; one column /
+// two, ms, event overhead included: mixed_z64 512^3 0.515 / 0.543, 384^3 0.235 /
+// 0.270, 512 x 512 x 128 0.135 / 0.145, 256^3 0.094 / 0.150.
+template <class F>
 __global__ void __launch_bounds__(kZThreads) k_zsolve(Geo g, F tab, int nyt, int ysym, typename F::Val* spec,
                                                       const DevStatus* __restrict__ st) {
   if (stopped(st)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int C = std::is_same<F, ZFormD>::value ? 2 : 1;  // entries per complex column
   const unsigned n = (unsigned)C * (unsigned)g.ny * (unsigned)g.nxh;  // entries of a row
-  const unsigned work = P == 2 ? (unsigned)C * (unsigned)nyt * (unsigned)g.nxh : n;
   const unsigned id = blockIdx.x * kZThreads + threadIdx.x;
   const unsigned col = id / C;
   const bool first = id < 32u;  // warp-uniform
@@ -87,19 +88,13 @@ __global__ void __launch_bounds__(kZThreads) k_zsolve(Geo g, F tab, int nyt, int
     if (C == 2 && id == 1u) mx = my;  // the scalars' second entry is the imaginary part
     if (col != 0u) mx = my = 0.0;
   }
-  if (id >= work) return;
+  if (id >= n) return;
   const unsigned ny = (unsigned)g.ny, nxh = (unsigned)g.nxh;
   const unsigned ky = col / nxh, kx = col - ky * nxh;
   const unsigned kyt = (ysym && 2u * ky > ny) ? ny - ky : ky;
   const size_t t = (size_t)kyt * nxh + kx, tstride = (size_t)nyt * nxh;
-  typename F::Val* vals[P];
-  vals[0] = spec + id;
-  if constexpr (P == 2) {
-    const unsigned ky2 = (ky == 0u || 2u * ky == ny) ? ky : ny - ky;
-    vals[1] = spec + (size_t)(ky2 * nxh + kx) * C + (id - col * C);
-  }
-  if (first) zsweep<F, P, true>(tab, vals, n, t, tstride, g.nz, nullptr, smem_raw, mx, my);
-  else zsweep<F, P, false>(tab, vals, n, t, tstride, g.nz, nullptr, smem_raw, 0.0, 0.0);
+  if (first) zsweep<F, true>(tab, spec + id, n, t, tstride, g.nz, nullptr, smem_raw, mx, my);
+  else zsweep<F, false>(tab, spec + id, n, t, tstride, g.nz, nullptr, smem_raw, 0.0, 0.0);
 }
 
 __global__ void __launch_bounds__(kZThreads, 8) k_tridiag_mixed(Geo g, const double* __restrict__ mtab,
@@ -232,35 +227,19 @@ cudaError_t launch_tridiag(const Geo& g, const double* invd, double2* spec, doub
 cudaError_t launch_tridiag_mixed(const Geo& g, const double* invd, const double* mtab, const TriF32& f32, float2* spec,
                                  const DevStatus* st, Queue s) {
   const size_t ncol = (size_t)g.ny * g.nxh;
-  return enqueue(s, k_tridiag_mixed, tri_mixed_blocks(ncol, f32.nlow), kZThreads, zsweep_smem<ZForm32, 1>(), g, mtab,
+  return enqueue(s, k_tridiag_mixed, tri_mixed_blocks(ncol, f32.nlow), kZThreads, zsweep_smem<ZForm32>(), g, mtab,
                  invd, f32, spec, st);
 }
 
-template <class F, int P>
-static cudaError_t launch_zsolve_p(const Geo& g, const F& form, int nyt, int ysym, size_t work, typename F::Val* spec,
-                                   const DevStatus* st, Queue s) {
-  static_assert(zsweep_smem<F, P>() <= 48 * 1024, "fits without the opt-in attribute");
-  return enqueue(s, k_zsolve<F, P>, (unsigned)((work + kZThreads - 1) / kZThreads), kZThreads, zsweep_smem<F, P>(), g,
-                 form, nyt, ysym, spec, st);
-}
-
-// Two columns a thread halve the table traffic and leave half the warps: it
-// pays from about 1.5 such warps an SM partition (measured, one column / two:
-// 512^3, 3.4 warps, 0.533 / 0.512 ms; 384^3, 1.9 warps, 0.235 / 0.214 ms;
-// 256^3, 0.85 warps, 0.088 / 0.115 ms).
 template <typename T>
 cudaError_t launch_zsolve(const Geo& g, const TriZ<T>& t, C2<T>* spec, const DevStatus* st, Queue s) {
-  const size_t ncol = (size_t)g.ny * g.nxh;
-  if constexpr (std::is_same<T, float>::value) {
-    const ZForm64 form{t.m, t.d, t.e};
-    const size_t pairs = (size_t)t.nyt * g.nxh;
-    if (t.ysym && pairs >= (size_t)152 * 4 * 32 * 3 / 2)
-      return launch_zsolve_p<ZForm64, 2>(g, form, t.nyt, t.ysym, pairs, spec, st, s);
-    return launch_zsolve_p<ZForm64, 1>(g, form, t.nyt, t.ysym, ncol, spec, st, s);
-  } else {
-    const ZFormD form{t.m, t.d, t.e};
-    return launch_zsolve_p<ZFormD, 1>(g, form, t.nyt, t.ysym, 2 * ncol, reinterpret_cast<double*>(spec), st, s);
-  }
+  using F = std::conditional_t<std::is_same<T, float>::value, ZForm64, ZFormD>;
+  using Val = typename F::Val;
+  constexpr size_t smem = zsweep_smem<F>();
+  static_assert(smem <= 48 * 1024, "fits without the opt-in attribute");
+  const size_t n = (size_t)g.ny * g.nxh * (sizeof(C2<T>) / sizeof(Val));
+  return enqueue(s, k_zsolve<F>, (unsigned)((n + kZThreads - 1) / kZThreads), kZThreads, smem, g, F{t.m, t.d, t.e},
+                 t.nyt, t.ysym, reinterpret_cast<Val*>(spec), st);
 }
 template cudaError_t launch_zsolve<float>(const Geo&, const TriZ<float>&, float2*, const DevStatus*, Queue);
 template cudaError_t launch_zsolve<double>(const Geo&, const TriZ<double>&, double2*, const DevStatus*, Queue);

@@ -1052,8 +1052,7 @@ __device__ __forceinline__ void stage_tridiag_col32(const Geo& g, const TriF32& 
   const int kx = (int)(col - (size_t)j * g.nxh);
   if (col == 0 || fabs(f.lamx[kx] + f.lamy[j]) < f.thr) return;
   const ZForm32 form{f.mtab, nullptr, f.invd};
-  float2* const vals[1] = {spec + col};
-  zsweep<ZForm32, 1, false>(form, vals, ncol, col, ncol, g.nz, f.zc, smem, 0.0, 0.0);
+  zsweep<ZForm32, false>(form, spec + col, ncol, col, ncol, g.nz, f.zc, smem, 0.0, 0.0);
 }
 
 // Block b of the mixed z solve: the first nblk_low blocks give one warp to

@@ -16,7 +16,7 @@
 // conversions and address arithmetic); the rest hides behind other warps.
 //
 // Measured (register prefetch -> this): PP_MIXED_Z64 256^3 0.250 -> 0.088 ms,
-// 512^3 0.597 -> 0.51 ms; FP64 128^3 0.105 -> 0.029 ms; the FP32 columns of
+// 512^3 0.597 -> 0.466 ms; FP64 128^3 0.105 -> 0.029 ms; the FP32 columns of
 // 192 x 160 x 144 0.075 -> 0.031 ms.  64 threads a block, 4 rows a group and
 // the group counts below were the fastest of {32, 64, 128} x {2, 4, 8} x
 // {2, 3, 4, 6} over 32^3 .. 512^3.
@@ -151,36 +151,32 @@ struct ZForm32 {
   static __device__ __forceinline__ Val bwd_value(State s) { return s; }
 };
 
-// Shared memory of one block of kZThreads threads holding P columns each.
-template <class F, int P>
+// Shared memory of one block of kZThreads threads, a column each.
+template <class F>
 constexpr size_t zsweep_smem() {
   return (size_t)kZRows * F::kGroups * kZThreads *
-         (P * sizeof(typename F::Val) + (F::kHasB ? sizeof(typename F::B) : 0) +
+         (sizeof(typename F::Val) + (F::kHasB ? sizeof(typename F::B) : 0) +
           (sizeof(typename F::A) > sizeof(typename F::E) ? sizeof(typename F::A) : sizeof(typename F::E)));
 }
 
-// One sweep over n rows of a thread's P columns, which share their table
-// column.  Row i lies at v[q] + i vstep (spectrum), ta + i tstep (first
-// table) and tb + i tstep (second table, HASB); step(state, value, a, i) is
-// the recurrence, value(state, b) what is stored in place of the row.
+// One sweep over n rows of a thread's column.  Row i lies at v + i vstep
+// (spectrum), ta + i tstep (first table) and tb + i tstep (second table, HASB);
+// step(state, value, a, i) is the recurrence, value(state, b) what is stored in
+// place of the row.
 //
 // A warp issues in order, so a row's conversions and store must not stand
 // between its FMA and the next row's: the value of row i is formed while the
 // FMA of row i + 1 is in flight.  The next group's entries are read into
 // registers before the current group's chain for the same reason.
-template <int P, bool HASB, int NG, class State, class Val, class A, class B, class Step, class Value>
-__device__ __forceinline__ void zsweep_rows(State (&s)[P], int n, Val* const (&v)[P], ptrdiff_t vstep, const A* ta,
-                                            const B* tb, ptrdiff_t tstep, Val* rv, A* ra, B* rb, Step&& step,
-                                            Value&& value) {
+template <bool HASB, int NG, class State, class Val, class A, class B, class Step, class Value>
+__device__ __forceinline__ void zsweep_rows(State& s, int n, Val* v, ptrdiff_t vstep, const A* ta, const B* tb,
+                                            ptrdiff_t tstep, Val* rv, A* ra, B* rb, Step&& step, Value&& value) {
   constexpr int R = kZRows, SLOTS = R * NG;
-  const Val* cv[P];
-  Val* out[P];
-#pragma unroll
-  for (int q = 0; q < P; ++q) cv[q] = out[q] = v[q];
+  const Val* cv = v;
+  Val* out = v;
   int left = n, slot = 0;  // rows not yet copied, slot of the next
   auto copy_row = [&](int at, ptrdiff_t vo, ptrdiff_t to) {
-#pragma unroll
-    for (int q = 0; q < P; ++q) zs_cp<sizeof(Val)>(rv + (q * SLOTS + at) * kZThreads, cv[q] + vo);
+    zs_cp<sizeof(Val)>(rv + at * kZThreads, cv + vo);
     zs_cp<sizeof(A)>(ra + at * kZThreads, ta + to);
     if constexpr (HASB) zs_cp<sizeof(B)>(rb + at * kZThreads, tb + to);
   };
@@ -188,8 +184,7 @@ __device__ __forceinline__ void zsweep_rows(State (&s)[P], int n, Val* const (&v
     if (left >= R) {
 #pragma unroll
       for (int u = 0; u < R; ++u) copy_row(slot + u, u * vstep, u * tstep);
-#pragma unroll
-      for (int q = 0; q < P; ++q) cv[q] += R * vstep;
+      cv += R * vstep;
       ta += R * tstep;
       if constexpr (HASB) tb += R * tstep;
     } else {
@@ -201,15 +196,14 @@ __device__ __forceinline__ void zsweep_rows(State (&s)[P], int n, Val* const (&v
   };
 #pragma unroll
   for (int q = 0; q < NG; ++q) issue();
-  Val f[P][R];
+  Val f[R];
   A a[R];
   B b[R];
   int rd = 0;
-  auto read = [&](Val (&ff)[P][R], A (&aa)[R], B (&bb)[R]) {  // slots past the last row hold old data, unused
+  auto read = [&](Val (&ff)[R], A (&aa)[R], B (&bb)[R]) {  // slots past the last row hold old data, unused
 #pragma unroll
     for (int u = 0; u < R; ++u) {
-#pragma unroll
-      for (int q = 0; q < P; ++q) ff[q][u] = rv[(q * SLOTS + rd + u) * kZThreads];
+      ff[u] = rv[(rd + u) * kZThreads];
       aa[u] = ra[(rd + u) * kZThreads];
       if constexpr (HASB) bb[u] = rb[(rd + u) * kZThreads];
       else bb[u] = B();
@@ -221,7 +215,7 @@ __device__ __forceinline__ void zsweep_rows(State (&s)[P], int n, Val* const (&v
   B bprev = B();
   int i = 0;
   for (; i + R <= n; i += R) {
-    Val f2[P][R];
+    Val f2[R];
     A a2[R];
     B b2[R];
     zs_wait<NG - 2>();
@@ -229,23 +223,16 @@ __device__ __forceinline__ void zsweep_rows(State (&s)[P], int n, Val* const (&v
     issue();
 #pragma unroll
     for (int u = 0; u < R; ++u) {
-      State t[P];
-#pragma unroll
-      for (int q = 0; q < P; ++q) t[q] = step(s[q], f[q][u], a[u], i + u);
-#pragma unroll
-      for (int q = 0; q < P; ++q) {
-        const Val w = value(s[q], bprev);  // row i + u - 1
-        if (u > 0 || i > 0) out[q][(u - 1) * vstep] = w;
-        s[q] = t[q];
-      }
+      const State t = step(s, f[u], a[u], i + u);
+      const Val w = value(s, bprev);  // row i + u - 1
+      if (u > 0 || i > 0) out[(u - 1) * vstep] = w;
+      s = t;
       bprev = b[u];
     }
-#pragma unroll
-    for (int q = 0; q < P; ++q) out[q] += R * vstep;
+    out += R * vstep;
 #pragma unroll
     for (int u = 0; u < R; ++u) {
-#pragma unroll
-      for (int q = 0; q < P; ++q) f[q][u] = f2[q][u];
+      f[u] = f2[u];
       a[u] = a2[u];
       b[u] = b2[u];
     }
@@ -253,31 +240,24 @@ __device__ __forceinline__ void zsweep_rows(State (&s)[P], int n, Val* const (&v
 #pragma unroll
   for (int u = 0; u < R; ++u) {
     if (i + u < n) {
-#pragma unroll
-      for (int q = 0; q < P; ++q) {
-        const State t = step(s[q], f[q][u], a[u], i + u);
-        if (i + u > 0) out[q][(u - 1) * vstep] = value(s[q], bprev);
-        s[q] = t;
-      }
+      const State t = step(s, f[u], a[u], i + u);
+      if (i + u > 0) out[(u - 1) * vstep] = value(s, bprev);
+      s = t;
       bprev = b[u];
     }
   }
-#pragma unroll
-  for (int q = 0; q < P; ++q)
-    if (n > 0) v[q][(n - 1) * vstep] = value(s[q], bprev);
+  if (n > 0) v[(n - 1) * vstep] = value(s, bprev);
   zs_wait<0>();
 }
 
-// Both sweeps of a thread's P columns.  vals: the columns' first entries,
-// vstride entries from row to row; t: their table offset, tstride entries
-// from row to row; zc: the super-diagonal of L_z (ZForm32 only).  ZERO:
-// m0x, m0y are subtracted from the right-hand side (the singular column's
-// mean).  Two of the columns may be the same one: both then compute and
-// store the same values.
-template <class F, int P, bool ZERO>
-__device__ __forceinline__ void zsweep(const F& tab, typename F::Val* const (&vals)[P], size_t vstride, size_t t,
-                                       size_t tstride, int nz, const float* __restrict__ zc, unsigned char* smem,
-                                       double m0x, double m0y) {
+// Both sweeps of a thread's column.  val: its first entry, vstride entries
+// from row to row; t: its table offset, tstride entries from row to row; zc:
+// the super-diagonal of L_z (ZForm32 only).  ZERO: m0x, m0y are subtracted from
+// the right-hand side (the singular column's mean).
+template <class F, bool ZERO>
+__device__ __forceinline__ void zsweep(const F& tab, typename F::Val* val, size_t vstride, size_t t, size_t tstride,
+                                       int nz, const float* __restrict__ zc, unsigned char* smem, double m0x,
+                                       double m0y) {
   using Val = typename F::Val;
   using A = typename F::A;
   using B = typename F::B;
@@ -286,32 +266,25 @@ __device__ __forceinline__ void zsweep(const F& tab, typename F::Val* const (&va
   constexpr int SLOTS = kZRows * F::kGroups;
   constexpr size_t kAE = sizeof(A) > sizeof(E) ? sizeof(A) : sizeof(E);
   Val* rv = reinterpret_cast<Val*>(smem) + threadIdx.x;
-  unsigned char* after_v = smem + P * sizeof(Val) * SLOTS * kZThreads;
+  unsigned char* after_v = smem + sizeof(Val) * SLOTS * kZThreads;
   A* ra = reinterpret_cast<A*>(after_v) + threadIdx.x;
   E* re = reinterpret_cast<E*>(after_v) + threadIdx.x;
   B* rb = reinterpret_cast<B*>(after_v + kAE * SLOTS * kZThreads) + threadIdx.x;
-  State s[P];
-#pragma unroll
-  for (int q = 0; q < P; ++q) s[q] = F::zero();
-  zsweep_rows<P, F::kHasB, F::kGroups>(
-      s, nz, vals, (ptrdiff_t)vstride, (const A*)tab.m + t, (const B*)tab.d + (F::kHasB ? t : 0),
-      (ptrdiff_t)tstride, rv, ra, rb,
+  State s = F::zero();
+  zsweep_rows<F::kHasB, F::kGroups>(
+      s, nz, val, (ptrdiff_t)vstride, (const A*)tab.m + t, (const B*)tab.d + (F::kHasB ? t : 0), (ptrdiff_t)tstride,
+      rv, ra, rb,
       [&](const State& p, const Val& f, const A& m, int) { return F::template fwd<ZERO>(p, f, m, m0x, m0y); },
       [](const State& p, const B& d) { return F::fwd_value(p, d); });
   // row nz - 1: x from the value just stored (this thread's own store)
   const E* te = (const E*)tab.e + t;
   constexpr bool F32 = std::is_same<F, ZForm32>::value;
-  Val* next[P];
-#pragma unroll
-  for (int q = 0; q < P; ++q) {
-    Val* top = vals[q] + (size_t)(nz - 1) * vstride;
-    s[q] = F::turn(*top, F32 ? te[(size_t)(nz - 1) * tstride] : E());
-    if constexpr (F32) *top = s[q];
-    next[q] = top - vstride;
-  }
+  Val* top = val + (size_t)(nz - 1) * vstride;
+  s = F::turn(*top, F32 ? te[(size_t)(nz - 1) * tstride] : E());
+  if constexpr (F32) *top = s;
   __threadfence_block();  // the forward values are read back by this thread's copies
-  zsweep_rows<P, false, F::kGroups>(
-      s, nz - 1, next, -(ptrdiff_t)vstride, te + (ptrdiff_t)(nz - 2) * (ptrdiff_t)tstride, (const B*)nullptr,
+  zsweep_rows<false, F::kGroups>(
+      s, nz - 1, top - vstride, -(ptrdiff_t)vstride, te + (ptrdiff_t)(nz - 2) * (ptrdiff_t)tstride, (const B*)nullptr,
       -(ptrdiff_t)tstride, rv, re, rb,
       [&](const State& p, const Val& v, const E& e, int i) { return F::bwd(p, v, e, F32 ? zc[nz - 2 - i] : 0.f); },
       [](const State& p, const B&) { return F::bwd_value(p); });
