@@ -194,18 +194,29 @@ def algorithmic(kernel, w, precision):
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per cell of a
 # launch of the pass kernels of mixed plans, from ncu captures on the
 # 512 x 512 x 128 case: the same kernels, block shapes and per-plane grids as
-# at 512^3, so the bytes scale with the cells processed (the captures and
-# their commands are summarised under profiles/).  The residual kernel's
-# figure is weighted over the 40-pass exact/update cycle: 18.75 B on an
-# update pass, 64.15 B on an exact pass (both from one capture of the kernel
-# as it stands, the paired-row update: profiles/launches_bubbles512_mixed_z64.md).
-# The z solve's is for the PP_MIXED_Z64 kernel
-# (profiles/pass_kernels_mixed_z64_bubbles512x512x128.md).
-RESID_DRAM_B_PER_CELL = {"update": 18.75, "exact": 64.15}
-DRAM_B_PER_CELL = {
-    "resid_fftx": 0.975 * RESID_DRAM_B_PER_CELL["update"] + 0.025 * RESID_DRAM_B_PER_CELL["exact"],
-    "tridiag_z": 17.23,
-}
+# at 512^3, so the bytes scale with the cells processed.  The residual
+# kernel's figures are weighted over the 40-pass exact/update cycle.  Rows of
+# 512 take k_resid_w<float, false, 512> (18.74 B on an update pass, 75.01 B on
+# an exact pass) and the z solve is k_zsolve<ZForm64>
+# (profiles/resid_zsolve_dram_bubbles512x512x128_z64.md); "resid_fftx" of the
+# table is the block kernel k_resid_fftx, which rows without a register
+# transform take (captured when 512 took it too:
+# profiles/launches_bubbles512_mixed_z64.md).
+def _cycle(update, exact):
+    return 0.975 * update + 0.025 * exact
+
+
+DRAM_B_PER_CELL = {"resid_fftx": _cycle(18.75, 64.15), "tridiag_z": 19.65}
+RESID_W512_DRAM_B_PER_CELL = _cycle(18.74, 75.01)
+
+
+def dram_bytes(kernel, nx, npts):
+    """Measured DRAM bytes of one launch, None where not captured (the residual's register forms up to 256)."""
+    if kernel == "resid_fftx" and nx == 512:
+        return int(RESID_W512_DRAM_B_PER_CELL * npts)
+    if kernel == "resid_fftx" and nx <= 256:
+        return None
+    return int(DRAM_B_PER_CELL[kernel] * npts) if kernel in DRAM_B_PER_CELL else None
 
 
 def run_ours(args, rank, world, local_rank):
@@ -295,8 +306,8 @@ def run_ours(args, rank, world, local_rank):
                 "frac": round(achieved / hbm_peak, 4), "traffic": None, "kernel": name,
                 "avg_launch_ms": round(avg_s * 1e3, 4), "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)"}
     if (args.precision == "mixed_z64" or (args.precision == "mixed" and name == "resid_fftx")) \
-            and DRAM_B_PER_CELL.get(name) is not None:
-        roof["traffic"] = int(DRAM_B_PER_CELL[name] * npts)
+            and dram_bytes(name, w.nx, npts) is not None:
+        roof["traffic"] = dram_bytes(name, w.nx, npts)
         roof["traffic_source"] = "ncu DRAM bytes per cell at 512x512x128, scaled to the launch's cells"
     kernels = {k: {"launches": n, "total_ms": round(t, 3), "avg_ms": round(t / n, 4),
                    "share": round(t / sum(x[1] for x in kern.values()), 4)} for k, (n, t) in kern.items()}

@@ -238,9 +238,7 @@ pp_status pressure_divergence_source(pp_plan plan, const double* phi, const doub
  * gravity[3], dt_new > 0, dt_old (> 0 with ru_prev), ru_prev[3] (RU^{n-1}
  * on the faces, or NULL).  Out: u_star[3] (u*, v*, w*; w wall planes zero),
  * ru_out[3] (RU^n for the next step, or NULL).  Device pointers only
- * (PP_ERR_INVALID_ARG otherwise); enqueued on the plan's stream.  Uses the
- * plan's workspace, so it must not overlap a pressure_correct on the same
- * plan. */
+ * (PP_ERR_INVALID_ARG otherwise); enqueued on the plan's stream. */
 pp_status pressure_predictor(pp_plan plan, const double* u, const double* v, const double* w,
                              const double* rho, const double* mu, const double* const force[3],
                              const double gravity[3], double dt_new, double dt_old,

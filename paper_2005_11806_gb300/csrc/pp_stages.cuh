@@ -97,9 +97,10 @@ __device__ __forceinline__ void load_twiddles_smem(const float2* __restrict__ tw
 // by the face's two cells where both are in the thread (5 x faces for 4
 // cells; with two rows taken together 3 y faces for 2 cells), then
 //   A delta = 2 [w_x (G_x+ - G_x-) + w_y+ G_y+ - w_y- G_y- + w_z+ G_z+ - w_z- G_z-]
-// with the layer (and row) factors w.  Coefficients formed per cell and face
-// took 131 instructions a cell, 35 of them range checks and selects of the
-// division; this form takes 89 with the transform.
+// with the layer (and row) factors w.  Coefficients formed per cell and face,
+// with the range checks of a division each, take 111 instructions a cell with
+// the transform and 0.098 ms at 256^3, 0.678 ms at 512^3; this form takes 87,
+// 0.091 ms and 0.644 ms.
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ float half_flux(float da, float db, float ha, float hb) {
   return (db - da) * rcp_f32(ha + hb);

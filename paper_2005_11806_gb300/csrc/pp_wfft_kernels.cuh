@@ -117,8 +117,8 @@ __device__ __forceinline__ void wfft512_line(float2* line, const float2* tw, int
 // block kernel (stage_resid_fftx) meets a block barrier after each of its
 // steps, and its smallest unit (2048 values) leaves most SMs without work on
 // small grids.  FP32: bound by the latency of its global loads (half of the
-// stalls, issue 45 % busy, DRAM 39 % at 256^3); FP64: by the FP64 pipe.  Block
-// kernel and loop-control kernel -> this, ms: mixed 256^3 0.114 -> 0.094, mixed
+// stalls, issue 49 % busy, DRAM 43 % at 256^3); FP64: by the FP64 pipe.  Block
+// kernel and loop-control kernel -> this, ms: mixed 256^3 0.114 -> 0.091, mixed
 // 512^3 0.805 -> 0.644, mixed 192 x 160 x 144 0.046 -> 0.029, FP64 128^3 0.142
 // -> 0.106, FP64 32^3 0.023 -> 0.016.  Measured and dropped: prefetching a later
 // block's rows into L2 (256^3: 0.106); four and three blocks an SM (192 x 160 x
