@@ -324,19 +324,37 @@ constexpr int kPredLanes = 30;  // useful lanes of a warp; lanes 0 and 31 hold t
 // with every term formed at both of its cells and three IEEE divisions.
 // 256^3: 9.7 ms -> 6.2 ms (FP64 pipe 86 % busy; 12 % of the lanes are the tiles'
 // neighbours at 256).
-__global__ void __launch_bounds__(128) k_predictor(Geo g, PredArgs A, int ntile, int nchunk, int chunk) {
+//
+// WHOLE (nx <= 32): a warp holds 32 / nx whole rows, neighbours by shuffles
+// around each row, so no lane is a tile's neighbour and a short row does not
+// leave most of the warp idle (8 x 64 x 500: 0.371 -> 0.117 ms, 32 x 96 x 96
+// 0.228 -> 0.117, both with chunks as before).
+template <bool WHOLE>
+__global__ void __launch_bounds__(128) k_predictor(Geo g, PredArgs A, int ntile, int ngroup, int nchunk, int chunk) {
   const int nx = g.nx, ny = g.ny, nz = g.nz;
   const int lane = threadIdx.x & 31;
   const unsigned wid = blockIdx.x * 4 + (threadIdx.x >> 5);
-  const unsigned rest = wid / (unsigned)ntile;
-  const int tile = (int)(wid - rest * ntile);
-  const int ch = (int)(rest / (unsigned)ny), j = (int)(rest - (unsigned)ch * ny);
+  const unsigned rest = WHOLE ? wid : wid / (unsigned)ntile;
+  const int ch = (int)(rest / (unsigned)ngroup);
   if (ch >= nchunk) return;
+  int i, j = (int)(rest - (unsigned)ch * ngroup);
+  bool emit_lane;
+  int from_left = 0, from_right = 0;  // WHOLE: the lanes of i - 1 and i + 1
+  if constexpr (WHOLE) {
+    const int rows = 32 / nx, q = lane / nx;
+    i = lane - q * nx;
+    j = j * rows + q;
+    emit_lane = q < rows && j < ny;
+    if (j >= ny) j = ny - 1;  // lanes without a row of their own only read
+    from_left = i == 0 ? lane + nx - 1 : lane - 1;
+    from_right = i + 1 == nx ? lane + 1 - nx : lane + 1;
+  } else {
+    const int at = (int)(wid - rest * ntile) * kPredLanes + lane - 1;  // -1 .. ; wraps
+    i = at < 0 ? at + nx : at;
+    while (i >= nx) i -= nx;
+    emit_lane = lane >= 1 && lane <= kPredLanes && at < nx;
+  }
   const int k0 = ch * chunk, k1 = min(k0 + chunk, nz);
-  const int at = tile * kPredLanes + lane - 1;  // -1 .. ; wraps
-  int i = at < 0 ? at + nx : at;
-  while (i >= nx) i -= nx;
-  const bool emit_lane = lane >= 1 && lane <= kPredLanes && at < nx;
   const bool ywall = g.ywall != 0;
   const bool wlo = ywall && j == 0, whi = ywall && j + 1 == ny;  // the row's low / high y edges are walls
   const int jm = j == 0 ? ny - 1 : j - 1, jp = j + 1 == ny ? 0 : j + 1;
@@ -345,8 +363,12 @@ __global__ void __launch_bounds__(128) k_predictor(Geo g, PredArgs A, int ntile,
   const size_t oc = (size_t)j * nx + i, om = (size_t)jm * nx + i, op = (size_t)jp * nx + i;
   const double idx = A.idx, idy = A.idy;
   constexpr unsigned full = 0xffffffffu;
-  auto left = [&](double a) { return __shfl_up_sync(full, a, 1); };     // value at i - 1
-  auto right = [&](double a) { return __shfl_down_sync(full, a, 1); };  // value at i + 1
+  auto left = [&](double a) {  // value at i - 1
+    return WHOLE ? __shfl_sync(full, a, from_left) : __shfl_up_sync(full, a, 1);
+  };
+  auto right = [&](double a) {  // value at i + 1
+    return WHOLE ? __shfl_sync(full, a, from_right) : __shfl_down_sync(full, a, 1);
+  };
 
   const int ks = k0 > 0 ? k0 - 1 : 0;  // the layer below the chunk only leaves its upper edges and centre
   size_t o = (size_t)ks * plane;
@@ -659,17 +681,35 @@ cudaError_t launch_predictor(const Geo& g, const double* u, const double* v, con
                              const double* mu, const double* const f[3], const double* const prev[3],
                              const double grav[3], double dt, double a, double b, double* const out[3],
                              double* const ru[3], cudaStream_t s) {
-  // a warp per 30 cells of a row and chunk of layers: long chunks (a chunk
-  // repeats one layer), but at least about 16 warps an SM
-  const int ntile = (g.nx + kPredLanes - 1) / kPredLanes;
-  const long long rows = (long long)ntile * g.ny;
+  // A warp per 30 cells of a row (or per 32 / nx rows) and chunk of layers: long
+  // chunks (a chunk repeats about 0.7 of a layer), but at least about 16 warps
+  // an SM.  Where chunks of eight leave fewer, the warps are counted: a warp
+  // takes about 6 us a layer, the FP64 unit's time, so an SM partition with a
+  // second warp takes twice as long (40^3, four layers a chunk: 0.059 ms, 800
+  // warps on 608 partitions; six layers, 560 warps: 0.047).
+  const bool whole = g.nx <= 32;
+  const int ntile = whole ? 1 : (g.nx + kPredLanes - 1) / kPredLanes;
+  const int ngroup = whole ? (g.ny + 32 / g.nx - 1) / (32 / g.nx) : g.ny;
+  const long long rows = (long long)ntile * ngroup;
+  auto warps = [&](int c) { return rows * ((g.nz + c - 1) / c); };
   int chunk = 64;
-  while (chunk > 4 && rows * ((g.nz + chunk - 1) / chunk) < 152 * 16) chunk >>= 1;
+  while (chunk > 8 && warps(chunk) < 152 * 16) chunk >>= 1;
+  if (warps(chunk) < 152 * 16) {
+    long long best = -1;
+    for (int c = 1; c <= 32; ++c) {
+      const long long cost = (warps(c) + 152 * 4 - 1) / (152 * 4) * (10 * c + 7);
+      if (best < 0 || cost < best) {
+        best = cost;
+        chunk = c;
+      }
+    }
+  }
   const int nchunk = (g.nz + chunk - 1) / chunk;
   const PredArgs A{u, v, w, rho, mu, f[0], f[1], f[2], prev[0], prev[1], prev[2], grav[0], grav[1], grav[2],
                    dt * a, dt * b, g.inv_dx, g.inv_dy, 0.5 * g.inv_dx, 0.5 * g.inv_dy, 8.0 * g.inv_dx,
                    8.0 * g.inv_dy, out[0], out[1], out[2], ru[0], ru[1], ru[2]};
-  k_predictor<<<(unsigned)((rows * nchunk + 3) / 4), 128, 0, s>>>(g, A, ntile, nchunk, chunk);
+  auto kern = whole ? k_predictor<true> : k_predictor<false>;
+  kern<<<(unsigned)((rows * nchunk + 3) / 4), 128, 0, s>>>(g, A, ntile, ngroup, nchunk, chunk);
   return cudaGetLastError();
 }
 
