@@ -140,7 +140,10 @@ cudaError_t launch_resid_fftx(const Geo& g, const Faces& fc, const FftDesc& fx, 
                               const double* b, double inv_dt, const double* rho, const double* p,
                               int p_zero, int scale_rho, C2<T>* spec, double* red, const LoopCheck* ck,
                               const DevStatus* st, Queue s, float* E, const float* delta) {
-  if (wfft_length(g.nx) || (g.nx == 512 && std::is_same<T, float>::value))
+  // FP32 rows of 512: the warp form for residuals; a plain solve's FP64 rows load
+  // faster with the block kernel's 32 warps an SM (warp form / block kernel:
+  // 512^3 0.953 / 0.855 ms, 512 x 512 x 128 0.247 / 0.222; 512 x 64 x 64 0.012 both)
+  if (wfft_length(g.nx) || (g.nx == 512 && std::is_same<T, float>::value && red != nullptr))
     return launch_resid_w<T>(g, fc, twx, b, rho, p, p_zero, scale_rho, spec, red, ck, st, s, E, delta);
   const int rpb = rows_per_block(g.nx, kEpt);
   const long nrows = (long)g.nz * g.ny;
